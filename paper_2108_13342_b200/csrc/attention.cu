@@ -28,6 +28,7 @@
 #include "lower.h"
 #include "tc_common.cuh"
 #include "tma_host.h"
+#include "warp_issue.cuh"
 
 namespace dnnf {
 
@@ -86,7 +87,7 @@ attention_kernel(const __grid_constant__ GemmParams pA, const __grid_constant__ 
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_qk + 5);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int D = q.D, Sk = q.Sk, sk16 = q.sk16;
   const int d_tiles = D >> 6, s_tiles = (sk16 + 63) >> 6;
   pdl_launch_dependents();
@@ -129,7 +130,7 @@ attention_kernel(const __grid_constant__ GemmParams pA, const __grid_constant__ 
   if (stage_mask && !q.mask_static && warp >= 2) load_mask_tile();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------- loads: the whole head at once ----------------
       mbar_expect_tx(bar_qk, (uint32_t)(d_tiles * (BM + sk16) * 128));
       for (int kt = 0; kt < d_tiles; ++kt) {
@@ -142,13 +143,13 @@ attention_kernel(const __grid_constant__ GemmParams pA, const __grid_constant__ 
           tma_load_4d(sV + (kt * d_tiles + j) * 8192, &q.tmV, bar_v, j * 64, kt * 64, q.v_batch[0] ? b0 : 0, q.v_batch[1] ? b1 : 0);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
-      const uint32_t idesc_s = idesc0 | ((uint32_t)(sk16 >> 3) << 17);                       // B = K, K-major
-      const uint32_t idesc_o = idesc0 | (1u << 16) | ((uint32_t)(D >> 3) << 17);             // B = V, MN-major
-      bool ok = mbar_wait(bar_qk, 0, abort_flag);
-      if (ok) {
+    // ---------------- MMA issuer ----------------
+    const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BM >> 4) << 24);
+    const uint32_t idesc_s = idesc0 | ((uint32_t)(sk16 >> 3) << 17);                       // B = K, K-major
+    const uint32_t idesc_o = idesc0 | (1u << 16) | ((uint32_t)(D >> 3) << 17);             // B = V, MN-major
+    bool ok = __all_sync(0xffffffffu, mbar_wait(bar_qk, 0, abort_flag));
+    if (ok) {
+      if (elect_one()) {
         for (int kt = 0; kt < d_tiles; ++kt) {
           const uint64_t da = make_desc(smem_u32(sQ) + kt * (BM * 128), 16, 1024);
           const uint64_t db = make_desc(smem_u32(sK) + kt * (sk16 * 128), 16, 1024);
@@ -156,11 +157,14 @@ attention_kernel(const __grid_constant__ GemmParams pA, const __grid_constant__ 
           for (int kk = 0; kk < 4; ++kk) tc_mma_bf16(tmem_base, da + 2 * kk, db + 2 * kk, idesc_s, (kt | kk) ? 1u : 0u);
         }
         tc_commit(bar_s);
-        ok = mbar_wait(bar_p, 0, abort_flag) && mbar_wait(bar_v, 0, abort_flag);
       }
-      if (ok) {
-        tc_fence_after();
-        const uint32_t d_o = tmem_base + (uint32_t)q.o_col;
+      __syncwarp();
+      ok = __all_sync(0xffffffffu, mbar_wait(bar_p, 0, abort_flag) && mbar_wait(bar_v, 0, abort_flag));
+    }
+    if (ok) {
+      tc_fence_after();
+      const uint32_t d_o = tmem_base + (uint32_t)q.o_col;
+      if (elect_one()) {
         for (int kt = 0; kt < s_tiles; ++kt) {
           const uint64_t da = make_desc(smem_u32(sP) + kt * (BM * 128), 16, 1024);
           const uint64_t db = make_desc(smem_u32(sV) + kt * d_tiles * 8192, 8192, 1024);

@@ -4,8 +4,8 @@
 // accumulator and stores through the block's output index map.
 //
 // One persistent CTA per SM, 320 threads, warp-specialised:
-//   warp 0      TMA producer (one elected lane)
-//   warp 1      TMEM allocation, then MMA issue (one elected lane)
+//   warp 0      TMA producer
+//   warp 1      TMEM allocation, then MMA issue
 //   warps 2..9  epilogue; warp w reads TMEM lanes 32*(w%4) .. 32*(w%4)+31, warps 2..5 the first
 //               half of the tile's columns, warps 6..9 the second half
 // A BK=64 shared-memory ring feeds the MMA; two accumulator stages in TMEM let the
@@ -23,6 +23,7 @@
 #include "ir.h"
 #include "tc_common.cuh"
 #include "tma_host.h"
+#include "warp_issue.cuh"
 
 namespace dnnf {
 
@@ -56,7 +57,7 @@ gemm_tc_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Gem
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint32_t* stage_area = tmem_slot + 8;          // TC_EPI_WARPS x kStageWords
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   pdl_launch_dependents();
   if (threadIdx.x == 0) TRACE(0);
   if (threadIdx.x == 0) {
@@ -82,21 +83,21 @@ gemm_tc_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Gem
   const int k_tiles = q.k_tiles;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer ----------------
-      // (stage index and phase advance by increments: a division by the run-time stage count costs this
-      // single thread some 200 cycles of dependent instructions per k-tile)
-      int s = 0; uint32_t ph = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        const int batch = (int)fd_div((uint32_t)tile, q.fd_tiles_mn), r = tile - batch * tiles_mn;
-        const int tm = (int)fd_div((uint32_t)r, q.fd_tiles_n), tn = r - tm * p.tiles_n;
-        const int b1 = (int)fd_div((uint32_t)batch, q.fd_batch0), b0 = batch - b1 * p.batch_ext[0];
-        // a batch dim an operand is broadcast over has stride 0 and extent 1 in its tensor map
-        const int ab0 = p.A.batch_stride[0] ? b0 : 0, ab1 = p.A.batch_stride[1] ? b1 : 0;
-        const int bb0 = p.B.batch_stride[0] ? b0 : 0, bb1 = p.B.batch_stride[1] ? b1 : 0;
-        for (int kt = 0; kt < k_tiles; ++kt) {
-          if (!mbar_wait(&empty_bar[s], ph ^ 1, abort_flag)) { ok = false; break; }
+    // ---------------- TMA producer (the whole warp walks the loop, one elected lane issues) ----------------
+    // (stage index and phase advance by increments: a division by the run-time stage count costs some 200 cycles of
+    // dependent instructions per k-tile)
+    int s = 0; uint32_t ph = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+      const int batch = (int)fd_div((uint32_t)tile, q.fd_tiles_mn), r = tile - batch * tiles_mn;
+      const int tm = (int)fd_div((uint32_t)r, q.fd_tiles_n), tn = r - tm * p.tiles_n;
+      const int b1 = (int)fd_div((uint32_t)batch, q.fd_batch0), b0 = batch - b1 * p.batch_ext[0];
+      // a batch dim an operand is broadcast over has stride 0 and extent 1 in its tensor map
+      const int ab0 = p.A.batch_stride[0] ? b0 : 0, ab1 = p.A.batch_stride[1] ? b1 : 0;
+      const int bb0 = p.B.batch_stride[0] ? b0 : 0, bb1 = p.B.batch_stride[1] ? b1 : 0;
+      for (int kt = 0; kt < k_tiles; ++kt) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph ^ 1, abort_flag))) { ok = false; break; }
+        if (elect_one()) {
           uint8_t* sa = smem + (size_t)s * stage_bytes;
           uint8_t* sb = sa + a_bytes;
           mbar_expect_tx(&full_bar[s], stage_bytes);
@@ -107,43 +108,42 @@ gemm_tc_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Gem
             for (int j = 0; j < BN / 64; ++j)
               tma_load_4d(sb + j * (64 * TC_BK * 2), &tmB, &full_bar[s], tn * BN + j * 64, kt * TC_BK, bb0, bb1);
           }
-          if (++s == stages) { s = 0; ph ^= 1; }
         }
+        if (++s == stages) { s = 0; ph ^= 1; }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      // instruction descriptor: D fp32, A/B bf16, A K-major, B per operand, N, M=128
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((q.b_kmajor ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) |
-                             ((uint32_t)(TC_BM >> 4) << 24);
-      uint32_t tcount = 0;
-      int s = 0; uint32_t ph = 0;
-      bool ok = true;
-      // descriptors of stage 0; a stage further on adds stage_bytes / 16 to the address field, a k-step 2 (32 bytes)
-      // or, for an MN-major B, 128 (2048 bytes)
-      const uint64_t da0 = make_desc(smem_u32(smem), 16, 1024);
-      const uint64_t db0 = q.b_kmajor ? make_desc(smem_u32(smem) + a_bytes, 16, 1024) : make_desc(smem_u32(smem) + a_bytes, 64 * TC_BK * 2, 1024);
-      const uint64_t dstage = stage_bytes >> 4, dbk = q.b_kmajor ? 2 : 128;
-      uint64_t da_s = da0, db_s = db0;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
-        const int acc = tcount & 1;
-        const uint32_t aph = (tcount >> 1) & 1;
-        if (!mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-        for (int kt = 0; kt < k_tiles; ++kt) {
-          if (!mbar_wait(&full_bar[s], ph, abort_flag)) { ok = false; break; }
-          // (no tcgen05 fence: TMA wrote the operands and the barrier orders its completion before the MMAs' reads)
+    // ---------------- MMA issuer ----------------
+    // instruction descriptor: D fp32, A/B bf16, A K-major, B per operand, N, M=128
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((q.b_kmajor ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) |
+                           ((uint32_t)(TC_BM >> 4) << 24);
+    uint32_t tcount = 0;
+    int s = 0; uint32_t ph = 0;
+    bool ok = true;
+    // descriptors of stage 0; a stage further on adds stage_bytes / 16 to the address field, a k-step 2 (32 bytes)
+    // or, for an MN-major B, 128 (2048 bytes)
+    const uint64_t da0 = make_desc(smem_u32(smem), 16, 1024);
+    const uint64_t db0 = q.b_kmajor ? make_desc(smem_u32(smem) + a_bytes, 16, 1024) : make_desc(smem_u32(smem) + a_bytes, 64 * TC_BK * 2, 1024);
+    const uint64_t dstage = stage_bytes >> 4, dbk = q.b_kmajor ? 2 : 128;
+    uint64_t da_s = da0, db_s = db0;
+    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
+      const int acc = tcount & 1;
+      const uint32_t aph = (tcount >> 1) & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag))) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+      for (int kt = 0; kt < k_tiles; ++kt) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], ph, abort_flag))) { ok = false; break; }
+        // (no tcgen05 fence: TMA wrote the operands and the barrier orders its completion before the MMAs' reads)
+        if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < TC_BK / 16; ++kk)
             tc_mma_bf16(d_tmem, da_s + 2 * kk, db_s + dbk * kk, idesc, (kt | kk) ? 1u : 0u);
           tc_commit(&empty_bar[s]);          // frees the smem stage once these MMAs have read it
-          da_s += dstage; db_s += dstage;
-          if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
+          if (kt + 1 == k_tiles) tc_commit(&tfull_bar[acc]);   // accumulator complete
         }
-        if (ok) tc_commit(&tfull_bar[acc]);  // accumulator complete
-        if (tcount == 0) TRACE(4);
+        da_s += dstage; db_s += dstage;
+        if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
       }
     }
   } else {

@@ -30,6 +30,7 @@
 #include "ir.h"
 #include "tc2_common.cuh"
 #include "tma_host.h"
+#include "warp_issue.cuh"
 
 namespace dnnf {
 
@@ -68,7 +69,7 @@ gemm_tc2_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Pa
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(c_bar + 2 * EPI_WARPS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const bool leader = rank == 0;
   pdl_launch_dependents();
@@ -96,25 +97,25 @@ gemm_tc2_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Pa
   const int total = n_tiles * q.ksplit;        // work items: (tile, K slice); item = slice * n_tiles + tile
 
   if (warp == 0 || warp == kProducer2) {
-    if (lane == 0) {
-      // ---------------- TMA producers (both CTAs): own 128 rows of A, own half of B ----------------
-      // Two producer threads take alternate ring stages: a stage costs its producer a wait, an expect and three or four
-      // TMA requests at 50 to 80 ns each, more than the MMA thread spends on it.
-      // (stage index and phase advance by increments: a division by the run-time stage count costs this
-      // single thread some 200 cycles of dependent instructions per k-tile)
-      const uint32_t mine = warp == 0 ? 0u : 1u;
-      uint32_t turn = 0;
-      int s = 0; uint32_t ph = 0;
-      bool ok = true;
-      for (int item = pair; item < total && ok; item += n_pairs) {
-        const int ks = (int)fd_div((uint32_t)item, q.fd_tiles), tile = item - ks * n_tiles;
-        const int tm = (int)fd_div((uint32_t)tile, q.fd_tiles_n), tn = tile - tm * tiles_n;
-        const int m0 = tm * 256 + (int)rank * BM, n0 = tn * BN + (int)rank * HB;
-        const int kt_end = min(k_tiles, (ks + 1) * q.kt_per);
-        for (int kt = ks * q.kt_per; kt < kt_end; kt += kpack, turn ^= 1u) {
-          if (turn == mine) {
-            { long long t0 = clock64(); if (!mbar_wait(&empty_bar[s], ph ^ 1, abort_flag)) { ok = false; break; } T2ACC(0, clock64() - t0); }
-            const uint32_t lbar = mapa(smem_u32(&full_bar[s]), 0);
+    // ---------------- TMA producers (both CTAs): own 128 rows of A, own half of B ----------------
+    // Two producer warps take alternate ring stages; the whole warp walks the loop, one elected lane issues.
+    // (stage index and phase advance by increments: a division by the run-time stage count costs some 200 cycles of
+    // dependent instructions per k-tile)
+    const uint32_t mine = warp == 0 ? 0u : 1u;
+    uint32_t turn = 0;
+    int s = 0; uint32_t ph = 0;
+    bool ok = true;
+    const uint32_t lbar0 = mapa(smem_u32(&full_bar[0]), 0);
+    for (int item = pair; item < total && ok; item += n_pairs) {
+      const int ks = (int)fd_div((uint32_t)item, q.fd_tiles), tile = item - ks * n_tiles;
+      const int tm = (int)fd_div((uint32_t)tile, q.fd_tiles_n), tn = tile - tm * tiles_n;
+      const int m0 = tm * 256 + (int)rank * BM, n0 = tn * BN + (int)rank * HB;
+      const int kt_end = min(k_tiles, (ks + 1) * q.kt_per);
+      for (int kt = ks * q.kt_per; kt < kt_end; kt += kpack, turn ^= 1u) {
+        if (turn == mine) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph ^ 1, abort_flag))) { ok = false; break; }
+          const uint32_t lbar = lbar0 + 8u * (uint32_t)s;
+          if (elect_one()) {
             if (leader) mbar_expect_tx(&full_bar[s], 2 * stage_bytes);
             // (a k-tile past K, when k_tiles is odd and kpack is 2, arrives as zeros: its MMAs add nothing)
             for (int u = 0; u < kpack; ++u) {
@@ -129,41 +130,38 @@ gemm_tc2_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Pa
               }
             }
           }
-          if (++s == stages) { s = 0; ph ^= 1; }
         }
+        if (++s == stages) { s = 0; ph ^= 1; }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      if (leader) {
-        // ---------------- MMA issuer (leader CTA only) ----------------
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((q.b_kmajor ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) |
-                               ((uint32_t)(256 >> 4) << 24);
-        uint32_t tcount = 0;
-        int s = 0; uint32_t ph = 0;
-        bool ok = true;
-        TR(long long r_tempty = 0, r_wait = 0, r_mma = 0, r_commit = 0, r_n = 0);
-        // descriptors of stage 0; a stage further on adds stage_bytes / 16 to the address field, a k-step 2 (32 bytes)
-        // or, for an MN-major B, 128 (2048 bytes); the barriers' cluster addresses are 8 bytes apart
-        const uint64_t da0 = make_desc(smem_u32(smem), 16, 1024);
-        const uint64_t db0 = q.b_kmajor ? make_desc(smem_u32(smem) + a_bytes, 16, 1024) : make_desc(smem_u32(smem) + a_bytes, 64 * BK * 2, 1024);
-        const uint64_t dstage = stage_bytes >> 4, dsub = sub_bytes >> 4, dbk = q.b_kmajor ? 2 : 128;
-        const uint32_t e_local = smem_u32(&empty_bar[0]);
-        uint64_t da_s = da0, db_s = db0;
-        for (int item = pair; item < total && ok; item += n_pairs, ++tcount) {
-          const int acc = tcount & 1;
-          const uint32_t aph = (tcount >> 1) & 1;
-          { long long t0 = clock64(); if (!mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag)) { ok = false; break; } TR(r_tempty += clock64() - t0); }
-          tc_fence_after();
-          const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-          const int ks = (int)fd_div((uint32_t)item, q.fd_tiles);
-          const int kt_begin = ks * q.kt_per, kt_end = min(k_tiles, kt_begin + q.kt_per);
-          for (int kt = kt_begin; kt < kt_end; kt += kpack) {
-            TR(const long long t0 = clock64());
-            if (!mbar_wait(&full_bar[s], ph, abort_flag)) { ok = false; break; }
-            TR(const long long t1 = clock64());
-            // (no tcgen05 fence here: the operands were written by TMA, and the barrier orders its completion before
-            // the MMAs' reads.  Every instruction of this thread that goes to an asynchronous unit costs 50 to 80 ns.)
+    if (leader) {
+      // ---------------- MMA issuer (leader CTA only) ----------------
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((q.b_kmajor ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) |
+                             ((uint32_t)(256 >> 4) << 24);
+      uint32_t tcount = 0;
+      int s = 0; uint32_t ph = 0;
+      bool ok = true;
+      // descriptors of stage 0; a stage further on adds stage_bytes / 16 to the address field, a k-step 2 (32 bytes)
+      // or, for an MN-major B, 128 (2048 bytes); the barriers' cluster addresses are 8 bytes apart
+      const uint64_t da0 = make_desc(smem_u32(smem), 16, 1024);
+      const uint64_t db0 = q.b_kmajor ? make_desc(smem_u32(smem) + a_bytes, 16, 1024) : make_desc(smem_u32(smem) + a_bytes, 64 * BK * 2, 1024);
+      const uint64_t dstage = stage_bytes >> 4, dsub = sub_bytes >> 4, dbk = q.b_kmajor ? 2 : 128;
+      const uint32_t e_local = smem_u32(&empty_bar[0]), t_local = smem_u32(&tfull_bar[0]);
+      uint64_t da_s = da0, db_s = db0;
+      for (int item = pair; item < total && ok; item += n_pairs, ++tcount) {
+        const int acc = tcount & 1;
+        const uint32_t aph = (tcount >> 1) & 1;
+        if (!__all_sync(0xffffffffu, mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag))) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+        const int ks = (int)fd_div((uint32_t)item, q.fd_tiles);
+        const int kt_begin = ks * q.kt_per, kt_end = min(k_tiles, kt_begin + q.kt_per);
+        for (int kt = kt_begin; kt < kt_end; kt += kpack) {
+          if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], ph, abort_flag))) { ok = false; break; }
+          // (no tcgen05 fence here: the operands were written by TMA, and the barrier orders its completion before
+          // the MMAs' reads)
+          if (elect_one()) {
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk)
               tc_mma2(d_tmem, da_s + 2 * kk, db_s + dbk * kk, idesc, ((kt - kt_begin) | kk) ? 1u : 0u);
@@ -174,15 +172,12 @@ gemm_tc2_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Pa
             }
             // stage free in both CTAs once these MMAs have read it: ONE commit, delivered to the barrier at this offset
             // in both CTAs of the pair.
-            TR(const long long t2 = clock64());
             tc_commit2_both(e_local + 8u * (uint32_t)s);
-            TR(const long long t3 = clock64(); r_wait += t1 - t0; r_mma += t2 - t1; r_commit += t3 - t2; r_n += 1);
-            da_s += dstage; db_s += dstage;
-            if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
+            if (kt + kpack >= kt_end) tc_commit2_both(t_local + 8u * (uint32_t)acc);
           }
-          if (ok) tc_commit2_both(smem_u32(&tfull_bar[acc]));
+          da_s += dstage; db_s += dstage;
+          if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
         }
-        TR(if (blockIdx.x == 0 && p.status) { long long* t = reinterpret_cast<long long*>(p.status) + 4; t[10] = r_tempty; t[11] = r_wait; t[12] = r_mma; t[13] = r_commit; t[14] = r_n; t[15] = clock64() - t_begin; });
       }
     }
   } else if (warp < 2 + EPI_WARPS) {

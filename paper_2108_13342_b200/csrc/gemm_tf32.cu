@@ -12,7 +12,7 @@
 // One persistent CTA per SM, 448 threads, warp-specialised:
 //   warp 0        TMA producer: raw fp32 row blocks of A (whole rows: one contiguous piece of memory
 //                 per block when A is dense) into a shared-memory ring; it starts before B is ready
-//   warp 1        TMEM allocation, then MMA issue (one elected lane); the A operand of every MMA
+//   warp 1        TMEM allocation, then MMA issue; the A operand of every MMA
 //                 comes from tensor memory, only B is read from shared memory
 //   warps 2..9    epilogue.  Fast form (dense fp32 output, row-invariant or dense operands): a lane
 //                 keeps 32 columns of its own row, row-invariant operands (scale, shift, bias) come
@@ -41,6 +41,7 @@
 #include "tc_common.cuh"
 #include "fp32_epilogues.h"
 #include "tma_host.h"
+#include "warp_issue.cuh"
 
 namespace dnnf {
 
@@ -275,7 +276,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint32_t* stage_area = reinterpret_cast<uint32_t*>(epi);       // general form: EPI_WARPS x kStageWords
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int n_epi = q.epi_warps, conv_sets = (EPI_WARPS + CONV_WARPS - n_epi) / 4;   // converter sets take chunks in turn
   const int rb = q.rb, units = BM / rb;                            // a raw block holds rb rows; `units` blocks per tile
   pdl_launch_dependents();
@@ -300,19 +301,19 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
 
   if (warp == 0) {
     // ---------------- TMA producer: starts at once, while the other warps still prepare B ----------------
-    if (lane == 0) {
-      pdl_wait();
-      // (ring positions and phases advance by increments everywhere: a division by a run-time stage count
-      // costs a lone thread some 200 cycles of dependent instructions)
-      int s = 0; uint32_t ph = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        for (int u = 0; u < units; ++u) {
-          { long long t0 = clock64(); if (!mbar_wait(&empty_bar[s], ph ^ 1, abort_flag)) { ok = false; break; } FACC(1, clock64() - t0); }
+    pdl_wait();
+    // (ring positions and phases advance by increments everywhere: a division by a run-time stage count
+    // costs some 200 cycles of dependent instructions)
+    int s = 0; uint32_t ph = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+      for (int u = 0; u < units; ++u) {
+        { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph ^ 1, abort_flag))) { ok = false; break; } if (lane == 0) FACC(1, clock64() - t0); }
+        if (elect_one()) {
           mbar_expect_tx(&raw_bar[s], (uint32_t)(rb * q.pitch * 4));
           tma_load_2d(ring + (size_t)s * q.unit_stride, &q.tmA, &raw_bar[s], 0, tile * BM + u * rb);
-          if (++s == stages) { s = 0; ph ^= 1; }
         }
+        if (++s == stages) { s = 0; ph ^= 1; }
       }
     }
   } else {
@@ -386,34 +387,34 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   }
 
   if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      // instruction descriptors: D fp32, A/B tf32, both K-major, M = 128, N = NP or 2*NP
-      const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BM >> 4) << 24);
-      const uint32_t idesc = idesc0 | ((uint32_t)(NP >> 3) << 17), idesc2 = idesc0 | ((uint32_t)(NP >> 2) << 17);
-      const uint32_t b_base = smem_u32(smem);
-      const bool dual = q.dual != 0;
-      uint32_t tcount = 0;
-      int s = 0; uint32_t ph = 0;
-      bool ok = true;
-      const uint64_t db0 = make_desc(b_base, 16, 1024);          // B_hi of K atom 0; + atom_bytes / 16 per atom, + lo_off / 16 for B_lo
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
-        const int acc = tcount & 1;
-        const uint32_t aph = (tcount >> 1) & 1;
-        { long long t0 = clock64(); if (!mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag)) { ok = false; break; } FACC(2, clock64() - t0); }
+    // ---------------- MMA issuer (the whole warp walks the loop, one elected lane issues) ----------------
+    // instruction descriptors: D fp32, A/B tf32, both K-major, M = 128, N = NP or 2*NP
+    const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BM >> 4) << 24);
+    const uint32_t idesc = idesc0 | ((uint32_t)(NP >> 3) << 17), idesc2 = idesc0 | ((uint32_t)(NP >> 2) << 17);
+    const uint32_t b_base = smem_u32(smem);
+    const bool dual = q.dual != 0;
+    uint32_t tcount = 0;
+    int s = 0; uint32_t ph = 0;
+    bool ok = true;
+    const uint64_t db0 = make_desc(b_base, 16, 1024);          // B_hi of K atom 0; + atom_bytes / 16 per atom, + lo_off / 16 for B_lo
+    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
+      const int acc = tcount & 1;
+      const uint32_t aph = (tcount >> 1) & 1;
+      { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag))) { ok = false; break; } if (lane == 0) FACC(2, clock64() - t0); }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * acc_cols);
+      const long long t_tile = clock64();
+      uint64_t dbh = db0;
+      int k_left = p.K;
+      for (int kc = 0; kc < k_chunks; ++kc, k_left -= BK, dbh += atom_bytes >> 4) {
+        { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&conv_bar[s], ph, abort_flag))) { ok = false; break; } if (lane == 0) FACC3(3, clock64() - t0); }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * acc_cols);
-        const long long t_tile = clock64();
-        uint64_t dbh = db0;
-        int k_left = p.K;
-        for (int kc = 0; kc < k_chunks; ++kc, k_left -= BK, dbh += atom_bytes >> 4) {
-          { long long t0 = clock64(); if (!mbar_wait(&conv_bar[s], ph, abort_flag)) { ok = false; break; } FACC3(3, clock64() - t0); }
-          tc_fence_after();
-          const long long t_issue = clock64();
-          const int ksteps = min(BK, k_left + 7) >> 3;                   // 8 tf32 per MMA
-          const uint32_t a_hi = tmem_base + a_cols0 + (uint32_t)(s * kAStageCols), a_lo = a_hi + BK;
-          // B descriptors advance by 32 bytes (2 units of 16) per k-step inside the swizzled atom
-          const uint64_t dbl = dbh + (lo_off >> 4);
+        const long long t_issue = clock64();
+        const int ksteps = min(BK, k_left + 7) >> 3;                   // 8 tf32 per MMA
+        const uint32_t a_hi = tmem_base + a_cols0 + (uint32_t)(s * kAStageCols), a_lo = a_hi + BK;
+        // B descriptors advance by 32 bytes (2 units of 16) per k-step inside the swizzled atom
+        const uint64_t dbl = dbh + (lo_off >> 4);
+        if (elect_one()) {
           if (q.debug & 2) {
           } else if (dual) {
 #pragma unroll
@@ -434,14 +435,14 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
             }
           }
           tc_commit(&afree_bar[s]);          // frees the A stage once these MMAs have read it
-          if (++s == a_stages) { s = 0; ph ^= 1; }
-          FACC3(4, clock64() - t_issue);
+          if (kc + 1 == k_chunks) tc_commit(&tfull_bar[acc]);  // accumulator complete
         }
-        FACC(10, clock64() - t_tile);
-        if (ok) tc_commit(&tfull_bar[acc]);  // accumulator complete
+        if (++s == a_stages) { s = 0; ph ^= 1; }
+        if (lane == 0) FACC3(4, clock64() - t_issue);
       }
-      FACC(11, clock64() - t_begin);
+      if (lane == 0) FACC(10, clock64() - t_tile);
     }
+    if (lane == 0) FACC(11, clock64() - t_begin);
   } else if (warp >= 2 && warp < 2 + n_epi) {
     // ---------------- epilogue warps ----------------
     const int sub = warp & 3;                 // TMEM sub-partition this warp may read

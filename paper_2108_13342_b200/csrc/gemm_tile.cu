@@ -28,6 +28,7 @@
 #include "ir.h"
 #include "tc2_common.cuh"
 #include "tma_host.h"
+#include "warp_issue.cuh"
 
 namespace dnnf {
 
@@ -78,14 +79,6 @@ __device__ __forceinline__ bool mbar_wait_cta(uint64_t* bar, uint32_t parity, vo
     if (*abort_flag) return false;
     if (wall_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; return false; }
   }
-}
-// One lane of a converged warp.  The role loops below run in ALL lanes of their warp with identical values and only
-// the issuing instruction sits under this predicate: the compiler then keeps descriptors, coordinates and barrier
-// addresses in uniform registers instead of moving them there, lane by lane, in front of every TMA / MMA instruction.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred;
-  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(pred));
-  return pred != 0;
 }
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
@@ -175,7 +168,7 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(c_bar + kEpiWarps);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   pdl_launch_dependents();
   if (threadIdx.x == 0) TSTAMP(0);
   if (threadIdx.x == 0) {
@@ -209,68 +202,68 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
 
   if (warp < 2) {
     // ---------------- TMA producers: warp j loads the k-tiles j, j+2, j+4, ... ----------------
-    // Each instruction that goes to an asynchronous unit (a barrier wait, a TMA request, an MMA, a commit) costs its
-    // issuing thread 50 to 80 ns, whatever the size of the operation (measured: a ring that only passes barriers back
-    // and forth, without loads or MMAs, still takes 210 ns per k-tile).  Two producers on alternate k-tiles keep the
-    // loads off the critical path; the issuer's own instructions (a wait, four MMAs, a commit) then set the pace.
-    if (lane == 0) {
-      auto load_b = [&](int s, int kt) {
-        uint8_t* sb = smem + (size_t)s * stage_bytes + a_bytes;
-        if (q.b_kmajor) {
-          tma_load_2d(sb, &q.tmB, &full_bar[s], (kt0 + kt) * BK, n0);
-        } else {
-          for (int j = 0; j < BN / 64; ++j) tma_load_2d(sb + j * (64 * BK * 2), &q.tmB, &full_bar[s], n0 + j * 64, (kt0 + kt) * BK);
-        }
-      };
-      auto load_a = [&](int s, int kt) { tma_load_2d(smem + (size_t)s * stage_bytes, &q.tmA, &full_bar[s], (kt0 + kt) * BK, m0); };
-      const int npre = min(stages, k_tiles);
-      // a weight operand is written by no kernel: its first stages are requested while the previous kernel still runs
-      if (q.b_static)
-        for (int kt = warp; kt < npre; kt += 2) { mbar_expect_tx(&full_bar[kt], stage_bytes); load_b(kt, kt); }
-      pdl_wait();
-      if (warp == 0) TSTAMP(2);
-      for (int kt = warp; kt < npre; kt += 2) {
+    // The whole warp walks the loop, one elected lane issues.  Two producers on alternate k-tiles keep the
+    // loads off the critical path: a k-tile of three requests costs its producer about as much as the issuer's four MMAs.
+    auto load_b = [&](int s, int kt) {
+      uint8_t* sb = smem + (size_t)s * stage_bytes + a_bytes;
+      if (q.b_kmajor) {
+        tma_load_2d(sb, &q.tmB, &full_bar[s], (kt0 + kt) * BK, n0);
+      } else {
+        for (int j = 0; j < BN / 64; ++j) tma_load_2d(sb + j * (64 * BK * 2), &q.tmB, &full_bar[s], n0 + j * 64, (kt0 + kt) * BK);
+      }
+    };
+    auto load_a = [&](int s, int kt) { tma_load_2d(smem + (size_t)s * stage_bytes, &q.tmA, &full_bar[s], (kt0 + kt) * BK, m0); };
+    const int npre = min(stages, k_tiles);
+    // a weight operand is written by no kernel: its first stages are requested while the previous kernel still runs
+    if (q.b_static)
+      for (int kt = warp; kt < npre; kt += 2)
+        if (elect_one()) { mbar_expect_tx(&full_bar[kt], stage_bytes); load_b(kt, kt); }
+    pdl_wait();
+    if (threadIdx.x == 0) TSTAMP(2);
+    for (int kt = warp; kt < npre; kt += 2) {
+      if (elect_one()) {
         if (!q.b_static) { mbar_expect_tx(&full_bar[kt], stage_bytes); load_b(kt, kt); }
         load_a(kt, kt);
       }
-      // first k-tile of this warp at or beyond the pre-issued ones
-      int kt = npre + ((npre ^ warp) & 1);
-      int s = kt - stages; uint32_t ph = 0;
-      while (s >= stages) { s -= stages; ph ^= 1; }
-      for (; kt < k_tiles; kt += 2) {
-        if (!mbar_wait_cta(&empty_bar[s], ph, abort_flag)) break;
+    }
+    // first k-tile of this warp at or beyond the pre-issued ones
+    int kt = npre + ((npre ^ warp) & 1);
+    int s = kt - stages; uint32_t ph = 0;
+    while (s >= stages) { s -= stages; ph ^= 1; }
+    for (; kt < k_tiles; kt += 2) {
+      if (!__all_sync(0xffffffffu, mbar_wait_cta(&empty_bar[s], ph, abort_flag))) break;
+      if (elect_one()) {
         mbar_expect_tx(&full_bar[s], stage_bytes);
         load_a(s, kt);
         load_b(s, kt);
-        s += 2;
-        if (s >= stages) { s -= stages; ph ^= 1; }
       }
+      s += 2;
+      if (s >= stages) { s -= stages; ph ^= 1; }
     }
     if (kSplit) { __syncwarp(); cluster_sync(); cluster_sync(); }
   } else if (warp == 2) {
     // ---------------- MMA issuer ----------------
     // (No tcgen05 fence inside the loop: the operands were written by TMA, whose completion the barrier itself orders
-    // before the MMAs' reads; an instruction saved per k-tile is 50 ns saved.)
-    if (lane == 0) {
-      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((q.b_kmajor ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) |
-                             ((uint32_t)(BM >> 4) << 24);
-      const uint64_t da0 = make_desc(smem_u32(smem), 16, 1024);
-      const uint64_t db0 = q.b_kmajor ? make_desc(smem_u32(smem) + a_bytes, 16, 1024) : make_desc(smem_u32(smem) + a_bytes, 64 * BK * 2, 1024);
-      const uint64_t dstage = stage_bytes >> 4, dbk = q.b_kmajor ? 2 : 128;
-      uint64_t da_s = da0, db_s = db0;
-      int s = 0; uint32_t ph = 0;
-      bool ok = true;
-      for (int kt = 0; kt < k_tiles; ++kt) {
-        if (!mbar_wait_cta(&full_bar[s], ph, abort_flag)) { ok = false; break; }
-        if (kt == 0) TSTAMP(3);
-        if (kt == k_tiles - 1) TSTAMP(4);
+    // before the MMAs' reads.)
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((q.b_kmajor ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) |
+                           ((uint32_t)(BM >> 4) << 24);
+    const uint64_t da0 = make_desc(smem_u32(smem), 16, 1024);
+    const uint64_t db0 = q.b_kmajor ? make_desc(smem_u32(smem) + a_bytes, 16, 1024) : make_desc(smem_u32(smem) + a_bytes, 64 * BK * 2, 1024);
+    const uint64_t dstage = stage_bytes >> 4, dbk = q.b_kmajor ? 2 : 128;
+    uint64_t da_s = da0, db_s = db0;
+    int s = 0; uint32_t ph = 0;
+    for (int kt = 0; kt < k_tiles; ++kt) {
+      if (!__all_sync(0xffffffffu, mbar_wait_cta(&full_bar[s], ph, abort_flag))) break;
+      if (kt == 0 && lane == 0) TSTAMP(3);
+      if (kt == k_tiles - 1 && lane == 0) TSTAMP(4);
+      if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk) tc_mma1(tmem_base, da_s + 2 * kk, db_s + dbk * kk, idesc, (kt | kk) ? 1u : 0u);
-        if (kt + stages < k_tiles) tc_commit1(&empty_bar[s]);     // only a stage that is refilled needs the signal
-        da_s += dstage; db_s += dstage;
-        if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
+        if (kt + stages < k_tiles) tc_commit1(&empty_bar[s]);         // only a stage that is refilled needs the signal
+        if (kt + 1 == k_tiles) tc_commit1(tfull_bar);                 // accumulator complete
       }
-      if (ok) tc_commit1(tfull_bar);         // accumulator complete
+      da_s += dstage; db_s += dstage;
+      if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
     }
     if (kSplit) { __syncwarp(); cluster_sync(); cluster_sync(); }
   } else {
