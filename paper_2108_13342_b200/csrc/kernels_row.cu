@@ -13,6 +13,9 @@ int launch_row_e(const Launch& L, cudaStream_t st);
 int launch_row_f(const Launch& L, cudaStream_t st);
 int launch_row_g(const Launch& L, cudaStream_t st);
 int launch_row_h(const Launch& L, cudaStream_t st);
+int launch_row_i(const Launch& L, cudaStream_t st);
+int launch_row_j(const Launch& L, cudaStream_t st);
+int launch_row_k(const Launch& L, cudaStream_t st);
 
 // variant encoding: V * 100000 + NV * 1000 + WPR * 10 + RPW
 int launch_row(const Launch& L, cudaStream_t st) {
@@ -25,6 +28,9 @@ int launch_row(const Launch& L, cudaStream_t st) {
   if (rc == 2) rc = launch_row_f(L, st);
   if (rc == 2) rc = launch_row_g(L, st);
   if (rc == 2) rc = launch_row_h(L, st);
+  if (rc == 2) rc = launch_row_i(L, st);
+  if (rc == 2) rc = launch_row_j(L, st);
+  if (rc == 2) rc = launch_row_k(L, st);
   return rc;
 }
 
@@ -61,10 +67,16 @@ bool finalize_row(Launch& L) {
       wpr = 8; int n8 = fit(8); nv = n8 <= 2 ? 2 : n8 <= 4 ? 4 : 8; if (n8 > 8) return false;
     }
   } else {
-    int need = (Lr + 31) / 32;
-    if (need <= 1) { nv = 1; rpw = 4; }
-    else if (need <= 16) nv = need <= 4 ? 4 : 16;
-    else { wpr = 8; int n8 = (Lr + 255) / 256; nv = n8 <= 8 ? 8 : 32; if (n8 > 32) return false; }
+    // Rows whose length or start fits no 16-byte vector: one element per lane and load, 128 (bf16: 64) contiguous bytes per
+    // warp instruction.  What bounds it is the loads in flight and the instructions per element, so the row gets the
+    // fewest elements per lane that hold it and the compile-time chain tables.  [8,12,197,197] fp32 masked softmax: 75.8 us
+    // with 16 elements per lane and the interpreted chain, 8.2 us with 8 and the table.  With few rows of more than 128
+    // elements (under eight warps per SM) eight warps share a row.
+    const int need = (Lr + 31) / 32;
+    if (need <= 1) { nv = 1; rpw = 4; while (rpw > 1 && (p.rows + rpw - 1) / rpw < target) rpw /= 2; if (rpw == 2) rpw = 1; }
+    else if (need <= 4) nv = 4;
+    else if (need <= 16 && p.rows >= 8L * sm_count()) nv = need <= 8 ? 8 : 16;
+    else { wpr = 8; const int n8 = (Lr + 255) / 256; nv = n8 <= 4 ? 4 : n8 <= 8 ? 8 : n8 <= 16 ? 16 : 32; if (n8 > 32) return false; }
   }
   // a warp's rows are consecutive along outer dim 1: they must not straddle it
   if (rpw > 1 && nd > 2 && p.it.extent[1] % rpw != 0) rpw = 1;
@@ -72,7 +84,7 @@ bool finalize_row(Launch& L) {
   int64_t warps = (p.rows + rpw - 1) / rpw;
   L.grid = wpr > 1 ? (int)p.rows : (int)((warps + kRowWarpsPerCta - 1) / kRowWarpsPerCta);
   L.threads = wpr > 1 ? 32 * wpr : 32 * kRowWarpsPerCta;
-  L.static_id = (V == 4 && (wpr < 8 || nv == 1)) ? StaticSet<RowStatic>::find(p.prog) : 0;
+  L.static_id = (V == 4 ? (wpr < 8 || nv == 1) : nv < 32) ? StaticSet<RowStatic>::find(p.prog) : 0;
   set_fastdiv(p.it);
   return true;
 }
