@@ -2,14 +2,17 @@
 //
 // Table 2 lists the operator under Many-to-Many: every result depends on all H x W positions of its own (image,
 // channel) plane.  Like the other Many-to-Many anchors it takes One-to-One successors as an epilogue and nothing in
-// front.  A CTA owns one image and a group of 4, 8, 16 or 32 neighbouring channels (one to eight 128-bit lanes; the host
-// picks the widest group that still gives two CTAs per SM; where images and channels are few it also splits the plane over
-// a cluster of 2, 4 or 8 CTAs whose partial sums meet through distributed shared memory and the cluster's hardware
-// barrier) and walks its part of the plane three times: sum -> mean, sum of squared
-// deviations -> variance (two passes, as the definition reads; no E[x^2] - mean^2 cancellation), then normalise, scale,
-// shift, run the chain and store.  The second and third walk find the slab in L1 / L2 (H x W x 16..128 bytes), so the
-// kernel's HBM traffic is the input once plus the output once.  Reductions: shuffles among the lanes of a warp that hold
-// the same channels, then one shared-memory exchange between the warps, always in the same order.
+// front.  A CTA owns one image, a group of 4, 8, 16 or 32 neighbouring channels (one to eight 128-bit lanes) and a part of
+// the plane; the parts of a plane form a cluster of up to 16 CTAs.
+//
+// The plane is read ONCE where its part fits the CTA's registers (kResident float4 per thread: 8 or 16), else a second time
+// out of L2 for the normalisation.  Mean and sum of squared deviations never pass through E[x^2] - mean^2: a CTA's
+// deviations are taken from its own mean (resident values exactly, streamed values by the pairwise update of Chan, Golub and
+// LeVeque in batches of eight pixels), and (count, mean, deviations) of the CTAs of a plane are merged by the same formula
+// in rank order after ONE exchange through distributed shared memory and the cluster's hardware barrier.
+// What bounds it: HBM where planes are large, else the latency of the exchange.  Three walks over the plane with
+// two exchanges and four loads in flight took 49.8 us for [8,256,256,16], 28.3 for [8,128,128,32] and 11.5 for [8,64,64,64] with
+// a ReLU (cold inputs); this form 26.4, 15.5 and 8.5.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -29,7 +32,9 @@ struct InstNormParams {
   float eps;
   int32_t lanes;           // 128-bit lanes per pixel a CTA works on: 1, 2, 4 or 8 (4 channels each)
   int32_t groups;          // channel groups per image: ceil(C / (4 * lanes))
-  int32_t split;           // CTAs (one cluster) that share a plane: 1, 2, 4 or 8
+  int32_t split;           // CTAs (one cluster) that share a plane: 1, 2, 4, 8 or 16
+  int32_t resident;        // pixels a thread keeps in registers: 0 (streamed twice), 8 or 16
+  FastDiv fd_w;
 };
 
 namespace {
@@ -56,30 +61,21 @@ __device__ __forceinline__ float4 plane_sum(float4 v, int lanes, float4 (*xchg)[
   return s;
 }
 
-// sum of the CTAs' results over the cluster, in rank order; `mine` is this CTA's slot in its own shared memory
-template <bool kCluster>
-__device__ __forceinline__ float4 cluster_sum(float4 v, float4* mine, int lanes, int split) {
-  if (!kCluster) return v;
-  namespace cg = cooperative_groups;
-  cg::cluster_group cluster = cg::this_cluster();
-  if ((int)threadIdx.x < lanes) mine[threadIdx.x] = v;
-  cluster.sync();
-  float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  for (int r = 0; r < split; ++r) {
-    const float4 t = *cluster.map_shared_rank(mine + threadIdx.x % lanes, r);
-    s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
-  }
-  return s;
+__device__ __forceinline__ void add_sq(float4& m2, const float4& v, const float4& mean) {
+  const float a = v.x - mean.x, b = v.y - mean.y, c = v.z - mean.z, d = v.w - mean.w;
+  m2.x = fmaf(a, a, m2.x); m2.y = fmaf(b, b, m2.y); m2.z = fmaf(c, c, m2.z); m2.w = fmaf(d, d, m2.w);
 }
+__device__ __forceinline__ void add_f4(float4& s, const float4& v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
 
-template <class SP, bool kCluster>
-__global__ void __launch_bounds__(kThreads) instnorm_kernel(const __grid_constant__ InstNormParams p) {
+// kResident: pixels a thread keeps in registers (0: the plane is read a second time for the normalisation)
+template <class SP, int kResident>
+__global__ void __launch_bounds__(kThreads, 2) instnorm_kernel(const __grid_constant__ InstNormParams p) {
+  namespace cg = cooperative_groups;
   __shared__ float4 xchg[kThreads / 32][8];
-  __shared__ float4 cpart[2][8];                     // this CTA's sums for the cluster: one slot per pass
+  __shared__ float4 cpart[2][8];                     // this CTA's mean and deviations, read by the cluster
   pdl_launch_dependents();
   pdl_wait();
-  const int lanes = p.lanes;
-  const int split = kCluster ? p.split : 1;
+  const int lanes = p.lanes, split = p.split;
   const int plane = blockIdx.x / split, rank = blockIdx.x - plane * split;     // a cluster is `split` consecutive CTAs
   const int n = plane / p.groups, grp = plane - n * p.groups;
   const int cl = threadIdx.x % lanes, pr = threadIdx.x / lanes, prs = kThreads / lanes;
@@ -87,70 +83,132 @@ __global__ void __launch_bounds__(kThreads) instnorm_kernel(const __grid_constan
   const bool live = c < p.d.C;                       // the last group of an image may be narrower
   const int HW = p.d.H * p.d.W;
   const int per = (HW + split - 1) / split;
-  const int q_begin = rank * per, q_end = min(HW, q_begin + per);
+  const int q_begin = min(HW, rank * per), q_end = min(HW, q_begin + per);
   const float* xb = p.d.x + (size_t)n * HW * p.d.C + (live ? c : 0);
-  const float inv = 1.0f / (float)HW;
-
-  float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   const float4 zero4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  if (live)
-    for (int q = q_begin + pr; q < q_end; q += 4 * prs) {          // four loads in flight per thread
-      float4 v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = q + u * prs < q_end ? __ldg(reinterpret_cast<const float4*>(xb + (size_t)(q + u * prs) * p.d.C)) : zero4;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) { s.x += v[u].x; s.y += v[u].y; s.z += v[u].z; s.w += v[u].w; }
-    }
-  s = cluster_sum<kCluster>(plane_sum(s, lanes, xchg), cpart[0], lanes, split);
-  const float4 mean = make_float4(s.x * inv, s.y * inv, s.z * inv, s.w * inv);
+  auto pixel = [&](int q) { return __ldg(reinterpret_cast<const float4*>(xb + (size_t)q * p.d.C)); };
+  const float count = (float)(q_end - q_begin), inv = count > 0.0f ? 1.0f / count : 0.0f;
 
-  float4 m2 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  if (live)
-    for (int q = q_begin + pr; q < q_end; q += 4 * prs) {
-      float4 v[4];
+  constexpr int kKeep = kResident ? kResident : 4;
+  float4 keep[kKeep];
+  float4 mean, m2 = zero4;                           // of this CTA's part
+  if (kResident) {
+    float4 s = zero4;
 #pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = q + u * prs < q_end ? __ldg(reinterpret_cast<const float4*>(xb + (size_t)(q + u * prs) * p.d.C)) : mean;
+    for (int u = 0; u < kKeep; ++u) { const int q = q_begin + pr + u * prs; keep[u] = live && q < q_end ? pixel(q) : zero4; }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {                                 // (a pixel past the end was given the mean: deviation 0)
-        const float a = v[u].x - mean.x, b = v[u].y - mean.y, e = v[u].z - mean.z, f = v[u].w - mean.w;
-        m2.x = fmaf(a, a, m2.x); m2.y = fmaf(b, b, m2.y); m2.z = fmaf(e, e, m2.z); m2.w = fmaf(f, f, m2.w);
+    for (int u = 0; u < kKeep; ++u) add_f4(s, keep[u]);
+    s = plane_sum(s, lanes, xchg);
+    mean = make_float4(s.x * inv, s.y * inv, s.z * inv, s.w * inv);
+#pragma unroll
+    for (int u = 0; u < kKeep; ++u) if (q_begin + pr + u * prs < q_end) add_sq(m2, keep[u], mean);
+  } else {
+    constexpr int B = 8;                             // loads in flight per thread
+    float4 tm = zero4;                               // running mean of this thread's pixels
+    float have = 0.0f;
+    if (live)
+      for (int q0 = q_begin + pr; q0 < q_end; q0 += B * prs) {
+        float4 v[B], s = zero4;
+        int on = 0;
+#pragma unroll
+        for (int u = 0; u < B; ++u) { const bool in = q0 + u * prs < q_end; on += in; v[u] = in ? pixel(q0 + u * prs) : zero4; }
+#pragma unroll
+        for (int u = 0; u < B; ++u) add_f4(s, v[u]);
+        const float nb = (float)on, ib = __fdividef(1.0f, nb), total = have + nb, w = __fdividef(nb, total);
+        const float4 mb = make_float4(s.x * ib, s.y * ib, s.z * ib, s.w * ib);
+#pragma unroll
+        for (int u = 0; u < B; ++u) if (u < on) add_sq(m2, v[u], mb);
+        const float4 d = make_float4(mb.x - tm.x, mb.y - tm.y, mb.z - tm.z, mb.w - tm.w);
+        const float k = have * w;
+        m2.x = fmaf(d.x * d.x, k, m2.x); m2.y = fmaf(d.y * d.y, k, m2.y); m2.z = fmaf(d.z * d.z, k, m2.z); m2.w = fmaf(d.w * d.w, k, m2.w);
+        tm.x = fmaf(d.x, w, tm.x); tm.y = fmaf(d.y, w, tm.y); tm.z = fmaf(d.z, w, tm.z); tm.w = fmaf(d.w, w, tm.w);
+        have = total;
+      }
+    float4 s = plane_sum(make_float4(tm.x * have, tm.y * have, tm.z * have, tm.w * have), lanes, xchg);
+    mean = make_float4(s.x * inv, s.y * inv, s.z * inv, s.w * inv);
+    const float4 d = make_float4(tm.x - mean.x, tm.y - mean.y, tm.z - mean.z, tm.w - mean.w);
+    m2.x = fmaf(d.x * d.x, have, m2.x); m2.y = fmaf(d.y * d.y, have, m2.y); m2.z = fmaf(d.z * d.z, have, m2.z); m2.w = fmaf(d.w * d.w, have, m2.w);
+  }
+  m2 = plane_sum(m2, lanes, xchg);
+  if (split > 1) {                                   // merge with the other parts of the plane, in rank order
+    cg::cluster_group cluster = cg::this_cluster();
+    if ((int)threadIdx.x < lanes) { cpart[0][threadIdx.x] = mean; cpart[1][threadIdx.x] = m2; }
+    cluster.sync();
+    float4 s = zero4;
+    for (int r = 0; r < split; ++r) {
+      const float4 t = *cluster.map_shared_rank(&cpart[0][cl], r);
+      const float cnt = (float)(min(HW, (r + 1) * per) - min(HW, r * per));
+      s.x = fmaf(t.x, cnt, s.x); s.y = fmaf(t.y, cnt, s.y); s.z = fmaf(t.z, cnt, s.z); s.w = fmaf(t.w, cnt, s.w);
+    }
+    const float iall = 1.0f / (float)HW;
+    const float4 all = make_float4(s.x * iall, s.y * iall, s.z * iall, s.w * iall);
+    float4 mm = zero4;
+    for (int r = 0; r < split; ++r) {
+      const float4 t = *cluster.map_shared_rank(&cpart[0][cl], r), e = *cluster.map_shared_rank(&cpart[1][cl], r);
+      const float cnt = (float)(min(HW, (r + 1) * per) - min(HW, r * per));
+      const float4 d = make_float4(t.x - all.x, t.y - all.y, t.z - all.z, t.w - all.w);
+      mm.x += fmaf(d.x * d.x, cnt, e.x); mm.y += fmaf(d.y * d.y, cnt, e.y); mm.z += fmaf(d.z * d.z, cnt, e.z); mm.w += fmaf(d.w * d.w, cnt, e.w);
+    }
+    mean = all; m2 = mm;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // done reading the others; waited for at the end
+  }
+  if (live) {
+    const float iall = 1.0f / (float)HW;
+    const float4 sc = __ldg(reinterpret_cast<const float4*>(p.scale + c)), sh = __ldg(reinterpret_cast<const float4*>(p.shift + c));
+    // y = (x - mean) / sqrt(var + eps) * scale + shift
+    const float4 g = make_float4(sc.x / sqrtf(m2.x * iall + p.eps), sc.y / sqrtf(m2.y * iall + p.eps), sc.z / sqrtf(m2.z * iall + p.eps),
+                                 sc.w / sqrtf(m2.w * iall + p.eps));
+    // four pixels per pass of the chain
+    BatchIO<DwIO, 4> b{{DwIO{p.d}, DwIO{p.d}, DwIO{p.d}, DwIO{p.d}}, {false, false, false, false}};
+    auto finish = [&](int q, const float4& v0, const float4& v1, const float4& v2, const float4& v3) {
+      const float4 v[4] = {v0, v1, v2, v3};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int qq = q + u * prs;
+        DwIO& io = b.io[u];
+        b.on[u] = qq < q_end;
+        io.accv[0] = fmaf(v[u].x - mean.x, g.x, sh.x); io.accv[1] = fmaf(v[u].y - mean.y, g.y, sh.y);
+        io.accv[2] = fmaf(v[u].z - mean.z, g.z, sh.z); io.accv[3] = fmaf(v[u].w - mean.w, g.w, sh.w);
+        io.n = n; io.c = c; io.h = fd_div((uint32_t)qq, p.fd_w); io.w = (uint32_t)qq - io.h * (uint32_t)p.d.W;
+      }
+      run_program<16, SP>(p.d.prog, b);
+    };
+    if (kResident) {
+#pragma unroll
+      for (int u = 0; u < kKeep; u += 4) {
+        const int q = q_begin + pr + u * prs;
+        if (q < q_end) finish(q, keep[u], keep[u + 1], keep[u + 2], keep[u + 3]);
+      }
+    } else {
+      // the next four pixels are loaded while the chain of these four runs
+      auto fetch = [&](int q, float4 (&t)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t[u] = q + u * prs < q_end ? pixel(q + u * prs) : zero4;
+      };
+      float4 v[4], w[4];
+      int q = q_begin + pr;
+      if (q < q_end) fetch(q, v);
+      for (; q < q_end; q += 4 * prs) {
+        fetch(q + 4 * prs, w);
+        finish(q, v[0], v[1], v[2], v[3]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = w[u];
       }
     }
-  m2 = cluster_sum<kCluster>(plane_sum(m2, lanes, xchg), cpart[1], lanes, split);
-  if (live) {
-  const float4 sc = __ldg(reinterpret_cast<const float4*>(p.scale + c)), sh = __ldg(reinterpret_cast<const float4*>(p.shift + c));
-  // y = (x - mean) / sqrt(var + eps) * scale + shift
-  const float4 g = make_float4(sc.x / sqrtf(m2.x * inv + p.eps), sc.y / sqrtf(m2.y * inv + p.eps), sc.z / sqrtf(m2.z * inv + p.eps),
-                               sc.w / sqrtf(m2.w * inv + p.eps));
-  // four pixels per pass of the chain
-  BatchIO<DwIO, 4> b{{DwIO{p.d}, DwIO{p.d}, DwIO{p.d}, DwIO{p.d}}, {false, false, false, false}};
-  for (int q = q_begin + pr; q < q_end; q += 4 * prs) {
-    float4 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int qq = q + u * prs;
-      b.on[u] = qq < q_end;
-      v[u] = b.on[u] ? __ldg(reinterpret_cast<const float4*>(xb + (size_t)qq * p.d.C)) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int qq = q + u * prs;
-      DwIO& io = b.io[u];
-      io.accv[0] = fmaf(v[u].x - mean.x, g.x, sh.x); io.accv[1] = fmaf(v[u].y - mean.y, g.y, sh.y);
-      io.accv[2] = fmaf(v[u].z - mean.z, g.z, sh.z); io.accv[3] = fmaf(v[u].w - mean.w, g.w, sh.w);
-      io.n = n; io.c = c; io.h = qq / p.d.W; io.w = qq - io.h * p.d.W;
-    }
-    run_program<16, SP>(p.d.prog, b);
   }
+  if (split > 1) {                                   // nobody leaves while its sums may still be read
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   }
-  if (kCluster) cooperative_groups::this_cluster().sync();      // nobody leaves while its sums may still be read
 }
 
 struct InLauncher {
   const Launch& L; cudaStream_t st; cudaError_t rc = cudaSuccess;
-  template <class SP> void run() {
+  template <class SP, int R> void go() {
     const InstNormParams& q = *reinterpret_cast<const InstNormParams*>(L.blob.data());
-    if (q.split == 1) { rc = launch_pdl(instnorm_kernel<SP, false>, L.grid, kThreads, 0, st, q); return; }
+    if (q.split == 1) { rc = launch_pdl(instnorm_kernel<SP, R>, L.grid, kThreads, 0, st, q); return; }
+    static PerDeviceOnce once;       // per instantiation
+    if (once.first_use()) cudaFuncSetAttribute(instnorm_kernel<SP, R>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(L.grid); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = 0; cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -159,7 +217,14 @@ struct InLauncher {
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    rc = cudaLaunchKernelEx(&cfg, instnorm_kernel<SP, true>, q);
+    rc = cudaLaunchKernelEx(&cfg, instnorm_kernel<SP, R>, q);
+  }
+  template <class SP> void run() {
+    const int r = reinterpret_cast<const InstNormParams*>(L.blob.data())->resident;
+    if constexpr (SP::n == 0) go<SP, 0>();
+    else if (r == 8) go<SP, 8>();
+    else if (r == 16) go<SP, 16>();
+    else go<SP, 0>();
   }
 };
 }  // namespace
@@ -221,14 +286,21 @@ int lower_instnorm(const Graph& g, const std::vector<int>& ops, int anchor, Bloc
   for (auto& a : cx.ins) { L.in_tensors.push_back(a.tensor); if (std::find(out.inputs.begin(), out.inputs.end(), a.tensor) == out.inputs.end()) out.inputs.push_back(a.tensor); }
   for (auto& a : cx.outs) { L.out_tensors.push_back(a.tensor); out.outputs.push_back(a.tensor); }
   // Two CTAs per SM are wanted.  The widest channel group reads whole 128-byte lines per pixel; where images x groups are
-  // too few, first the plane is split over a cluster (as long as every CTA keeps 512 pixels), then the group narrows.
+  // too few, first the plane is split over a cluster (as long as every CTA keeps 512 pixels), then the group narrows, down to
+  // the 32 bytes of a memory sector, then the cluster grows to 16 CTAs.
   int lanes = 8, split = 1;
   while (lanes > 1 && lanes > dp.C / 4) lanes >>= 1;
   const int64_t hw = (int64_t)dp.H * dp.W, want = 2ll * sm_count();
   auto ctas = [&]() { return (int64_t)dp.N * ((dp.C / 4 + lanes - 1) / lanes) * split; };
-  while (ctas() < want && split < 8 && hw / (2 * split) >= 512) split *= 2;
-  while (ctas() < want && lanes > 1) lanes >>= 1;
+  while (2 * ctas() <= want && split < 8 && hw / (2 * split) >= 512) split *= 2;
+  while (2 * ctas() <= want && lanes > 2) lanes >>= 1;
+  if (2 * ctas() <= want && split == 8 && hw >= 16 * 512) split = 16;
   q.lanes = lanes; q.split = split;
+  q.fd_w = make_fastdiv((uint32_t)dp.W);
+  {
+    const int64_t per_thread = ((hw + split - 1) / split * lanes + kThreads - 1) / kThreads;
+    q.resident = per_thread <= 8 ? 8 : per_thread <= 16 ? 16 : 0;
+  }
   q.groups = (dp.C / 4 + lanes - 1) / lanes;
   const int64_t grid = ctas();
   if (grid >= (1ll << 31)) return refuse("too many planes");
