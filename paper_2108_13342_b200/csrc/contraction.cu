@@ -39,6 +39,12 @@ void mbconv_patch(Launch& L, const std::vector<void*>& ip, const std::vector<voi
 int mbconv_launch(const Launch& L, cudaStream_t st);
 int attention_launch(const Launch& L, void* status_words, int block_index, cudaStream_t st);
 size_t tf32_blob_bytes();
+size_t tf32s_blob_bytes();
+bool tf32s_gemm_eligible(const GemmParams& gp);
+int64_t tf32s_tiles(int64_t M, int64_t N, int64_t K);
+void tf32s_gemm_plan(Launch& L);
+bool tf32s_gemm_prepare(Launch& L, std::string& err);
+int tf32s_gemm_launch(const Launch& L, cudaStream_t st);
 bool tf32_gemm_eligible(const GemmParams& gp);
 void tf32_gemm_plan(Launch& L);
 bool tf32_gemm_prepare(Launch& L, std::string& err);
@@ -289,7 +295,7 @@ int lower_contraction(const Graph& g, const std::vector<int>& ops, uint32_t flag
 
   Launch& L = out.launch;
   L = Launch{};
-  L.blob.assign(sizeof(GemmParams) + sizeof(GemmTcParams) + std::max({tc2_blob_bytes(), tf32_blob_bytes(), tile_blob_bytes()}), 0);
+  L.blob.assign(sizeof(GemmParams) + sizeof(GemmTcParams) + std::max({tc2_blob_bytes(), tf32_blob_bytes(), tf32s_blob_bytes(), tile_blob_bytes()}), 0);
   GemmParams& gp = gp_of(L);
 
   // ---- operands ----------------------------------------------------------------
@@ -491,8 +497,14 @@ int lower_contraction(const Graph& g, const std::vector<int>& ops, uint32_t flag
   } else if (tc_gemm_eligible(gp)) {
     L.variant = 1;
     tc_gemm_plan(L);
-  } else if (conv_small_eligible(gp) && (gp.M <= small_m_limit() || !tf32_gemm_eligible(gp))) {
+  } else if (conv_small_eligible(gp) && (gp.M <= small_m_limit() || !(tf32_gemm_eligible(gp) || tf32s_gemm_eligible(gp)))) {
     conv_small_plan(L);
+  } else if (tf32s_gemm_eligible(gp) && (!tf32_gemm_eligible(gp) || tf32s_tiles(gp.M, gp.N, gp.K) <= 2 * sm_count() || dev_env("DNNF_TF32S_PREFER")) &&
+             !dev_env("DNNF_TF32S_NEVER")) {
+    // One wave of co-resident 128 x BN tiles finishes sooner than the persistent kernel with its resident B (rows x K x N, us:
+    // 3136 x 24 x 144 4.2 / 6.7, 12544 x 32 x 192 5.8 / 8.9, 25088 x 192 x 32 8.4 / 10.3, 32768 x 64 x 64 6.5 / 8.1); with more
+    // tiles the latter's set-up is paid back (25088 x 24 x 144 11.2 / 8.7, 100352 x 144 x 24 25.5 / 18.7).
+    tf32s_gemm_plan(L);
   } else if (tf32_gemm_eligible(gp)) {
     tf32_gemm_plan(L);
   } else if (A.kind == DNNF_OP_CONV1X1 && conv1x1_direct_eligible(gp)) {
@@ -517,14 +529,15 @@ void patch_contraction(Launch& L, const std::vector<void*>& ip, const std::vecto
   gp.A.ptr = ip[0]; gp.B.ptr = ip[1];
   for (int i = 0; i < gp.n_in; ++i) gp.in[i].ptr = ip[2 + i];
   for (int i = 0; i < gp.n_out; ++i) gp.out[i].ptr = op[i];
-  if (L.variant != 1 && L.variant != 3 && L.variant != 4 && L.variant != 5) return;
+  if (L.variant != 1 && L.variant != 3 && L.variant != 4 && L.variant != 5 && L.variant != 8) return;
   // The tensor maps embed addresses: encode them again whenever ANY pointer of the block differs from the
   // ones they were made for (an epilogue operand in any position may be read through a map).
   std::vector<void*> now(ip);
   now.insert(now.end(), op.begin(), op.end());
   if (L.tc_ready && now == L.encoded_ptrs) return;
   L.tc_ready = false;
-  bool ok = L.variant == 1 ? tc_gemm_prepare(L, err) : L.variant == 3 ? tc2_gemm_prepare(L, err) : L.variant == 5 ? tile_gemm_prepare(L, err) : tf32_gemm_prepare(L, err);
+  bool ok = L.variant == 1 ? tc_gemm_prepare(L, err) : L.variant == 3 ? tc2_gemm_prepare(L, err) : L.variant == 5 ? tile_gemm_prepare(L, err) :
+            L.variant == 8 ? tf32s_gemm_prepare(L, err) : tf32_gemm_prepare(L, err);
   if (ok) { L.tc_ready = true; L.encoded_ptrs = now; }
   else if (err.empty()) err = "cannot encode the tensor maps of a contraction block";
 }
@@ -538,7 +551,7 @@ int launch_contraction(const Launch& L, void* status_words, int block_index, cud
   if (L.family == DNNF_FAMILY_DWCONV) { int rc = dwconv_launch(L, status_words, block_index, st); if (rc) err = "depthwise convolution launch failed"; return rc; }
   if (L.variant == 2) { int rc = conv1x1_direct_launch(L, st); if (rc) err = "pointwise convolution launch failed"; return rc; }
   if (L.variant == 7) { int rc = conv_small_launch(L, st); if (rc) err = "pointwise convolution launch failed"; return rc; }
-  if ((L.variant == 1 || L.variant == 3 || L.variant == 4 || L.variant == 5) && !L.tc_ready) { err = "tensor maps of the block are not encoded"; return 1; }
+  if ((L.variant == 1 || L.variant == 3 || L.variant == 4 || L.variant == 5 || L.variant == 8) && !L.tc_ready) { err = "tensor maps of the block are not encoded"; return 1; }
   GemmParams gp = gp_of(L);
   gp.status = reinterpret_cast<int32_t*>(status_words);
   gp.block_index = block_index;
@@ -561,6 +574,13 @@ int launch_contraction(const Launch& L, void* status_words, int block_index, cud
     Launch& M = const_cast<Launch&>(L);
     gp_of(M).status = gp.status; gp_of(M).block_index = block_index;
     int rc = tf32_gemm_launch(L, st);
+    if (rc) err = "tensor-core fp32 GEMM launch failed";
+    return rc;
+  }
+  if (L.variant == 8) {
+    Launch& M = const_cast<Launch&>(L);
+    gp_of(M).status = gp.status; gp_of(M).block_index = block_index;
+    int rc = tf32s_gemm_launch(L, st);
     if (rc) err = "tensor-core fp32 GEMM launch failed";
     return rc;
   }

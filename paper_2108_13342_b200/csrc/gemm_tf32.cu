@@ -40,6 +40,7 @@
 #include "ir.h"
 #include "tc_common.cuh"
 #include "fp32_epilogues.h"
+#include "tf32_common.cuh"
 #include "tma_host.h"
 #include "warp_issue.cuh"
 
@@ -58,12 +59,10 @@ namespace tf32 {
 #define FACC(slot, v) do {} while (0)
 #endif
 
-constexpr int BM = 128, BK = 32, EPI_WARPS = 8, CONV_WARPS = 4, THREADS = 64 + 32 * (EPI_WARPS + CONV_WARPS);
+constexpr int EPI_WARPS = 8, CONV_WARPS = 4, THREADS = 64 + 32 * (EPI_WARPS + CONV_WARPS);
 constexpr int kSmemMax = 227 * 1024;
 constexpr int kMaxStages = 8;                               // raw row blocks in the ring
-constexpr int kAStageCols = 2 * BK;                         // TMEM columns of one A stage: hi, then lo
-constexpr int kChunkBytes = 32 * 128;                       // 32 rows x 32 fp32, swizzled
-constexpr int kMaxVec = 4, kVecFloats = 256 + 32;           // staged row-invariant operands
+constexpr int kVecFloats = 256 + 32;                        // per staged row-invariant operand
 constexpr int kMinEpiBytes = EPI_WARPS * 2 * kChunkBytes;   // >= EPI_WARPS * kStageWords * 4 (the general form's staging)
 constexpr int kFixedNoEpi = 1024 + 512 + kMaxVec * kVecFloats * 4;          // alignment slack, barriers, staged vectors
 // chunk buffers of the fast epilogue: one per 32-column chunk a warp handles in a tile, so that a tile's stores are
@@ -82,7 +81,8 @@ constexpr int kMaxBBytes = 88 * 1024;                       // hi + lo images of
 struct Params {
   CUtensorMap tmA, tmD;
   int32_t k_chunks;          // ceil(K / 32)
-  int32_t npad;              // N rounded up to 16
+  int32_t npad;              // N (of a part) rounded up to 16
+  int32_t part_n;            // columns of a part (N, or a multiple of 32); p.tiles_n parts
   int32_t total_tiles;
   int32_t stages;            // raw row blocks in the shared-memory ring
   int32_t epi_warps;         // 8 epilogue + 4 converter warps, or 4 + 8 when the tile is one 32-column chunk wide
@@ -121,41 +121,6 @@ __device__ __forceinline__ bool mbar_wait_poll(uint64_t* bar, uint32_t parity, v
 }
 #define mbar_wait mbar_wait_poll
 #endif
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, uint64_t* bar, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-               ::"r"(smem_u32(dst)), "l"(tm), "r"(smem_u32(bar)), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}"
-               ::"r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void mma_tf32_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t accumulate) {
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}"
-               ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
-               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
-                 "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
-                 "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]),
-                 "r"(r[30]), "r"(r[31]) : "memory");
-}
-__device__ __forceinline__ void tc_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ float to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, const void* src, int c0, int c1) {
-  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-               ::"l"(tm), "r"(smem_u32(src)), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void tma_store_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
-__device__ __forceinline__ void tma_store_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 // Fast epilogue IO: a lane owns 32 consecutive columns [c, c+32) of its own row.
 struct RowEpiIO {
   static constexpr int VV = 32;
@@ -166,7 +131,7 @@ struct RowEpiIO {
   const float* vec_s;        // staged row-invariant operands: [kMaxVec][kVecFloats]
   uint32_t row;              // global row of this lane
   bool row_ok;
-  int lane, c;
+  int lane, c, n;            // first column: inside the part, in the result
   __device__ __forceinline__ void load(int idx, float (&dst)[VV]) const {
     const int slot = q.slot[idx];
     if (slot >= 0) {           // every lane reads the same words: broadcast
@@ -179,11 +144,11 @@ struct RowEpiIO {
       return;
     }
     const TensorArg& a = p.in[idx];
-    const float* src = reinterpret_cast<const float*>(a.ptr) + a.base + (int64_t)row * a.stride[1] + c;
+    const float* src = reinterpret_cast<const float*>(a.ptr) + a.base + (int64_t)row * a.stride[1] + n;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (row_ok && c + 4 * j < p.N) w = __ldg(reinterpret_cast<const float4*>(src + 4 * j));
+      if (row_ok && n + 4 * j < p.N) w = __ldg(reinterpret_cast<const float4*>(src + 4 * j));
       dst[4 * j] = w.x; dst[4 * j + 1] = w.y; dst[4 * j + 2] = w.z; dst[4 * j + 3] = w.w;
     }
   }
@@ -298,6 +263,9 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   const int total_tiles = q.total_tiles;
+  // A result wider than the accumulators is cut into column parts; a CTA keeps one part's B images for all its tiles.
+  const int parts = p.tiles_n, part = (int)blockIdx.x % parts, first_tile = (int)blockIdx.x / parts, tile_step = (int)gridDim.x / parts;
+  const int n_base = part * q.part_n, n_here = min(q.part_n, p.N - n_base);
 
   if (warp == 0) {
     // ---------------- TMA producer: starts at once, while the other warps still prepare B ----------------
@@ -306,7 +274,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     // costs some 200 cycles of dependent instructions)
     int s = 0; uint32_t ph = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+    for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
       for (int u = 0; u < units; ++u) {
         { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph ^ 1, abort_flag))) { ok = false; break; } if (lane == 0) FACC(1, clock64() - t0); }
         if (elect_one()) {
@@ -346,7 +314,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
           int k, n;
           if (n_fast) { k = (int)fd_div((uint32_t)i, q.fd_npad); n = i - k * NP; } else { n = (int)fd_div((uint32_t)i, q.fd_kpad); k = i - n * kpad; }
           kk[u] = k; nn[u] = n;
-          x[u] = (i < total && k < p.K && n < p.N) ? __ldg(W + (int64_t)k * p.B.stride_row + (int64_t)n * p.B.stride_col) : 0.0f;
+          x[u] = (i < total && k < p.K && n < n_here) ? __ldg(W + (int64_t)k * p.B.stride_row + (int64_t)(n_base + n) * p.B.stride_col) : 0.0f;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) if (i0 + u * nthr < total) put_b(kk[u], nn[u], x[u]);
@@ -359,7 +327,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
         if (slot < 0 || (((p.static_mask >> (1 + idx)) & 1u) != 0) != want_static) continue;
         const TensorArg& a = p.in[idx];
         for (int n = tid; n < kVecFloats; n += nthr)
-          vec_s[slot * kVecFloats + n] = n < p.N ? load_scalar<false>(a, (uint32_t)a.base + (uint32_t)n * (uint32_t)a.stride[0]) : 0.0f;
+          vec_s[slot * kVecFloats + n] = n < n_here ? load_scalar<false>(a, (uint32_t)a.base + (uint32_t)(n_base + n) * (uint32_t)a.stride[0]) : 0.0f;
       }
     };
     // An external input is written by no kernel of the graph: reading it may overlap the previous kernel's tail.
@@ -397,7 +365,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     int s = 0; uint32_t ph = 0;
     bool ok = true;
     const uint64_t db0 = make_desc(b_base, 16, 1024);          // B_hi of K atom 0; + atom_bytes / 16 per atom, + lo_off / 16 for B_lo
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
+    for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++tcount) {
       const int acc = tcount & 1;
       const uint32_t aph = (tcount >> 1) & 1;
       { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag))) { ok = false; break; } if (lane == 0) FACC(2, clock64() - t0); }
@@ -450,7 +418,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     const int cstep = 8 * n_epi;              // 64 or 32 columns
     uint32_t tcount = 0, nstore = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x, ++tcount) {
+    for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++tcount) {
       const int acc = tcount & 1;
       const uint32_t aph = (tcount >> 1) & 1;
       { long long t0 = clock64(); if (!mbar_wait(&tfull_bar[acc], aph, abort_flag)) { ok = false; break; } if (warp == 2 && lane == 0) FACC(5, clock64() - t0); }
@@ -490,7 +458,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
           io8.chunk = my_chunks;
           run_program<8, SP, false>(p.prog, io8);
         } else
-        for (int c = cgroup * 32; c < p.N; c += cstep, ++slot) {
+        for (int c = cgroup * 32; c < n_here; c += cstep, ++slot) {
           uint32_t raw[32];
           const long long t0 = clock64();
           tc_ld32_issue(t_row + c, raw);
@@ -504,7 +472,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
             for (int j = 0; j < 32; ++j) io.accv[j] += __uint_as_float(raw[j]);
           }
           const long long t1 = clock64();
-          io.c = c;
+          io.c = c; io.n = n_base + c;
           io.chunk = my_chunks + slot * kChunkBytes;
           run_program<32, SP, false>(p.prog, io);
           if (warp == 2 && lane == 0) { FACC(12, t1 - t0); FACC(13, clock64() - t1); }
@@ -518,7 +486,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
         __syncwarp();
         if (lane == 0) {
           slot = 0;
-          for (int c = cgroup * 32; c < p.N; c += cstep, ++slot) tma_store_2d(&q.tmD, my_chunks + slot * kChunkBytes, c, tile * BM + sub * 32);
+          for (int c = cgroup * 32; c < n_here; c += cstep, ++slot) tma_store_2d(&q.tmD, my_chunks + slot * kChunkBytes, n_base + c, tile * BM + sub * 32);
           tma_store_commit();
         }
         (void)nstore;
@@ -539,7 +507,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
           io.row_out[k] = 0;
           if (k < p.n_out) io.row_out[k] = (uint32_t)p.out[k].base + tc_digits(p, p.out[k], p.n_nd, p.m_nd, mm);
         }
-        for (int c = cgroup * 32; c < p.N; c += cstep) {
+        for (int c = cgroup * 32; c < n_here; c += cstep) {
           uint32_t raw[32];
           tc_ld32_issue(t_row + c, raw);
           tc_ld_wait();
@@ -559,7 +527,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
 #pragma unroll
             for (int e = 0; e < 4; ++e) io.accv[i * 4 + e] = __uint_as_float(stage[((lane >> 3) + 4 * i) * 33 + (lane & 7) * 4 + e]);
           __syncwarp();
-          io.n0 = (uint32_t)c;
+          io.n0 = (uint32_t)(n_base + c);
           run_program<32, SP, false>(p.prog, io);
         }
       }
@@ -583,7 +551,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     // raw-block ring position of this warp's block (advances by `units` per tile) and A-stage ring position
     int s = unit % stages; uint32_t rph = (uint32_t)(unit / stages) & 1;
     int as = 0, turn = 0; uint32_t aph = 0;
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+    for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
       // (votes keep the warp together: the tensor-memory stores below are warp-wide)
       { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&raw_bar[s], rph, abort_flag))) { ok = false; break; } if (warp == 13 && lane == 0) FACC(7, clock64() - t0); }
       const float4* src = reinterpret_cast<const float4*>(ring + (size_t)s * q.unit_stride) + row * pieces;
@@ -667,8 +635,6 @@ size_t tf32_blob_bytes() { return sizeof(tf32::Params); }
 
 static int tf32_npad(int n) { return (n + 15) / 16 * 16; }
 static int tf32_b_bytes_of(int N, int K) { return 2 * tf32_npad(N) * 128 * ((K + tf32::BK - 1) / tf32::BK); }
-static int tf32_b_bytes(const GemmParams& gp) { return tf32_b_bytes_of(gp.N, gp.K); }
-
 // The part of the eligibility test that depends on the problem's shape alone (the planner asks it before it
 // splits a contraction that is too deep into several that fit).
 bool tf32_shape_fits(int64_t M, int64_t N, int64_t K) {
@@ -687,81 +653,76 @@ bool tf32_shape_fits(int64_t M, int64_t N, int64_t K) {
   return true;
 }
 
+// Columns of a part: the whole result, or the fewest equal parts of a multiple of 32 columns (a 32-column store must not reach
+// into the next part) that fit; 0 if none do.
+static int tf32_part(int64_t N, int64_t K) {
+  if (N <= 192) return (int)N;
+  for (int64_t parts = (N + 191) / 192; parts <= 16; ++parts) {
+    const int64_t part = ((N + parts - 1) / parts + 31) / 32 * 32;
+    if (part <= 192 && tf32_shape_fits(1 << 20, part, K)) return (int)part;
+  }
+  return 0;
+}
+// The same for a result that may be cut into column parts inside the kernel.
+bool tf32_parts_fit(int64_t M, int64_t N, int64_t K) {
+  if (plan_flag(DNNF_PLAN_SPLIT_ALWAYS)) return tf32_shape_fits(M, N, K);
+  const int part = tf32_part(N, K);
+  return part > 0 && tf32_shape_fits(M, part, K);
+}
+
 bool tf32_gemm_eligible(const GemmParams& gp) {
   if (gp.A.dtype != DNNF_F32 || gp.B.dtype != DNNF_F32) return false;
   if (gp.batch_ext[0] * gp.batch_ext[1] != 1) return false;
   if (gp.A.stride_col != 1 || gp.A.stride_row % 4 || gp.A.base % 4 || gp.A.stride_row <= 0) return false;
-  return tf32_shape_fits(gp.M, gp.N, gp.K);
-}
-
-// The fast epilogue form: one dense fp32 output [M x N] (unit stride along n, rows 16-byte aligned),
-// every epilogue input either row-invariant (staged in shared memory) or dense like the output.
-static bool fast_epilogue(const GemmParams& gp, int8_t* slot) {
-  if (gp.n_nd != 1 || gp.m_nd != 1 || gp.n_out != 1 || gp.N % 4) return false;
-  auto dense = [](const TensorArg& a) { return a.dtype == DNNF_F32 && a.stride[0] == 1 && a.stride[1] > 0 && a.stride[1] % 4 == 0 && a.base % 4 == 0; };
-  if (!dense(gp.out[0])) return false;
-  int nslot = 0;
-  for (int i = 0; i < gp.n_in; ++i) {
-    slot[i] = -1;
-    if (gp.in[i].mode == 1) { if (nslot == tf32::kMaxVec) return false; slot[i] = (int8_t)nslot++; }
-    else if (!dense(gp.in[i])) return false;
-  }
-  return true;
+  return tf32_parts_fit(gp.M, gp.N, gp.K);
 }
 
 void tf32_gemm_plan(Launch& L) {
   GemmParams& gp = gp_of(L);
   tf32::Params& q = fp_of(L);
   q.k_chunks = (gp.K + tf32::BK - 1) / tf32::BK;
-  q.npad = tf32_npad(gp.N);
+  q.part_n = tf32_part(gp.N, gp.K);
+  const int PN = q.part_n, parts = (gp.N + PN - 1) / PN;
+  q.npad = tf32_npad(PN);
   // tensor memory: two accumulator stages (twice as wide in the dual form) and at least two A stages must fit 512 columns
   q.dual = 4 * q.npad + 2 * tf32::kAStageCols <= 512 && !dev_env("DNNF_TF32_NO_DUAL");
-  q.fast_epi = fast_epilogue(gp, q.slot) && !dev_env("DNNF_TF32_GENERAL_EPILOGUE");
+  q.fast_epi = tf32::fast_epilogue(gp, q.slot) && !dev_env("DNNF_TF32_GENERAL_EPILOGUE");
   q.b_static = gp.static_mask & 1u;
   q.fd_n = make_fastdiv((uint32_t)gp.N); q.fd_npad = make_fastdiv((uint32_t)q.npad); q.fd_kpad = make_fastdiv((uint32_t)(q.k_chunks * tf32::BK));
-  q.epi_warps = (gp.N <= 32 && !dev_env("DNNF_TF32_EPI8")) ? 4 : 8;
+  q.epi_warps = (PN <= 32 && !dev_env("DNNF_TF32_EPI8")) ? 4 : 8;
   q.debug = dev_env("DNNF_TF32_DEBUG") ? atoi(dev_env("DNNF_TF32_DEBUG")) : 0;
   gp.tiles_m = (gp.M + tf32::BM - 1) / tf32::BM;
-  gp.tiles_n = 1;
+  gp.tiles_n = parts;
   q.total_tiles = gp.tiles_m;
-  L.grid = std::min(q.total_tiles, 148);
+  L.grid = std::min(q.total_tiles, std::max(1, sm_count() / parts)) * parts;
   L.threads = tf32::THREADS;
   // shared-memory row of a raw block: K rounded up to 4 floats plus padding that makes the pitch an odd
   // number of 16-byte pieces (conflict-free 128-bit reads down a column of rows)
   const int kr = (gp.K + 3) / 4 * 4;
   q.pitch = kr + ((kr / 4) % 2 == 0 ? 4 : 8);
-  q.epi_bytes = tf32::epi_bytes_for(gp.N, gp.K, q.fast_epi != 0);
-  { const int chunks = (gp.N + 31) / 32; q.chunks_per_warp = q.epi_warps == 4 ? chunks : (chunks + 1) / 2; }
+  q.epi_bytes = tf32::epi_bytes_for(PN, gp.K, q.fast_epi != 0);
+  { const int chunks = (PN + 31) / 32; q.chunks_per_warp = q.epi_warps == 4 ? chunks : (chunks + 1) / 2; }
   const int fixed = tf32::kFixedNoEpi + q.epi_bytes;
-  const int ring_budget = tf32::kSmemMax - fixed - tf32_b_bytes(gp);
+  const int ring_budget = tf32::kSmemMax - fixed - tf32_b_bytes_of(PN, gp.K);
   q.rb = 32;                                                 // one block per converter warp
   q.unit_stride = (q.rb * q.pitch * 4 + 1023) / 1024 * 1024;
   q.stages = std::min(tf32::kMaxStages, ring_budget / q.unit_stride);
   q.a_stages = std::min(6, (512 - 2 * (q.dual ? 2 : 1) * q.npad) / tf32::kAStageCols);
-  L.smem = (size_t)tf32_b_bytes(gp) + (size_t)q.stages * q.unit_stride + fixed;
-  q.b_dense = gp.B.stride_col == 1 && gp.B.stride_row == gp.N && gp.N % 4 == 0 && gp.B.base % 4 == 0 &&
+  L.smem = (size_t)tf32_b_bytes_of(PN, gp.K) + (size_t)q.stages * q.unit_stride + fixed;
+  q.b_dense = parts == 1 && gp.B.stride_col == 1 && gp.B.stride_row == gp.N && gp.N % 4 == 0 && gp.B.base % 4 == 0 &&
               (int64_t)gp.K * gp.N * 4 <= q.epi_bytes && !dev_env("DNNF_TF32_NO_BULK_B");
   L.variant = 4;
   L.static_id = StaticSet<tf32::Static>::find(gp.prog);
-}
-
-// fp32 [rows x cols] matrix, unit stride along cols, box = box_cols x box_rows
-static bool encode_f32(CUtensorMap* tm, float* base, int64_t cols, int64_t rows, int64_t row_stride, int box_cols, int box_rows,
-                       CUtensorMapSwizzle swizzle, std::string& err) {
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)row_stride * 4};
-  cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-  return tma_encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, swizzle, err);
 }
 
 bool tf32_gemm_prepare(Launch& L, std::string& err) {
   GemmParams& gp = gp_of(L);
   tf32::Params& q = fp_of(L);
   float* a = reinterpret_cast<float*>(gp.A.ptr) + gp.A.base;
-  if (!encode_f32(&q.tmA, a, gp.K, gp.M, gp.A.stride_row, q.pitch, q.rb, CU_TENSOR_MAP_SWIZZLE_NONE, err)) return false;
+  if (!tf32::encode_f32(&q.tmA, a, gp.K, gp.M, gp.A.stride_row, q.pitch, q.rb, CU_TENSOR_MAP_SWIZZLE_NONE, err)) return false;
   if (q.fast_epi) {
     float* d = reinterpret_cast<float*>(gp.out[0].ptr) + gp.out[0].base;
-    if (!encode_f32(&q.tmD, d, gp.N, gp.M, gp.out[0].stride[1], 32, 32, CU_TENSOR_MAP_SWIZZLE_128B, err)) return false;
+    if (!tf32::encode_f32(&q.tmD, d, gp.N, gp.M, gp.out[0].stride[1], 32, 32, CU_TENSOR_MAP_SWIZZLE_128B, err)) return false;
   }
   return true;
 }

@@ -353,6 +353,8 @@ double block_cost_us(const Graph& g, const Block& b) {
 }
 
 bool tf32_shape_fits(int64_t M, int64_t N, int64_t K);
+bool tf32s_shape_fits(int64_t M, int64_t N, int64_t K);
+bool tf32_parts_fit(int64_t M, int64_t N, int64_t K);
 bool conv_small_shape_fits(int64_t M, int64_t N, int64_t K);
 
 // Whether a split into parts x slices tensor-core kernels beats the kernel the contraction would otherwise run on.
@@ -389,8 +391,12 @@ static void split_deep_pointwise(Graph& g, const std::set<int>& decided) {
     const int64_t K = g.tensors[w].dims[0], N = g.tensors[w].dims[1], M = g.tensors[x].numel() / K;
     if (tf32_shape_fits(M, N, K)) continue;
     int s = 0;
-    for (int c : {2, 3, 4, 5, 6, 8}) if (K % (4 * c) == 0 && tf32_shape_fits(M, N, K / c)) { s = c; break; }
-    if (!s || (!decided.count((int)oi) && !split_pays(M, N, K, 1, s))) continue;      // parts of a column split were costed as a whole
+    // What the streaming kernel, or the resident one with its column parts, takes is never cut.  A wide result (N > 192) is
+    // recorded as ONE product over [pixels, K], the form its column blocks have where a split still applies; the rest stays
+    // the operator it is.
+    if (tf32s_shape_fits(M, N, K) || tf32_parts_fit(M, N, K)) { if (N <= 192 || g.ops[oi].kind == DNNF_OP_MATMUL) continue; s = 1; }
+    else for (int c : {2, 3, 4, 5, 6, 8}) if (K % (4 * c) == 0 && tf32_shape_fits(M, N, K / c)) { s = c; break; }
+    if (!s || (s > 1 && !decided.count((int)oi) && !split_pays(M, N, K, 1, s))) continue;      // parts of a column split were costed as a whole
     const int source = g.ops[oi].source_id;
     auto add = [&](int kind, std::vector<int> in, const Attrs& at, int reuse_out) -> int {
       Op o; o.id = (int)g.ops.size(); o.kind = kind; o.in = std::move(in); o.at = at; o.source_id = source;
@@ -421,14 +427,16 @@ static void split_deep_pointwise(Graph& g, const std::set<int>& decided) {
       ax.axis = 1; ax.start = i * ks; ax.end = (i + 1) * ks;
       aw.axis = 0; aw.start = i * ks; aw.end = (i + 1) * ks;
       int ws;
-      if (wcol >= 0) {                       // W is itself a column block of a wider matrix: rows first, then the columns
+      if (s == 1) {
+        ws = w;
+      } else if (wcol >= 0) {                       // W is itself a column block of a wider matrix: rows first, then the columns
         Attrs ac; ac.axis = 1; ac.start = wc0; ac.end = wc1;
         const int wr = add(DNNF_OP_SLICE, {wcol}, aw, -1);
         ws = wr < 0 ? -1 : add(DNNF_OP_SLICE, {wr}, ac, -1);
       } else {
         ws = add(DNNF_OP_SLICE, {w}, aw, -1);
       }
-      const int xs = add(DNNF_OP_SLICE, {x2}, ax, -1);
+      const int xs = s == 1 ? x2 : add(DNNF_OP_SLICE, {x2}, ax, -1);
       if (xs < 0 || ws < 0) { ok = false; break; }
       const int c = add(DNNF_OP_MATMUL, {xs, ws}, Attrs{}, -1);
       if (c < 0) { ok = false; break; }
@@ -461,7 +469,7 @@ static void split_wide_pointwise(Graph& g, std::set<int>& decided) {
     const int x = g.ops[oi].in[0], w = g.ops[oi].in[1], y = g.ops[oi].out[0];
     if (g.tensors[x].dtype != DNNF_F32 || g.tensors[w].dtype != DNNF_F32) continue;
     const int64_t K = g.tensors[w].dims[0], N = g.tensors[w].dims[1], M = g.tensors[x].numel() / K;
-    if (M < 512 || N % 4 || tf32_shape_fits(M, N, K)) continue;
+    if (M < 512 || N % 4 || tf32_shape_fits(M, N, K) || tf32s_shape_fits(M, N, K) || tf32_parts_fit(M, N, K)) continue;
     // the widest part (a multiple of 16 columns) that the kernel takes at this depth; every part reads x again, so
     // only splits into a few parts are worth it (deeper or wider problems stay with the FMA kernel)
     int64_t nw = 0, best = 1 << 30;

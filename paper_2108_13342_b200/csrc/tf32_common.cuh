@@ -1,0 +1,77 @@
+// Pieces shared by the two split-TF32 tensor-core kernels for fp32 contractions: PTX wrappers, tile constants, the test for
+// the fast epilogue form and the tensor-map encoding.
+#pragma once
+#include <cuda.h>
+#include <cuda_runtime.h>
+
+#include "gemm_params.h"
+#include "ir.h"
+#include "tc_common.cuh"
+#include "tma_host.h"
+
+namespace dnnf {
+namespace tf32 {
+
+constexpr int BM = 128, BK = 32;
+constexpr int kAStageCols = 2 * BK;                         // TMEM columns of one A stage: hi, then lo
+constexpr int kChunkBytes = 32 * 128;                       // 32 rows x 32 fp32, swizzled
+constexpr int kMaxVec = 4;                                  // staged row-invariant operands
+
+__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, uint64_t* bar, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
+               ::"r"(smem_u32(dst)), "l"(tm), "r"(smem_u32(bar)), "r"(c0), "r"(c1) : "memory");
+}
+__device__ __forceinline__ void mma_tf32_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t db, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}"
+               ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+                 "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
+                 "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]),
+                 "r"(r[30]), "r"(r[31]) : "memory");
+}
+__device__ __forceinline__ void tc_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ float to_tf32(float x) {
+  uint32_t r;
+  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+  return __uint_as_float(r);
+}
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, const void* src, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
+               ::"l"(tm), "r"(smem_u32(src)), "r"(c0), "r"(c1) : "memory");
+}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+
+// The fast epilogue form: one dense fp32 output [M x N] (unit stride along n, rows 16-byte aligned),
+// every epilogue input either row-invariant (staged in shared memory) or dense like the output.
+inline bool fast_epilogue(const GemmParams& gp, int8_t* slot) {
+  if (gp.n_nd != 1 || gp.m_nd != 1 || gp.n_out != 1 || gp.N % 4) return false;
+  auto dense = [](const TensorArg& a) { return a.dtype == DNNF_F32 && a.stride[0] == 1 && a.stride[1] > 0 && a.stride[1] % 4 == 0 && a.base % 4 == 0; };
+  if (!dense(gp.out[0])) return false;
+  int nslot = 0;
+  for (int i = 0; i < gp.n_in; ++i) {
+    slot[i] = -1;
+    if (gp.in[i].mode == 1) { if (nslot == kMaxVec) return false; slot[i] = (int8_t)nslot++; }
+    else if (!dense(gp.in[i])) return false;
+  }
+  return true;
+}
+
+// fp32 [rows x cols] matrix, unit stride along cols, box = box_cols x box_rows
+inline bool encode_f32(CUtensorMap* tm, float* base, int64_t cols, int64_t rows, int64_t row_stride, int box_cols, int box_rows,
+                       CUtensorMapSwizzle swizzle, std::string& err) {
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)row_stride * 4};
+  cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
+  return tma_encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, swizzle, err);
+}
+
+}  // namespace tf32
+}  // namespace dnnf

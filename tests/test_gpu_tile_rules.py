@@ -67,3 +67,71 @@ def test_rows_that_fit_no_vector(rows, cols, kind, dtype):
         y = g.add("Softmax", [g.add("MulC", ["X"], c=0.5) if kind == "softmax" else g.add("Sigmoid", ["X"])], axis=-1)
     g.mark_output(y)
     check(W.Workload(g, ins), RTOL_F32 if dtype == "f32" else RTOL_BF16_ROUNDING, expect_blocks=1)
+
+
+def conv1x1(m, k, n, tail):
+    g = graph()
+    g.ext("X", (1, 1, m, k)); g.ext("Wt", (k, n), kind="weight")
+    ins = {"X": rnd((1, 1, m, k), 920, -1, 1), "Wt": rnd((k, n), 921, -0.1, 0.1)}
+    y = g.add("Conv1x1", ["X", "Wt"])
+    if tail != "none":
+        g.ext("s", (n,), kind="weight"); g.ext("t", (n,)); ins.update(s=rnd((n,), 922, 0.5, 1.5), t=rnd((n,), 923, -0.5, 0.5))
+        y = g.add("ScaleShift", [y, "s", "t"], axis=-1)
+    if tail == "residual":
+        g.ext("R", (1, 1, m, n)); ins["R"] = rnd((1, 1, m, n), 924, -1, 1)
+        y = g.add("Add", [y, "R"])
+    if tail == "two_outputs":
+        g.mark_output(y); y = g.add("Sigmoid", [y])
+    g.mark_output(y)
+    return W.Workload(g, ins)
+
+
+@pytest.mark.parametrize("mkn", [(1025, 16, 8), (1280, 20, 12), (1300, 32, 16), (1100, 100, 32), (1500, 64, 48), (2000, 260, 64), (1111, 576, 100),
+                                 (3000, 192, 96), (6272, 96, 576), (1030, 1024, 20), (1154, 252, 196), (5000, 36, 200)])
+@pytest.mark.parametrize("tail", ["none", "bn", "residual", "two_outputs"])
+def test_streaming_fp32_contraction(mkn, tail):
+    """The K-streamed split-TF32 kernel: every tile width, with and without an accumulator of its own for the small products,
+    one or two CTAs per SM, ragged M, N and K, the transposing epilogue."""
+    m, k, n = mkn
+    # a sum of K / 8 additions, each cut by at most 2^-23 of the running sum: 1.5e-5 at K = 1024
+    s = check(conv1x1(m, k, n, tail), RTOL_F32 if k <= 512 else 2e-5, FUSED, expect_blocks=1)
+    assert s.g.blocks()[0]["variant"] == 8, s.g.blocks()
+
+
+@pytest.mark.parametrize("mkn", [(60000, 24, 200), (40000, 64, 512), (50001, 32, 388)])
+@pytest.mark.parametrize("tail", ["none", "bn", "residual", "two_outputs"])
+def test_resident_fp32_contraction_in_column_parts(mkn, tail):
+    """The persistent split-TF32 kernel with a result wider than its accumulators: two to four column parts per launch, the last
+    one narrower."""
+    m, k, n = mkn
+    s = check(conv1x1(m, k, n, tail), RTOL_F32, FUSED, expect_blocks=1)
+    assert s.g.blocks()[0]["variant"] == 4, s.g.blocks()
+
+
+@pytest.mark.parametrize("nhwc", [(1, 1, 1, 4), (2, 3, 5, 12), (3, 17, 19, 20), (1, 64, 64, 4), (1, 100, 91, 8), (2, 90, 97, 12), (8, 40, 40, 64),
+                                  (1, 128, 130, 16), (2, 256, 255, 8)])
+@pytest.mark.parametrize("tail", ["none", "residual", "interpreted"])
+def test_instance_normalisation_splits(nhwc, tail):
+    """Planes kept in registers (8 or 16 pixels per thread) and streamed ones, clusters of 1 to 16 CTAs with ragged parts, a mean
+    far from zero (no cancellation: the deviations are taken from local means)."""
+    n, h, w, c = nhwc
+    g = graph()
+    g.ext("X", nhwc); g.ext("s", (c,)); g.ext("t", (c,))
+    ins = {"X": rnd(nhwc, 930, 9.0, 11.0), "s": rnd((c,), 931, 0.5, 1.5), "t": rnd((c,), 932, -0.5, 0.5)}
+    y = g.add("InstanceNorm", ["X", "s", "t"], eps=1e-5)
+    if tail == "residual":
+        g.ext("R", nhwc); ins["R"] = rnd(nhwc, 933, -1, 1)
+        y = g.add("Add", [y, "R"])
+    elif tail == "interpreted":
+        y = g.add("Tanh", [g.add("MulC", [y], c=0.5)])
+    g.mark_output(y)
+    # x - mean loses 2^-24 * 10 / std(x) = 1.03e-6 relative to the deviations' size; the rest as in the other fp32 chains
+    check(W.Workload(g, ins), 2e-5, FUSED, expect_blocks=1)
+
+
+@pytest.mark.parametrize("seq", [136, 200, 248, 256])
+def test_attention_with_many_keys(seq):
+    """Single-kernel attention whose mask tile shares the probabilities' shared memory."""
+    from paper_2108_13342_b200.workloads import encoder
+    from util import check_blocks
+    check_blocks(encoder(layers=1, batch=2, seq=seq, hidden=128, heads=2, ffn=128), B.PLAN_BEYOND_TABLE3, B.REWRITE_CANON_MACRO, min_checked=1)
