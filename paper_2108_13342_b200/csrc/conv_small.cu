@@ -7,7 +7,7 @@
 // a lane reads the eight weight values of its B fragments straight from global memory (L2 serves the re-reads of the
 // other row tiles), splits them on the fly, and reads its rows of A with 128-bit loads.  Split TF32 on mma.sync m16n8k8,
 // three products per step (lo*hi + hi*lo + hi*hi, fp32 accumulate), the same k order inside an instruction as in the
-// single-kernel inverted-residual block.  The block's chain runs on the summed fragments in warp 0.
+// single-kernel inverted-residual block.  Warp j sums n-tile j and runs the block's chain on it.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -76,11 +76,17 @@ struct SmallIO {
 
 __device__ __noinline__ void run_interpreted(const Program& prog, SmallIO& io) { run_program<4, DynProg>(prog, io); }
 
-// K is a multiple of 8; N is even (the last column group of a row tile may hold fewer than 4 n-tiles, the last n-tile
+// Brings the line of p into L1 while something else is waited for; the value is not used.
+__device__ __forceinline__ void touch(const float* p) {
+  [[maybe_unused]] float x;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(x) : "l"(p));
+}
+
+// K is a multiple of 8; N is even (the last column group of a row tile may hold fewer than NT n-tiles, the last n-tile
 // fewer than 8 columns).
 template <int NT, class SP>
 __global__ void __launch_bounds__(THREADS) conv_small_kernel(const __grid_constant__ GemmParams p) {
-  __shared__ float part[WARPS - 1][NT * 4][32];
+  __shared__ float part[WARPS][NT * 4][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   const int n_groups = (p.N + 8 * NT - 1) / (8 * NT);
   const int mt = blockIdx.x / n_groups, ng = blockIdx.x - mt * n_groups;
@@ -88,8 +94,6 @@ __global__ void __launch_bounds__(THREADS) conv_small_kernel(const __grid_consta
   const bool ok0 = r0 < p.M, ok1 = r1 < p.M;
   const int n0 = ng * 8 * NT;
   const int nt_here = min(NT, (p.N - n0 + 7) >> 3);              // the last n-tile of a row may be narrower than 8 columns
-  pdl_launch_dependents();
-  pdl_wait();
   const float* X = reinterpret_cast<const float*>(p.A.ptr) + p.A.base;
   const float* W = reinterpret_cast<const float*>(p.B.ptr) + p.B.base;
   const float* x0 = X + (int64_t)(ok0 ? r0 : 0) * p.A.stride_row;
@@ -101,14 +105,8 @@ __global__ void __launch_bounds__(THREADS) conv_small_kernel(const __grid_consta
 #pragma unroll
   for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
   const float4 z4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  // the loads of block b + 1 are issued before the instructions of block b (the loop is a chain of global-memory
-  // latencies otherwise)
-  float4 u = z4, w = z4, un = z4, wn = z4;
-  float wv[NT][4], wvn[NT][4];
-  auto fetch = [&](int b, float4& fu, float4& fw, float (&fv)[NT][4]) {
+  auto fetch_w = [&](int b, float (&fv)[NT][4]) {
     const int kb = 16 * b + 4 * t;                                // this lane's four consecutive k
-    fu = ok0 ? __ldg(reinterpret_cast<const float4*>(x0 + kb)) : z4;
-    fw = ok1 ? __ldg(reinterpret_cast<const float4*>(x1 + kb)) : z4;
     // weights W[kb + {0, 1, 2, 3}][n0 + 8 j + g]: the B fragments of two steps
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
@@ -118,9 +116,12 @@ __global__ void __launch_bounds__(THREADS) conv_small_kernel(const __grid_consta
       for (int e = 0; e < 4; ++e) fv[j][e] = in ? __ldg(wp + (size_t)e * p.N) : 0.0f;
     }
   };
-  if (b_begin < b_end) fetch(b_begin, u, w, wv);
-  for (int b = b_begin; b < b_end; ++b) {
-    if (b + 1 < b_end) fetch(b + 1, un, wn, wvn);
+  auto fetch_x = [&](int b, float4& fu, float4& fw) {
+    const int kb = 16 * b + 4 * t;
+    fu = ok0 ? __ldg(reinterpret_cast<const float4*>(x0 + kb)) : z4;
+    fw = ok1 ? __ldg(reinterpret_cast<const float4*>(x1 + kb)) : z4;
+  };
+  auto step = [&](const float4& u, const float4& w, const float (&wv)[NT][4]) {
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
       uint32_t h0, h1, h2, h3, l0, l1, l2, l3;
@@ -137,11 +138,40 @@ __global__ void __launch_bounds__(THREADS) conv_small_kernel(const __grid_consta
 #pragma unroll
       for (int j = 0; j < NT; ++j) mma_tf32(acc[j], h0, h1, h2, h3, bh0[j], bh1[j]);
     }
-    u = un; w = wn;
-#pragma unroll
-    for (int j = 0; j < NT; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) wv[j][e] = wvn[j][e];
+  };
+  pdl_launch_dependents();
+  // A weight is written by no kernel of the graph: the first two blocks of it, and the lines of the chain's per-channel
+  // operands, are requested before the wait on the previous kernel.
+  const bool w_static = (p.static_mask & 1u) != 0;
+  float4 u0 = z4, v0 = z4, u1 = z4, v1 = z4;
+  float wv0[NT][4], wv1[NT][4];
+  auto first_weights = [&]() {
+    if (b_begin < b_end) fetch_w(b_begin, wv0);
+    if (b_begin + 1 < b_end) fetch_w(b_begin + 1, wv1);
+  };
+  const bool finisher = warp < nt_here;                           // warp j finishes n-tile j
+  if (w_static) first_weights();
+  if (finisher)
+    for (int i = 0; i < p.n_in; ++i)
+      if (((p.static_mask >> (1 + i)) & 1u) && p.in[i].stride[1] == 0)
+        touch(reinterpret_cast<const float*>(p.in[i].ptr) + p.in[i].base + (int64_t)(n0 + 8 * warp) * p.in[i].stride[0]);
+  pdl_wait();
+  if (!w_static) first_weights();
+  if (b_begin < b_end) fetch_x(b_begin, u0, v0);
+  if (b_begin + 1 < b_end) fetch_x(b_begin + 1, u1, v1);
+  if (finisher)                                                   // the rows of a full-size operand (a residual), 32 bytes each
+    for (int i = 0; i < p.n_in; ++i)
+      if (p.in[i].stride[1] != 0 && lane < 16 && mt * 16 + lane < p.M)
+        touch(reinterpret_cast<const float*>(p.in[i].ptr) + p.in[i].base + (int64_t)(mt * 16 + lane) * p.in[i].stride[1] + (int64_t)(n0 + 8 * warp) * p.in[i].stride[0]);
+  // the loads of the next two blocks are in flight while a block's instructions run (the loop is a chain of
+  // global-memory latencies otherwise)
+  for (int b = b_begin; b < b_end; b += 2) {
+    step(u0, v0, wv0);
+    if (b + 2 < b_end) { fetch_w(b + 2, wv0); fetch_x(b + 2, u0, v0); }
+    if (b + 1 < b_end) {
+      step(u1, v1, wv1);
+      if (b + 3 < b_end) { fetch_w(b + 3, wv1); fetch_x(b + 3, u1, v1); }
+    }
   }
   if ((p.K & 8) && warp == WARPS - 1) {                           // a K that is 8 mod 16 ends with one step on k = 16 blocks + 2 t + {0, 1}
     const int kb = 16 * blocks + 2 * t;
@@ -161,32 +191,26 @@ __global__ void __launch_bounds__(THREADS) conv_small_kernel(const __grid_consta
       mma_tf32(acc[j], h0, h1, h2, h3, bh0, bh1);
     }
   }
-  if (warp > 0) {
 #pragma unroll
-    for (int j = 0; j < NT; ++j)
+  for (int j = 0; j < NT; ++j)
 #pragma unroll
-      for (int v = 0; v < 4; ++v) part[warp - 1][j * 4 + v][lane] = acc[j][v];
-  }
+    for (int v = 0; v < 4; ++v) part[warp][j * 4 + v][lane] = acc[j][v];
   __syncthreads();
-  if (warp != 0) return;
+  if (!finisher) return;
   SmallIO io{p};
   io.pix0 = (uint32_t)(ok0 ? r0 : 0); io.pix1 = (uint32_t)(ok1 ? r1 : 0);
   io.ok0 = ok0; io.ok1 = ok1;
+  io.okc = n0 + 8 * warp + 2 * t < p.N;                           // N is even: a pair of columns is inside or outside together
+  io.col = (uint32_t)(io.okc ? n0 + 8 * warp + 2 * t : 0);
 #pragma unroll
-  for (int j = 0; j < NT; ++j) {
-    io.okc = j < nt_here && n0 + 8 * j + 2 * t < p.N;           // N is even: a pair of columns is inside or outside together
-    io.col = (uint32_t)(io.okc ? n0 + 8 * j + 2 * t : 0);
+  for (int v = 0; v < 4; ++v) {
+    float sum = part[0][warp * 4 + v][lane];
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      float sum = acc[j][v];
-#pragma unroll
-      for (int r = 0; r < WARPS - 1; ++r) sum += part[r][j * 4 + v][lane];
-      io.accv[v] = sum;
-    }
-    if (j >= nt_here) continue;
-    if constexpr (SP::n == 0) run_interpreted(p.prog, io);
-    else run_program<4, SP>(p.prog, io);
+    for (int r = 1; r < WARPS; ++r) sum += part[r][warp * 4 + v][lane];
+    io.accv[v] = sum;
   }
+  if constexpr (SP::n == 0) run_interpreted(p.prog, io);
+  else run_program<4, SP>(p.prog, io);
 }
 
 }  // namespace pws
