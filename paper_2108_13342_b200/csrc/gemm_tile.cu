@@ -11,11 +11,13 @@
 //   * the B operand of a block is normally a weight, which no kernel of the graph writes: its
 //     first ring stages are requested BEFORE the wait on the previous kernel, as are the bias
 //     vectors; only the loads of A (and of a residual tile) wait;
-//   * the chunk buffers of the epilogue reuse the operand ring, which is idle by then, unless a
-//     residual tile has to be prefetched into them while the main loop runs.
-// Roles: warps 0, 1 TMA producers (one lane each; producer j loads the k-tiles j, j+2, ...), warp 2 tensor-memory
-// allocation and MMA issue (one lane), warps 3..6 epilogue: tcgen05.ld -> micro-op program -> bf16 ->
-// swizzled 32 x 64 chunk -> TMA store.
+//   * the chunk buffers of the epilogue reuse the operand ring, which is idle by then; a residual is read straight into
+//     registers, the first chunk's values before the accumulator is waited for.
+// Roles: warps 0, 1 TMA producers (producer j loads the k-tiles j, j+2, ...), warp 2 tensor-memory allocation and MMA
+// issue, warps 3..10 epilogue (two warps per 32 rows, half of the tile's columns each): tcgen05.ld -> micro-op program on 16
+// columns at a time -> bf16 -> swizzled 32 x 32 chunk -> TMA store.With four warps and 32 columns at a time the epilogue
+// was the longer half of these kernels: 248 x 2304 x 768 + bias 6.1 -> 5.4 us, 248 x 768 x 768 5.5 -> 4.8, 248 x 3072 x 768 +
+// GELU 6.8 -> 6.0, 1024 x 768 x 768 6.0 -> 5.4.
 // Every wait is bounded; on expiry the CTA records DNNF_ERR_TIMEOUT and releases tensor memory.
 //
 // Every TMA load in this file is a plain per-CTA load; no clusters are used.
@@ -36,17 +38,17 @@ namespace tile {
 
 using namespace tc2;
 
-constexpr int kEpiWarps = 4, kThreads = 96 + 32 * kEpiWarps;         // 2 producer warps, 1 issuer warp, 4 epilogue warps
+constexpr int kEpiWarps = 8, kThreads = 96 + 32 * kEpiWarps;         // 2 producer warps, 1 issuer warp, 8 epilogue warps
+constexpr int kChunkB = 32 * 64;                                     // 32 rows x 32 bf16, 64-byte swizzle
 constexpr int kVecBytes = kEpiWarps * kMaxVec * kBiasFloats * 4;     // staged row-invariant operands, per warp
 constexpr int kBarBytes = 256;
 constexpr int kSmemTwoPerSm = 112 * 1024;                            // two CTAs of this size fit one SM
 
 struct Params {
-  CUtensorMap tmA, tmB, tmD, tmC;
+  CUtensorMap tmA, tmB, tmD;
   int32_t b_kmajor, k_tiles, bn, tiles_n;
-  int32_t c_input;           // index of the epilogue input that is a full tile (TMA-loaded), or -1
+  int32_t c_input;           // index of the epilogue input that is a full tile, or -1
   int32_t stages;
-  int32_t cbuf_off;          // chunk buffers, bytes from the ring's start: 0 (they reuse the ring) or behind the ring
   int32_t tail_off;          // staged vectors, then barriers
   int32_t b_static;          // B is never written by a kernel of the graph
   int32_t tmem_cols;
@@ -84,37 +86,49 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
 }
 
-// Epilogue IO of the split-K form: a thread owns 32 consecutive columns of its row of the CTA's column slice, reads a
-// full-tile operand (a residual) and writes the result straight from / to global memory with 16-byte accesses.
-struct SliceIO {
-  static constexpr int VV = 32;
+__device__ __forceinline__ void unpack_bf16(const uint4& w, float* d) {
+  d[0] = __uint_as_float(w.x << 16); d[1] = __uint_as_float(w.x & 0xffff0000u);
+  d[2] = __uint_as_float(w.y << 16); d[3] = __uint_as_float(w.y & 0xffff0000u);
+  d[4] = __uint_as_float(w.z << 16); d[5] = __uint_as_float(w.z & 0xffff0000u);
+  d[6] = __uint_as_float(w.w << 16); d[7] = __uint_as_float(w.w & 0xffff0000u);
+}
+__device__ __forceinline__ uint4 pack_bf16(const float* v) {
+  __nv_bfloat162 a0 = __floats2bfloat162_rn(v[0], v[1]), a1 = __floats2bfloat162_rn(v[2], v[3]);
+  __nv_bfloat162 a2 = __floats2bfloat162_rn(v[4], v[5]), a3 = __floats2bfloat162_rn(v[6], v[7]);
+  return make_uint4(*reinterpret_cast<uint32_t*>(&a0), *reinterpret_cast<uint32_t*>(&a1), *reinterpret_cast<uint32_t*>(&a2),
+                    *reinterpret_cast<uint32_t*>(&a3));
+}
+// 16 tensor-memory columns of this thread's lane.  The wait names the registers so that no use moves in front of it.
+__device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                 "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]),
+                 "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]) :: "memory");
+}
+
+// Epilogue IO: a thread owns 16 consecutive columns of its own row (TMEM layout: lane = row).  kDirect (the split-K form): the
+// result goes straight to global memory with 16-byte accesses; else into a swizzled 32 x 32 chunk buffer, where the 16-byte
+// piece j of row r sits at r * 64 + ((j ^ ((r >> 1) & 3)) * 16).
+template <bool kDirect>
+struct TileIO {
+  static constexpr int VV = 16;
   const GemmParams& p;
-  float accv[32];
+  float accv[16];
+  uint4 res[2];              // the full-tile operand's 16 values of this row
   const float* vec_s;        // staged row-invariant operands of this warp: [kMaxVec][kBiasFloats], indexed by tile column
-  int c_input;
-  int col;                   // first tile column of the 32
+  uint8_t* chunk;            // chunk buffer of this warp
+  int c_input, col;          // first tile column of the 16
   int n;                     // its global column
-  uint32_t res_off, out_off; // element offsets of (row, column 0) in the residual and in the result
+  int lane, h;               // half of the chunk
+  uint32_t out_off;          // element offset of (row, column 0) in the result
   bool row_ok;
   __device__ __forceinline__ void load(int idx, float (&dst)[VV]) const {
-    const TensorArg& a = p.in[idx];
-    if (idx == c_input) {
-      const __nv_bfloat16* src = reinterpret_cast<const __nv_bfloat16*>(a.ptr) + res_off + n;
+    if (idx == c_input) { unpack_bf16(res[0], dst); unpack_bf16(res[1], dst + 8); return; }
+    const float* s = vec_s + p.in[idx].mode * kBiasFloats + col;     // every lane reads the same words: broadcast
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (row_ok && n + 8 * j < p.N) w = __ldg(reinterpret_cast<const uint4*>(src + 8 * j));
-        float* d = &dst[8 * j];
-        d[0] = __uint_as_float(w.x << 16); d[1] = __uint_as_float(w.x & 0xffff0000u);
-        d[2] = __uint_as_float(w.y << 16); d[3] = __uint_as_float(w.y & 0xffff0000u);
-        d[4] = __uint_as_float(w.z << 16); d[5] = __uint_as_float(w.z & 0xffff0000u);
-        d[6] = __uint_as_float(w.w << 16); d[7] = __uint_as_float(w.w & 0xffff0000u);
-      }
-      return;
-    }
-    const float* s = vec_s + a.mode * kBiasFloats + col;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < 4; ++j) {
       float4 w = *reinterpret_cast<const float4*>(s + 4 * j);
       dst[4 * j] = w.x; dst[4 * j + 1] = w.y; dst[4 * j + 2] = w.z; dst[4 * j + 3] = w.w;
     }
@@ -124,14 +138,14 @@ struct SliceIO {
     for (int v = 0; v < VV; ++v) dst[v] = accv[v];
   }
   __device__ __forceinline__ void store(int, const float (&val)[VV]) const {
-    __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.out[0].ptr) + out_off + n;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      __nv_bfloat162 a0 = __floats2bfloat162_rn(val[8 * j], val[8 * j + 1]), a1 = __floats2bfloat162_rn(val[8 * j + 2], val[8 * j + 3]);
-      __nv_bfloat162 a2 = __floats2bfloat162_rn(val[8 * j + 4], val[8 * j + 5]), a3 = __floats2bfloat162_rn(val[8 * j + 6], val[8 * j + 7]);
-      if (row_ok && n + 8 * j < p.N)
-        *reinterpret_cast<uint4*>(dst + 8 * j) = make_uint4(*reinterpret_cast<uint32_t*>(&a0), *reinterpret_cast<uint32_t*>(&a1),
-                                                            *reinterpret_cast<uint32_t*>(&a2), *reinterpret_cast<uint32_t*>(&a3));
+    for (int j = 0; j < 2; ++j) {
+      const uint4 w = pack_bf16(&val[8 * j]);
+      if (kDirect) {
+        if (row_ok && n + 8 * j < p.N) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out[0].ptr) + out_off + n + 8 * j) = w;
+      } else {
+        *reinterpret_cast<uint4*>(chunk + lane * 64 + (((2 * h + j) ^ ((lane >> 1) & 3)) << 4)) = w;
+      }
     }
   }
   __device__ __forceinline__ void row_reduce(int, float (&)[VV]) const {}
@@ -164,8 +178,7 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(tail + kVecBytes);   // [stages] bytes of one stage
   uint64_t* empty_bar = full_bar + 8;         // [stages] 1 arrival (commit)
   uint64_t* tfull_bar = empty_bar + 8;        // accumulator complete
-  uint64_t* c_bar = tfull_bar + 1;            // [kEpiWarps] residual chunks landed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(c_bar + kEpiWarps);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
@@ -174,7 +187,6 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     mbar_init(tfull_bar, 1);
-    for (int s = 0; s < kEpiWarps; ++s) mbar_init(&c_bar[s], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -183,7 +195,6 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   } else if (warp == 0 && lane == 0) {
     prefetch_tmap(&q.tmA); prefetch_tmap(&q.tmB); prefetch_tmap(&q.tmD);
-    if (q.c_input >= 0) prefetch_tmap(&q.tmC);
   }
   tc_fence_before();
   __syncthreads();
@@ -267,12 +278,12 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     }
     if (kSplit) { __syncwarp(); cluster_sync(); cluster_sync(); }
   } else {
-    // ---------------- epilogue warps 3..6: a warp may read the tensor-memory lanes 32 (warp % 4) .. + 31 ----------------
-    const int ew = warp - 3, sub = warp & 3;
-    const int chunks = BN / 64;
-    uint8_t* cbuf = smem + q.cbuf_off + (size_t)ew * chunks * kChunkBytes;
+    // ---------------- epilogue warps 3..10: a warp may read the tensor-memory lanes 32 (warp % 4) .. + 31 ----------------
+    const int ew = warp - 3, sub = warp & 3, half = ew >> 2;
+    const int half_cols = BN >> 1;
+    uint8_t* cbuf = smem + (size_t)ew * (half_cols >> 5) * kChunkB;      // (the operand ring is idle by then)
     float* vec_s = reinterpret_cast<float*>(tail) + ew * (kMaxVec * kBiasFloats);
-    const int mw0 = m0 + sub * 32;
+    const int m = m0 + sub * 32 + lane;
     auto stage_vectors = [&](bool want_static) {
       for (int k = 0; k < p.n_in; ++k) {
         const TensorArg& a = p.in[k];
@@ -283,19 +294,28 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
         }
       }
     };
+    const bool row_ok = m < p.M;
+    const uint32_t mm = row_ok ? (uint32_t)m : 0u;
+    const __nv_bfloat16* rsrc = q.c_input >= 0 ? reinterpret_cast<const __nv_bfloat16*>(p.in[q.c_input].ptr) + p.in[q.c_input].base +
+                                                     (int64_t)mm * p.in[q.c_input].stride[1] : nullptr;
+    auto fetch_residual = [&](int n, uint4 (&r)[4]) {              // 32 columns of this lane's row
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        r[j] = make_uint4(0u, 0u, 0u, 0u);
+        if (row_ok && n + 8 * j < p.N) r[j] = __ldg(reinterpret_cast<const uint4*>(rsrc + n + 8 * j));
+      }
+    };
     stage_vectors(true);
     pdl_wait();
-    if (!kSplit && q.c_input >= 0 && lane == 0) {                 // the residual tile of this warp: all chunks at once
-      mbar_expect_tx(&c_bar[ew], (uint32_t)(chunks * kChunkBytes));
-      for (int c = 0; c < chunks; ++c) tma_load_2d(cbuf + c * kChunkBytes, &q.tmC, &c_bar[ew], n0 + c * 64, mw0);
-    }
     stage_vectors(false);
+    uint4 res[4];
+    if (!kSplit && q.c_input >= 0) fetch_residual(n0 + half * half_cols, res);
     __syncwarp();
-    bool ok = mbar_wait_cta(tfull_bar, 0, abort_flag);
-    if (!kSplit && ok && q.c_input >= 0) ok = mbar_wait_cta(&c_bar[ew], 0, abort_flag);
-    ok = __all_sync(0xffffffffu, ok);        // the tensor-memory loads below are warp-wide
+    bool ok = __all_sync(0xffffffffu, mbar_wait_cta(tfull_bar, 0, abort_flag));
     if (ew == 0 && lane == 0) TSTAMP(5);
     const uint32_t t_row = tmem_base + ((uint32_t)(sub * 32) << 16);
+    TileIO<kSplit> io{p};
+    io.lane = lane; io.c_input = q.c_input; io.vec_s = vec_s; io.row_ok = row_ok;
     if (kSplit) {
       const int slice = BN / S;                                    // 64 or 32 columns per owner
       const int pieces = slice >> 2;                               // 16-byte pieces of a row of a slice
@@ -304,17 +324,17 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
       cluster_sync();                                              // every CTA of the cluster is through its main loop
       if (ew == 0 && lane == 0) TSTAMP(6);
       if (ok) {
-        // hand the partial sums of the other CTAs' slices over: receive buffer [sender][piece][row] of float4
+        // hand the partial sums of the other CTAs' slices over: receive buffer [sender][piece][row] of float4; the two
+        // warps of a row group take alternate groups of 16 columns
         for (int j = 0; j < S; ++j) {
           if (j == rank) continue;
           const int slot = rank < j ? rank : rank - 1;
           const uint32_t remote = mapa(smem_u32(smem), (uint32_t)j) + (uint32_t)((slot * pieces) * BM + row) * 16u;
-          for (int c = 0; c < slice; c += 32) {
-            uint32_t raw[32];
-            tc_ld32(t_row + j * slice + c, raw);
-            tc_ld_wait();
+          for (int c = half * 16; c < slice; c += 32) {
+            uint32_t raw[16];
+            ld16(t_row + j * slice + c, raw);
 #pragma unroll
-            for (int v = 0; v < 8; ++v)
+            for (int v = 0; v < 4; ++v)
               st_cluster_f4(remote + (uint32_t)(((c >> 2) + v) * BM) * 16u,
                             make_float4(__uint_as_float(raw[4 * v]), __uint_as_float(raw[4 * v + 1]), __uint_as_float(raw[4 * v + 2]), __uint_as_float(raw[4 * v + 3])));
           }
@@ -324,56 +344,56 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
       cluster_sync();                                              // all partial sums have arrived
       if (ew == 0 && lane == 0) TSTAMP(8);
       if (ok) {
-        SliceIO io{p};
-        io.vec_s = vec_s; io.c_input = q.c_input;
-        const int m = mw0 + lane;
-        io.row_ok = m < p.M;
-        const uint32_t mm = io.row_ok ? (uint32_t)m : 0u;
         io.out_off = (uint32_t)p.out[0].base + mm * (uint32_t)p.out[0].stride[1];
-        io.res_off = q.c_input >= 0 ? (uint32_t)p.in[q.c_input].base + mm * (uint32_t)p.in[q.c_input].stride[1] : 0u;
         const float4* rcv = reinterpret_cast<const float4*>(smem);
-        for (int c = 0; c < slice; c += 32) {
-          uint32_t raw[32];
-          tc_ld32(t_row + rank * slice + c, raw);
-          tc_ld_wait();
+        for (int c = half * 16; c < slice; c += 32) {
+          io.col = rank * slice + c;
+          io.n = n0 + io.col;
+          if (q.c_input >= 0) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) io.accv[i] = __uint_as_float(raw[i]);
+            for (int j = 0; j < 2; ++j) {
+              io.res[j] = make_uint4(0u, 0u, 0u, 0u);
+              if (row_ok && io.n + 8 * j < p.N) io.res[j] = __ldg(reinterpret_cast<const uint4*>(rsrc + io.n + 8 * j));
+            }
+          }
+          uint32_t raw[16];
+          ld16(t_row + io.col, raw);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) io.accv[i] = __uint_as_float(raw[i]);
           for (int sl = 0; sl < S - 1; ++sl) {
 #pragma unroll
-            for (int v = 0; v < 8; ++v) {
+            for (int v = 0; v < 4; ++v) {
               const float4 w = rcv[(sl * pieces + (c >> 2) + v) * BM + row];
               io.accv[4 * v] += w.x; io.accv[4 * v + 1] += w.y; io.accv[4 * v + 2] += w.z; io.accv[4 * v + 3] += w.w;
             }
           }
-          io.col = rank * slice + c;
-          io.n = n0 + io.col;
-          run_program<32, SP, true>(p.prog, io);
+          run_program<16, SP, true>(p.prog, io);
         }
       }
       if (ew == 0 && lane == 0) TSTAMP(9);
     } else if (ok) {
-      EpiIO io{p};
-      io.lane = lane; io.c_input = q.c_input; io.vec_s = vec_s;
       tc_fence_after();
-      for (int c = 0; c < chunks; ++c) {
-        io.chunk = cbuf + c * kChunkBytes;
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          uint32_t raw[32];
-          tc_ld32(t_row + c * 64 + h * 32, raw);
-          tc_ld_wait();
+      for (int c = 0; c < half_cols; c += 32) {
+        const int col = half * half_cols + c;
+        if (n0 + col >= p.N) break;                                // (uniform over the warp)
+        io.chunk = cbuf + (c >> 5) * kChunkB;
 #pragma unroll
-          for (int i = 0; i < 32; ++i) io.accv[i] = __uint_as_float(raw[i]);
-          io.col_in_chunk = h * 32;
-          io.col_in_half = c * 64 + h * 32;
-          run_program<32, SP, true>(p.prog, io);
+        for (int h = 0; h < 2; ++h) {
+          uint32_t raw[16];
+          ld16(t_row + col + 16 * h, raw);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) io.accv[i] = __uint_as_float(raw[i]);
+          io.res[0] = res[2 * h]; io.res[1] = res[2 * h + 1];
+          if (h == 1 && q.c_input >= 0 && c + 32 < half_cols) fetch_residual(n0 + col + 32, res);
+          io.col = col + 16 * h; io.n = n0 + io.col; io.h = h;
+          run_program<16, SP, true>(p.prog, io);
         }
         fence_async_smem();
         __syncwarp();
-        if (lane == 0) { tma_store_2d(&q.tmD, io.chunk, n0 + c * 64, mw0); tma_store_commit(); }
+        if (elect_one()) { tma_store_2d(&q.tmD, io.chunk, n0 + col, m0 + sub * 32); tma_store_commit(); }
       }
       if (ew == 0 && lane == 0) TSTAMP(6);
-      if (lane == 0) tma_store_wait_all();
+      if (elect_one()) tma_store_wait_all();
       if (ew == 0 && lane == 0) TSTAMP(7);
     }
   }
@@ -479,18 +499,13 @@ void tile_gemm_plan(Launch& L) {
   }
   q.b_static = (gp.static_mask & 1u) ? 1 : 0;
   const int stage_bytes = tc2::BM * tc2::BK * 2 + q.bn * tc2::BK * 2;
-  // chunk buffers: a residual tile is prefetched into its own ones; without one they reuse the ring; the split form
-  // reads and writes global memory directly and needs none
-  const bool own_cbuf = q.c_input >= 0 && S == 1;
-  const int cbuf_bytes = tc2::BM * q.bn * 2;
-  const int fixed = 1024 + tile::kVecBytes + tile::kBarBytes + (own_cbuf ? cbuf_bytes : 0);
+  const int fixed = 1024 + tile::kVecBytes + tile::kBarBytes;
   int budget = tile::kSmemTwoPerSm;
   if (dev_env("DNNF_TILE_SMEM")) budget = atoi(dev_env("DNNF_TILE_SMEM")) * 1024;
   q.stages = std::max(2, std::min({8, q.kt_per, (budget - fixed) / stage_bytes}));
-  int ring = q.stages * stage_bytes;
+  int ring = q.stages * stage_bytes;                               // (the chunk buffers, 128 x bn bf16, are never more than that)
   if (S > 1) ring = std::max(ring, (S - 1) * (q.bn / S / 4) * tc2::BM * 16);          // the ring doubles as the receive buffer
-  q.cbuf_off = own_cbuf ? ring : 0;
-  q.tail_off = own_cbuf ? ring + cbuf_bytes : (S > 1 ? ring : std::max(ring, cbuf_bytes));
+  q.tail_off = ring;
   q.tmem_cols = q.bn < 32 ? 32 : q.bn;
   L.counter_bytes = L.scratch_bytes = 0;
   L.grid = (int)(tiles * S);
@@ -501,11 +516,11 @@ void tile_gemm_plan(Launch& L) {
 }
 
 static bool encode2d(CUtensorMap* tm, void* base, int64_t ext_inner, int64_t ext_outer, int64_t stride_outer_elems, int box_inner, int box_outer,
-                     std::string& err) {
+                     std::string& err, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   cuuint64_t dims[2] = {(cuuint64_t)ext_inner, (cuuint64_t)ext_outer};
   cuuint64_t strides[1] = {(cuuint64_t)stride_outer_elems * 2};
   cuuint32_t box[2] = {(cuuint32_t)box_inner, (cuuint32_t)box_outer};
-  return tma_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B, err);
+  return tma_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, swizzle, err);
 }
 
 bool tile_gemm_prepare(Launch& L, std::string& err) {
@@ -518,14 +533,9 @@ bool tile_gemm_prepare(Launch& L, std::string& err) {
   if (!encode2d(&q.tmA, a, gp.K, gp.M, gp.A.stride_row, tc2::BK, tc2::BM, err)) return false;
   if (q.b_kmajor) { if (!encode2d(&q.tmB, b, gp.K, gp.N, gp.B.stride_col, tc2::BK, q.bn, err)) return false; }
   else { if (!encode2d(&q.tmB, b, gp.N, gp.K, gp.B.stride_row, 64, tc2::BK, err)) return false; }
-  if (!encode2d(&q.tmD, d, gp.N, gp.M, gp.out[0].stride[1], 64, 32, err)) return false;
-  if (q.c_input >= 0) {
-    const TensorArg& c = gp.in[q.c_input];
-    uint16_t* cp = reinterpret_cast<uint16_t*>(c.ptr) + c.base;
-    if ((uintptr_t)cp & 15) { err = "epilogue operand is not 16-byte aligned"; return false; }
-    if (!encode2d(&q.tmC, cp, gp.N, gp.M, c.stride[1], 64, 32, err)) return false;
-  } else {
-    q.tmC = q.tmD;
+  if (!encode2d(&q.tmD, d, gp.N, gp.M, gp.out[0].stride[1], 32, 32, err, CU_TENSOR_MAP_SWIZZLE_64B)) return false;
+  if (q.c_input >= 0 && ((uintptr_t)(reinterpret_cast<uint16_t*>(gp.in[q.c_input].ptr) + gp.in[q.c_input].base) & 15)) {
+    err = "epilogue operand is not 16-byte aligned"; return false;
   }
   return true;
 }
