@@ -312,7 +312,9 @@ class Graph:
         self._check(lib.dnnf_bind_workspace(self.h, C.c_void_p(dev_ptr), nbytes))
 
     def run(self, stream=0):
-        self._check(lib.dnnf_run(self.h, C.c_void_p(stream)))
+        rc = lib.dnnf_run(self.h, stream)              # (an integer handle: the argument type converts it)
+        if rc != OK:
+            self._check(rc)
 
     def run_static_ws(self, stream=0):
         """dnnf_run with the between-block intermediates in the library's built-in array (no workspace needed)."""

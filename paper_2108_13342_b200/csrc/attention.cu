@@ -475,9 +475,10 @@ int lower_attention(const Graph& g, const std::vector<int>& ops, uint32_t flags,
 
 void attention_patch(Launch& L, const std::vector<void*>& ip, const std::vector<void*>& op, std::string& err) {
   AttnBlob& ab = ab_of(L);
+  if (L.tc_ready && L.encoded_ptrs.size() == ip.size() + op.size() && std::equal(ip.begin(), ip.end(), L.encoded_ptrs.begin()) &&
+      std::equal(op.begin(), op.end(), L.encoded_ptrs.begin() + ip.size())) return;
   std::vector<void*> now(ip);
   now.insert(now.end(), op.begin(), op.end());
-  if (L.tc_ready && now == L.encoded_ptrs) return;
   L.tc_ready = false;
   ab.a.A.ptr = ip[0]; ab.a.B.ptr = ip[1];
   for (int i = 0; i < ab.a.n_in; ++i) ab.a.in[i].ptr = ip[2 + i];

@@ -532,9 +532,10 @@ void patch_contraction(Launch& L, const std::vector<void*>& ip, const std::vecto
   if (L.variant != 1 && L.variant != 3 && L.variant != 4 && L.variant != 5 && L.variant != 8) return;
   // The tensor maps embed addresses: encode them again whenever ANY pointer of the block differs from the
   // ones they were made for (an epilogue operand in any position may be read through a map).
+  if (L.tc_ready && L.encoded_ptrs.size() == ip.size() + op.size() && std::equal(ip.begin(), ip.end(), L.encoded_ptrs.begin()) &&
+      std::equal(op.begin(), op.end(), L.encoded_ptrs.begin() + ip.size())) return;
   std::vector<void*> now(ip);
   now.insert(now.end(), op.begin(), op.end());
-  if (L.tc_ready && now == L.encoded_ptrs) return;
   L.tc_ready = false;
   bool ok = L.variant == 1 ? tc_gemm_prepare(L, err) : L.variant == 3 ? tc2_gemm_prepare(L, err) : L.variant == 5 ? tile_gemm_prepare(L, err) :
             L.variant == 8 ? tf32s_gemm_prepare(L, err) : tf32_gemm_prepare(L, err);

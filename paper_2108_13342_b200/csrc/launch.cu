@@ -29,12 +29,15 @@ int run_blocks(Graph& g, int only, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   g.last_status_base = g.ws_ptr;
   // Resolve every pointer first so that a failure launches nothing.
+  std::vector<void*> ip, op;
+  ip.reserve(16); op.reserve(8);
+  std::string err;
   for (int bi : g.run_order) {
     if (only >= 0 && bi != only) continue;
     Block& b = g.blocks[bi];
     Launch& L = b.launch;
     if (L.family == DNNF_FAMILY_ALIAS) continue;
-    std::vector<void*> ip, op;
+    ip.clear(); op.clear();
     for (int t : L.in_tensors) { void* p = resolve(g, t); if (!p) { g.err = "tensor '" + g.tensors[t].name + "' is not bound"; return DNNF_ERR_UNBOUND; } ip.push_back(p); }
     for (int t : L.out_tensors) { void* p = resolve(g, t); if (!p) { g.err = "output tensor is not bound"; return DNNF_ERR_UNBOUND; } op.push_back(p); }
     if (L.family == DNNF_FAMILY_ROW) {
@@ -44,7 +47,6 @@ int run_blocks(Graph& g, int only, void* stream) {
       for (size_t i = 0; i < ip.size(); ++i) L.ew.in[i].ptr = ip[i];
       for (size_t i = 0; i < op.size(); ++i) L.ew.out[i].ptr = op[i];
     } else {
-      std::string err;
       patch_contraction(L, ip, op, err);
       if (!err.empty()) { g.err = err; return DNNF_ERR_CUDA; }
     }
@@ -58,7 +60,7 @@ int run_blocks(Graph& g, int only, void* stream) {
       case DNNF_FAMILY_ALIAS: break;
       case DNNF_FAMILY_ELEMENTWISE: case DNNF_FAMILY_TRANSPOSE: rc = launch_ew(L, st); break;
       case DNNF_FAMILY_ROW: rc = launch_row(L, st); break;
-      default: { std::string err; rc = launch_contraction(L, g.ws_ptr, bi, st, err); if (rc) g.err = err; break; }
+      default: rc = launch_contraction(L, g.ws_ptr, bi, st, err); if (rc) g.err = err; break;
     }
     if (rc) {
       if (g.err.empty()) g.err = "kernel launch failed";

@@ -64,8 +64,14 @@ class Session:
         self.g.bind(self.ids[name], dev.data_ptr())
 
     def run(self, stream=None):
-        s = self.torch.cuda.current_stream(self.device) if stream is None else stream
-        self.g.run(s.cuda_stream)
+        # (a graph of one small kernel is bound by this call: a torch Stream object alone costs 1 us)
+        self.g.run(self._current_stream() if stream is None else stream.cuda_stream)
+
+    def _current_stream(self):
+        """Handle of torch's current stream on the session's device."""
+        if self.device.index is None:
+            return self.torch.cuda.current_stream(self.device).cuda_stream
+        return self.torch._C._cuda_getCurrentRawStream(self.device.index)
 
     def run_block(self, b, stream=None):
         s = self.torch.cuda.current_stream(self.device) if stream is None else stream
