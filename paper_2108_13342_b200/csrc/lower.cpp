@@ -178,6 +178,13 @@ bool backward_views(LowerCtx& cx, const Op& op, const View& vout, std::vector<Vi
 }
 
 // 1 = derived, 0 = not derivable from this operand (try another), -1 = error
+// Whether two views are the same index map over these extents (a dim of one element has no say).
+static bool same_map(const std::vector<int64_t>& ext, const View& a, const View& b) {
+  if (a.c0 != b.c0) return false;
+  for (size_t d = 0; d < ext.size(); ++d) if (ext[d] != 1 && a.coef[d] != b.coef[d]) return false;
+  return true;
+}
+
 static int forward_view_i(LowerCtx& cx, const Op& op, int slot, const View& vi, View& vo) {
   const Graph& g = cx.g;
   const Tensor& in = g.tensors[op.in[slot]];
@@ -232,7 +239,7 @@ static int forward_view_i(LowerCtx& cx, const Op& op, int slot, const View& vi, 
     std::vector<View> vin;
     SplitRequest keep = cx.split;
     if (!backward_views(cx, op, cand, vin)) { if (cx.split.dim >= 0) return -1; cx.split = keep; cx.why.clear(); return 0; }
-    if (!(vin[slot] == vi)) return 0;
+    if (!same_map(cx.ext, vin[slot], vi)) return 0;
     vo = cand; return 1;
   }
   cx.why = std::string("no index map through ") + op_name(k);
@@ -252,7 +259,7 @@ static bool derive_once(LowerCtx& cx, int ref, const std::set<int>& stop_ops) {
   auto set_view = [&](int t, const View& v) -> bool {
     auto it = cx.views.find(t);
     if (it == cx.views.end()) { cx.views[t] = v; q.push_back(t); return true; }
-    if (!(it->second == v)) { cx.why = "one value is needed under two different index maps"; return false; }
+    if (!same_map(cx.ext, it->second, v)) { cx.why = "one value is needed under two different index maps"; return false; }
     return true;
   };
   while (!q.empty()) {

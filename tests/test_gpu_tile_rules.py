@@ -135,3 +135,20 @@ def test_attention_with_many_keys(seq):
     from paper_2108_13342_b200.workloads import encoder
     from util import check_blocks
     check_blocks(encoder(layers=1, batch=2, seq=seq, hidden=128, heads=2, ffn=128), B.PLAN_BEYOND_TABLE3, B.REWRITE_CANON_MACRO, min_checked=1)
+
+
+@pytest.mark.parametrize("batch,heads,seq,d", [(1, 4, 200, 64), (1, 1, 72, 64), (2, 1, 136, 64), (1, 12, 248, 64)])
+def test_head_merge_after_a_product_with_unit_dims_is_store_indexing(batch, heads, seq, d):
+    """[batch, heads] with extents of one: their strides carry no index, so the Transpose joins the product's block."""
+    g = graph()
+    g.ext("P", (batch, heads, seq, seq), "bf16"); g.ext("V", (batch, heads, seq, d), "bf16")
+    t = g.add("MatMul", ["P", "V"])
+    t = g.add("Transpose", [t], perm=(0, 2, 1, 3))
+    t = g.add("Reshape", [t], shape=(batch, seq, heads * d))
+    g.mark_output(t)
+    ins = {"P": _bf(rnd((batch, heads, seq, seq), 960, 0, 0.1)), "V": _bf(rnd((batch, heads, seq, d), 961, -1, 1))}
+    wl = W.Workload(g, ins)
+    s, got, ref = run_both(wl, FUSED)
+    (name,) = wl.graph.outputs
+    close(got[name], ref[name], RTOL_BF16)
+    assert len([b for b in s.g.blocks() if b["family"] != "alias"]) == 1
