@@ -30,6 +30,7 @@ int tc2_gemm_launch(const Launch& L, cudaStream_t st);
 void tc2_set_scratch(Launch& L, void* ws_base);
 size_t tile_blob_bytes();
 bool tile_gemm_eligible(const GemmParams& gp);
+void tile_set_scratch(Launch& L, void* ws_base);
 bool tile_gemm_preferred(const GemmParams& gp);
 void tile_gemm_plan(Launch& L);
 bool tile_gemm_prepare(Launch& L, std::string& err);
@@ -567,6 +568,7 @@ int launch_contraction(const Launch& L, void* status_words, int block_index, cud
   if (L.variant == 5) {
     Launch& M = const_cast<Launch&>(L);
     gp_of(M).status = gp.status; gp_of(M).block_index = block_index;
+    tile_set_scratch(M, status_words);
     int rc = tile_gemm_launch(L, st);
     if (rc) err = "tensor-core tile GEMM launch failed";
     return rc;

@@ -15,9 +15,15 @@
 //     registers, the first chunk's values before the accumulator is waited for.
 // Roles: warps 0, 1 TMA producers (producer j loads the k-tiles j, j+2, ...), warp 2 tensor-memory allocation and MMA
 // issue, warps 3..10 epilogue (two warps per 32 rows, half of the tile's columns each): tcgen05.ld -> micro-op program on 16
-// columns at a time -> bf16 -> swizzled 32 x 32 chunk -> TMA store.With four warps and 32 columns at a time the epilogue
+// columns at a time -> bf16 -> swizzled 32 x 32 chunk -> TMA store.  With four warps and 32 columns at a time the epilogue
 // was the longer half of these kernels: 248 x 2304 x 768 + bias 6.1 -> 5.4 us, 248 x 768 x 768 5.5 -> 4.8, 248 x 3072 x 768 +
 // GELU 6.8 -> 6.0, 1024 x 768 x 768 6.0 -> 5.4.
+// Long K, few tiles: the k-tiles of a tile are shared by up to four CTAs that meet in the workspace (kMode 2): every epilogue
+// warp writes its partial sums to scratch and bumps its part's counter; the warp whose bump is the last adds all slices in
+// slice order and finishes.  Nobody waits for anybody, no cluster is launched, and the set-up of the CTAs overlaps the previous
+// kernel: 248 x 768 x 3072 14.0 (CTA pairs) -> 10.5 us, 1024 x 768 x 3072 13.7 -> 12.9.  About 5 us of that is the hand-over (write,
+// fence, counter, read back in two rounds); 128-column tiles (16.5 us) or more slices (18.6 us with 4) lose, reading the
+// partial sums as float4, three slices at once, costs more registers than the 80 a thread has here (14.8 us).
 // Every wait is bounded; on expiry the CTA records DNNF_ERR_TIMEOUT and releases tensor memory.
 //
 // Every TMA load in this file is a plain per-CTA load; no clusters are used.
@@ -39,6 +45,7 @@ namespace tile {
 using namespace tc2;
 
 constexpr int kEpiWarps = 8, kThreads = 96 + 32 * kEpiWarps;         // 2 producer warps, 1 issuer warp, 8 epilogue warps
+constexpr int kMaxSlices = 4;                                        // CTAs that share a tile through the workspace
 constexpr int kChunkB = 32 * 64;                                     // 32 rows x 32 bf16, 64-byte swizzle
 constexpr int kVecBytes = kEpiWarps * kMaxVec * kBiasFloats * 4;     // staged row-invariant operands, per warp
 constexpr int kBarBytes = 256;
@@ -52,7 +59,11 @@ struct Params {
   int32_t tail_off;          // staged vectors, then barriers
   int32_t b_static;          // B is never written by a kernel of the graph
   int32_t tmem_cols;
-  int32_t ksplit, kt_per;    // CTAs of a cluster that share a tile (1, 2 or 4) and the k-tiles each of them takes
+  int32_t ksplit, kt_per;    // CTAs that share a tile (a cluster's, or through the workspace) and the k-tiles each of them takes
+  int32_t ws_split;          // they meet in the workspace
+  FastDiv fd_tiles;
+  float* scratch;            // partial sums: [tile][epilogue warp][slice][column][32 rows] fp32
+  int32_t* counters;         // arrivals, one per tile and epilogue warp; zero between runs
   FastDiv fd_tiles_n;
 };
 
@@ -167,9 +178,10 @@ __device__ __forceinline__ void st_cluster_f4(uint32_t cluster_addr, float4 v) {
 // into CTA j's operand ring (idle by then), and CTA j adds them to its own accumulator, runs the epilogue program on
 // its slice and stores it.  Two cluster barriers frame the exchange: all main loops done (the rings are free), all
 // partial sums written.  The main loop shrinks S-fold, and so does each CTA's epilogue.
-template <class SP, bool kSplit>
+template <class SP, int kMode>          // 0: a CTA per tile, 1: cluster split over K, 2: split over K through the workspace
 __global__ void __launch_bounds__(kThreads, 2)
 gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Params q) {
+  constexpr bool kSplit = kMode == 1;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int BN = q.bn, stages = q.stages;
@@ -202,14 +214,14 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   const uint32_t tmem_base = *tmem_slot;
   if (threadIdx.x == 0) TSTAMP(1);
 
-  const int S = kSplit ? q.ksplit : 1;
-  const int rank = kSplit ? (int)cluster_rank() : 0;
-  const int tile = kSplit ? (int)(blockIdx.x / (unsigned)S) : (int)blockIdx.x;
+  const int S = kMode ? q.ksplit : 1;
+  const int rank = kSplit ? (int)cluster_rank() : kMode == 2 ? (int)fd_div(blockIdx.x, q.fd_tiles) : 0;
+  const int tile = kSplit ? (int)(blockIdx.x / (unsigned)S) : kMode == 2 ? (int)blockIdx.x - rank * (int)q.fd_tiles.d : (int)blockIdx.x;
   const int tm = (int)fd_div((uint32_t)tile, q.fd_tiles_n), tn = tile - tm * q.tiles_n;
   const int m0 = tm * BM, n0 = tn * BN;
   // this CTA's k-tiles
-  const int kt0 = kSplit ? rank * q.kt_per : 0;
-  const int k_tiles = kSplit ? min(q.k_tiles - kt0, q.kt_per) : q.k_tiles;
+  const int kt0 = kMode ? rank * q.kt_per : 0;
+  const int k_tiles = kMode ? min(q.k_tiles - kt0, q.kt_per) : q.k_tiles;
 
   if (warp < 2) {
     // ---------------- TMA producers: warp j loads the k-tiles j, j+2, j+4, ... ----------------
@@ -373,16 +385,57 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
       if (ew == 0 && lane == 0) TSTAMP(9);
     } else if (ok) {
       tc_fence_after();
-      for (int c = 0; c < half_cols; c += 32) {
+      bool finish = true;
+      const float* parts = nullptr;
+      if (kMode == 2) {
+        const uint32_t unit = (uint32_t)tile * kEpiWarps + (uint32_t)ew;
+        float* mine = q.scratch + ((size_t)unit * S + rank) * (size_t)(half_cols * 32) + lane;
+#pragma unroll 1
+        for (int c = 0; c < half_cols; c += 16) {
+          uint32_t raw[16];
+          ld16(t_row + half * half_cols + c, raw);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) mine[(c + i) * 32] = __uint_as_float(raw[i]);      // a 128-byte line per instruction
+        }
+        __threadfence();                         // this lane's partial sums are visible before the counter moves
+        __syncwarp();
+        int old = 0;
+        if (lane == 0) old = atomicAdd(&q.counters[unit], 1);
+        old = __shfl_sync(0xffffffffu, old, 0);
+        finish = old == S - 1;                   // else somebody else finishes this part (uniform over the warp)
+        if (finish) {
+          if (lane == 0) q.counters[unit] = 0;   // all slices have arrived: ready for the next run
+          __threadfence();
+          parts = q.scratch + (size_t)unit * S * (size_t)(half_cols * 32) + lane;
+        }
+      }
+      for (int c = 0; finish && c < half_cols; c += 32) {
         const int col = half * half_cols + c;
         if (n0 + col >= p.N) break;                                // (uniform over the warp)
         io.chunk = cbuf + (c >> 5) * kChunkB;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          uint32_t raw[16];
-          ld16(t_row + col + 16 * h, raw);
+          if (kMode == 2) {
+            // slices in order, two slices' loads in flight (written by other SMs: read from L2)
 #pragma unroll
-          for (int i = 0; i < 16; ++i) io.accv[i] = __uint_as_float(raw[i]);
+            for (int i = 0; i < 16; ++i) io.accv[i] = 0.0f;
+            for (int sl = 0; sl < S; sl += 2) {
+              const float* o = parts + (size_t)sl * (size_t)(half_cols * 32) + (c + 16 * h) * 32;
+              const bool two = sl + 1 < S;
+              float v0[16], v1[16];
+#pragma unroll
+              for (int i = 0; i < 16; ++i) v0[i] = __ldcg(o + i * 32);
+#pragma unroll
+              for (int i = 0; i < 16; ++i) v1[i] = two ? __ldcg(o + half_cols * 32 + i * 32) : 0.0f;
+#pragma unroll
+              for (int i = 0; i < 16; ++i) io.accv[i] = (io.accv[i] + v0[i]) + v1[i];
+            }
+          } else {
+            uint32_t raw[16];
+            ld16(t_row + col + 16 * h, raw);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) io.accv[i] = __uint_as_float(raw[i]);
+          }
           io.res[0] = res[2 * h]; io.res[1] = res[2 * h + 1];
           if (h == 1 && q.c_input >= 0 && c + 32 < half_cols) fetch_residual(n0 + col + 32, res);
           io.col = col + 16 * h; io.n = n0 + io.col; io.h = h;
@@ -444,18 +497,27 @@ bool tile_gemm_eligible(const GemmParams& gp) {
   return full <= 1 && vec <= tc2::kMaxVec;
 }
 
-// Measured on the projection and feed-forward shapes of a 1024-token encoder layer: a k-tile costs a CTA about 0.35 us
+// Slices of K that meet in the workspace: with long K (the hand-over costs about 5 us, a k-tile 0.22) and few enough 128 x 64
+// tiles for three or four CTAs each, two per SM, and at least eight k-tiles per CTA.  Two slices are no gain over CTA pairs
+// (1024 x 768 x 3072: 13.9 against 13.7 us; with three 12.9).
+static int ws_slices(const GemmParams& gp) {
+  const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
+  const int64_t tiles = (int64_t)((gp.M + tc2::BM - 1) / tc2::BM) * ((gp.N + 63) / 64);
+  if (k_tiles < 32 || plan_flag(DNNF_PLAN_NO_SPLIT_K) || plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K)) return 1;
+  const int64_t s = std::min<int64_t>({tile::kMaxSlices, 2 * sm_count() / tiles, k_tiles / 8});
+  return s >= 3 ? (int)s : 1;
+}
+
+// Measured on the projection and feed-forward shapes of a 1024-token encoder layer: a k-tile costs a CTA about 0.22 us
 // whatever the tile's size, so a problem with few 256 x 256 tiles and a short K finishes sooner as many small tiles
-// (1024 x 768 x 768: 7.2 against 7.8 us; 1024 x 2304 x 768: 7.4 against 8.1; 1024 x 3072 x 768: 9.7 against 11.1), while a
-// long K is better off with the CTA-pair kernel and its split over K (1024 x 768 x 3072: 14.2 against 18.5 us).
+// (1024 x 768 x 768: 5.4 against 7.8 us; 1024 x 2304 x 768: 7.4 against 8.1; 1024 x 3072 x 768: 10.1 against 11.1); with a long K
+// only where CTAs can share its k-tiles through the workspace.
 bool tile_gemm_preferred(const GemmParams& gp) {
   if (plan_flag(DNNF_PLAN_NO_TILE_GEMM)) return false;
   if (dev_env("DNNF_GEMM_TILE")) return atoi(dev_env("DNNF_GEMM_TILE")) != 0;
   const int64_t pair_tiles = (int64_t)((gp.M + 255) / 256) * ((gp.N + 255) / 256);
   const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
-  // a long K is better off with the CTA-pair kernel and its split over K (1024 x 768 x 3072: 14.2 us against 22.6 us
-  // here without a split and 15.5 us with the cluster split below)
-  return pair_tiles < sm_count() / 2 && (k_tiles <= 16 || plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K));
+  return pair_tiles < sm_count() / 2 && (k_tiles <= 16 || plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K) || ws_slices(gp) > 1);
 }
 
 void tile_gemm_plan(Launch& L) {
@@ -479,8 +541,17 @@ void tile_gemm_plan(Launch& L) {
   // 1024 x 768 x 768 ends after 2.6 instead of 5.9 us, but the hand-over (0.6 us barrier, 1.2 us of remote stores, 2 us
   // until every CTA's stores have arrived) and 2.5 us more per launch of a cluster in a chain of dependent kernels eat
   // all of it (11.5 against 8.5 us per launch), hence off by default.
-  const int64_t tiles = (int64_t)tiles_m * q.tiles_n;
   int S = 1;
+  q.ws_split = ws_slices(gp) > 1;
+  if (q.ws_split) {
+    S = ws_slices(gp);
+    q.bn = 64;
+    q.tiles_n = (gp.N + 63) / 64;
+    q.fd_tiles_n = make_fastdiv((uint32_t)q.tiles_n);
+    gp.tiles_n = q.tiles_n;
+  }
+  const int64_t tiles = (int64_t)tiles_m * q.tiles_n;
+  q.fd_tiles = make_fastdiv((uint32_t)tiles);
   if (plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K) && !plan_flag(DNNF_PLAN_NO_SPLIT_K)) {
     for (int cand : {4, 2}) {
       if (q.bn / cand < 32) continue;
@@ -490,7 +561,7 @@ void tile_gemm_plan(Launch& L) {
   if (dev_env("DNNF_TILE_SPLIT")) { const int v = atoi(dev_env("DNNF_TILE_SPLIT")); if ((v == 1 || v == 2 || v == 4) && q.bn / v >= 32 && q.k_tiles >= v) S = v; }
   q.ksplit = S;
   q.kt_per = (q.k_tiles + S - 1) / S;
-  if ((S - 1) * q.kt_per >= q.k_tiles) { q.ksplit = S = 1; q.kt_per = q.k_tiles; }     // every CTA of the cluster needs a k-tile
+  if ((S - 1) * q.kt_per >= q.k_tiles) { q.ksplit = S = 1; q.kt_per = q.k_tiles; q.ws_split = 0; }     // every CTA that shares a tile needs a k-tile
   q.c_input = -1;
   int vec_slot = 0;
   for (int i = 0; i < gp.n_in; ++i) {
@@ -504,10 +575,11 @@ void tile_gemm_plan(Launch& L) {
   if (dev_env("DNNF_TILE_SMEM")) budget = atoi(dev_env("DNNF_TILE_SMEM")) * 1024;
   q.stages = std::max(2, std::min({8, q.kt_per, (budget - fixed) / stage_bytes}));
   int ring = q.stages * stage_bytes;                               // (the chunk buffers, 128 x bn bf16, are never more than that)
-  if (S > 1) ring = std::max(ring, (S - 1) * (q.bn / S / 4) * tc2::BM * 16);          // the ring doubles as the receive buffer
+  if (S > 1 && !q.ws_split) ring = std::max(ring, (S - 1) * (q.bn / S / 4) * tc2::BM * 16);          // the ring doubles as the receive buffer
   q.tail_off = ring;
   q.tmem_cols = q.bn < 32 ? 32 : q.bn;
-  L.counter_bytes = L.scratch_bytes = 0;
+  L.counter_bytes = q.ws_split ? tiles * tile::kEpiWarps * 4 : 0;
+  L.scratch_bytes = q.ws_split ? tiles * S * tc2::BM * q.bn * 4 : 0;
   L.grid = (int)(tiles * S);
   L.threads = tile::kThreads;
   L.smem = (size_t)q.tail_off + tile::kVecBytes + tile::kBarBytes + 1024;
@@ -542,16 +614,17 @@ bool tile_gemm_prepare(Launch& L, std::string& err) {
 
 struct TileLauncher {
   const Launch& L; cudaStream_t st; cudaError_t rc;
+  template <class SP, int kMode> void plain() {
+    static PerDeviceOnce once;       // per instantiation
+    if (once.first_use()) cudaFuncSetAttribute(tile::gemm_tile_kernel<SP, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    rc = launch_pdl(tile::gemm_tile_kernel<SP, kMode>, dim3(L.grid), dim3(tile::kThreads), L.smem, st, gp_of(L), tl_of(L));
+  }
   template <class SP> void run() {
     const int S = tl_of(L).ksplit;
-    if (S <= 1) {
-      static PerDeviceOnce once;       // per instantiation
-      if (once.first_use()) cudaFuncSetAttribute(tile::gemm_tile_kernel<SP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      rc = launch_pdl(tile::gemm_tile_kernel<SP, false>, dim3(L.grid), dim3(tile::kThreads), L.smem, st, gp_of(L), tl_of(L));
-      return;
-    }
+    if (S <= 1) { plain<SP, 0>(); return; }
+    if (tl_of(L).ws_split) { plain<SP, 2>(); return; }
     static PerDeviceOnce once;
-    if (once.first_use()) cudaFuncSetAttribute(tile::gemm_tile_kernel<SP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (once.first_use()) cudaFuncSetAttribute(tile::gemm_tile_kernel<SP, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(L.grid); cfg.blockDim = dim3(tile::kThreads); cfg.dynamicSmemBytes = L.smem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -560,9 +633,16 @@ struct TileLauncher {
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    rc = cudaLaunchKernelEx(&cfg, tile::gemm_tile_kernel<SP, true>, gp_of(L), tl_of(L));
+    rc = cudaLaunchKernelEx(&cfg, tile::gemm_tile_kernel<SP, 1>, gp_of(L), tl_of(L));
   }
 };
+
+// split-K scratch and counters live in the bound workspace at the offsets the planner chose
+void tile_set_scratch(Launch& L, void* ws_base) {
+  tile::Params& q = tl_of(L);
+  q.scratch = L.scratch_off >= 0 ? reinterpret_cast<float*>(reinterpret_cast<char*>(ws_base) + L.scratch_off) : nullptr;
+  q.counters = L.counter_off >= 0 ? reinterpret_cast<int32_t*>(reinterpret_cast<char*>(ws_base) + L.counter_off) : nullptr;
+}
 
 int tile_gemm_launch(const Launch& L, cudaStream_t st) {
   TileLauncher F{L, st, cudaSuccess};
