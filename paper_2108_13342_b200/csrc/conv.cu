@@ -237,10 +237,11 @@ template <class SP>
 __global__ void __launch_bounds__(256, 4) dwconv_kernel(const __grid_constant__ DwParams p, int HS) {
   extern __shared__ float4 kws[];                // [9][C/4]
   pdl_launch_dependents();
-  pdl_wait();
   const int C4 = p.C / 4;
+  if (!p.k_static) pdl_wait();                   // else the weights arrive while the previous kernel ends
   for (int i = threadIdx.x; i < 9 * C4; i += 256) kws[i] = __ldg(reinterpret_cast<const float4*>(p.k) + i);
   __syncthreads();
+  if (p.k_static) pdl_wait();
   const int strips = (p.H + HS - 1) / HS;
   int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const int64_t total = (int64_t)p.N * strips * p.W * C4;
@@ -274,7 +275,7 @@ __global__ void __launch_bounds__(256, 4) dwconv_kernel(const __grid_constant__ 
 }
 
 size_t dwconv_tma_blob_bytes();
-bool dwconv_tma_plan(Launch& L);
+bool dwconv_tma_plan(Launch& L, bool weights_static, uint32_t static_inputs);
 bool dwconv_tma_prepare(Launch& L, std::string& err);
 int dwconv_tma_launch(const Launch& L, int32_t* status, int block_index, cudaStream_t st);
 
@@ -348,7 +349,11 @@ int lower_dwconv(const Graph& g, const std::vector<int>& ops, int anchor, Block&
   for (auto& a : cx.outs) { L.out_tensors.push_back(a.tensor); out.outputs.push_back(a.tensor); }
   L.family = DNNF_FAMILY_DWCONV;
   L.flops = 2ll * 9 * Y.numel();
-  if (dwconv_tma_plan(L)) { out.lowered = true; return DNNF_OK; }
+  auto is_static = [&](int t) { return g.tensors[t].external && g.tensors[t].producer < 0 && !g.tensors[t].is_output; };
+  uint32_t static_inputs = 0;
+  for (size_t i = 0; i < cx.ins.size(); ++i) if (is_static(cx.ins[i].tensor)) static_inputs |= 1u << i;
+  dp.k_static = is_static(A.in[1]);
+  if (dwconv_tma_plan(L, dp.k_static, static_inputs)) { out.lowered = true; return DNNF_OK; }
   // rows per thread: enough threads to fill the machine, long enough strips to reuse the window
   int hs = dp.H;
   int64_t threads_full = (int64_t)dp.N * dp.W * (dp.C / 4);

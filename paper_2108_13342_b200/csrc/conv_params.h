@@ -9,10 +9,12 @@
 
 namespace dnnf {
 
-struct DwParams {
+// (its size is a multiple of 16: a block's tensor map follows it and is encoded in place)
+struct alignas(16) DwParams {
   int32_t N, H, W, C;
   const float* x;
   const float* k;          // [3][3][C]
+  int32_t k_static;        // k is a graph input nobody writes: it may be read before the previous kernel has ended
   int32_t n_in, n_out;
   TensorArg in[kMaxIn];    // strides over (c, w, h, n), innermost first
   TensorArg out[kMaxOut];

@@ -172,3 +172,15 @@ def test_head_merge_after_a_product_with_unit_dims_is_store_indexing(batch, head
     (name,) = wl.graph.outputs
     close(got[name], ref[name], RTOL_BF16)
     assert len([b for b in s.g.blocks() if b["family"] != "alias"]) == 1
+
+
+@pytest.mark.parametrize("cfg", [(32, 14, 14, 384), (2, 56, 56, 144), (40, 7, 9, 960), (1, 120, 33, 100), (64, 15, 16, 20)])
+def test_dwconv_tiles_of_rows_columns_and_channel_blocks(cfg):
+    n, h, w, c = cfg
+    g = graph()
+    g.ext("X", (n, h, w, c)); g.ext("Kd", (3, 3, c), kind="weight"); g.ext("s", (c,), kind="weight"); g.ext("t", (c,), kind="weight")
+    e = g.add("ScaleShift", [g.add("DwConv3x3", ["X", "Kd"]), "s", "t"], axis=-1)
+    g.mark_output(g.add("Clip", [e], lo=0.0, hi=6.0))
+    ins = {"X": rnd((n, h, w, c), 21, -1, 1), "Kd": rnd((3, 3, c), 22, -0.5, 0.5), "s": rnd((c,), 23, 0.5, 1.5), "t": rnd((c,), 24, -0.5, 0.5)}
+    s = check(W.Workload(g, ins), RTOL_F32, FUSED, expect_blocks=1)
+    assert s.g.blocks()[0]["variant"] == -1
