@@ -184,3 +184,18 @@ def test_dwconv_tiles_of_rows_columns_and_channel_blocks(cfg):
     ins = {"X": rnd((n, h, w, c), 21, -1, 1), "Kd": rnd((3, 3, c), 22, -0.5, 0.5), "s": rnd((c,), 23, 0.5, 1.5), "t": rnd((c,), 24, -0.5, 0.5)}
     s = check(W.Workload(g, ins), RTOL_F32, FUSED, expect_blocks=1)
     assert s.g.blocks()[0]["variant"] == -1
+
+
+@pytest.mark.parametrize("kind", ["AveragePool", "MaxPool"])
+@pytest.mark.parametrize("n,k,c", [(1, 33, 132), (2, 32, 128), (3, 17, 4), (1, 64, 260)])
+def test_wide_pool_slices_shared_by_the_warps(kind, n, k, c):
+    """Global pools sliced over 8 to 100 CTAs; the last one to arrive adds the slices with all its warps, twice on one workspace."""
+    g = graph()
+    g.ext("X", (n, k, k, c))
+    g.mark_output(g.add(kind, ["X"], kernel=k, stride=1, pad=0))
+    s = check(W.Workload(g, {"X": rnd((n, k, k, c), 980, -1, 1)}), RTOL_F32, FUSED, expect_blocks=1)
+    (name,) = s.desc.outputs
+    first = s.output(name)
+    s.buffers[name].fill_(float("nan"))
+    s.run()
+    assert np.array_equal(s.output(name), first)
