@@ -50,6 +50,9 @@ bool tf32_gemm_eligible(const GemmParams& gp);
 void tf32_gemm_plan(Launch& L);
 bool tf32_gemm_prepare(Launch& L, std::string& err);
 int tf32_gemm_launch(const Launch& L, cudaStream_t st);
+bool conv_thin_eligible(const GemmParams& gp);
+void conv_thin_plan(Launch& L);
+int conv_thin_launch(const Launch& L, cudaStream_t st);
 bool conv_small_eligible(const GemmParams& gp);
 void conv_small_plan(Launch& L);
 int conv_small_launch(const Launch& L, cudaStream_t st);
@@ -498,6 +501,8 @@ int lower_contraction(const Graph& g, const std::vector<int>& ops, uint32_t flag
   } else if (tc_gemm_eligible(gp)) {
     L.variant = 1;
     tc_gemm_plan(L);
+  } else if (conv_thin_eligible(gp)) {
+    conv_thin_plan(L);
   } else if (conv_small_eligible(gp) && (gp.M <= small_m_limit() || !(tf32_gemm_eligible(gp) || tf32s_gemm_eligible(gp)))) {
     conv_small_plan(L);
   } else if (tf32s_gemm_eligible(gp) && (!tf32_gemm_eligible(gp) || tf32s_tiles(gp.M, gp.N, gp.K) <= 2 * sm_count() || dev_env("DNNF_TF32S_PREFER")) &&
@@ -552,6 +557,7 @@ int launch_contraction(const Launch& L, void* status_words, int block_index, cud
   if (L.family == DNNF_FAMILY_INSTNORM) { int rc = instnorm_launch(L, st); if (rc) err = "instance normalisation launch failed"; return rc; }
   if (L.family == DNNF_FAMILY_DWCONV) { int rc = dwconv_launch(L, status_words, block_index, st); if (rc) err = "depthwise convolution launch failed"; return rc; }
   if (L.variant == 2) { int rc = conv1x1_direct_launch(L, st); if (rc) err = "pointwise convolution launch failed"; return rc; }
+  if (L.variant == 9) { int rc = conv_thin_launch(L, st); if (rc) err = "pointwise convolution launch failed"; return rc; }
   if (L.variant == 7) { int rc = conv_small_launch(L, st); if (rc) err = "pointwise convolution launch failed"; return rc; }
   if ((L.variant == 1 || L.variant == 3 || L.variant == 4 || L.variant == 5 || L.variant == 8) && !L.tc_ready) { err = "tensor maps of the block are not encoded"; return 1; }
   GemmParams gp = gp_of(L);

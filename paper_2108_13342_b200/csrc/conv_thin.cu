@@ -1,0 +1,172 @@
+// fp32 pointwise convolution / matrix product with a thin result: [M x K] * [K x N] with N = 4 or 8 and many rows.
+//
+// What bounds it: reading x once (64 bytes a row at K = 16) and writing 16 or 32 bytes a row; the products are a few
+// hundred FMAs a row.  On the tensor-core kernels a 128-row tile has the price of a whole tile (split, MMA, epilogue:
+// about 1 us) whatever its width.  Here four neighbouring lanes share a row: each takes every fourth 16-byte piece of it
+// (a warp's load covers whole rows, run after run of bytes) and forms partial results for four rows; the four lanes then
+// trade partial sums so that each ends up with ONE complete row, 3 x N shuffles for four rows.  Weights sit in shared memory, read
+// as 16-byte words that the eight row groups of a warp share.  Rows x K x N + bias + tanh, us, split-TF32 kernels / here:
+// 524288 x 16 x 4 27.8 / 11.7 (3.6 TB/s), 65536 x 16 x 4 6.7 / 3.6, 4096 x 16 x 4 4.0 / 2.6, 65536 x 32 x 8 7.0 / 5.4.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "chain.cuh"
+#include "conv_params.h"
+#include "gemm_params.h"
+#include "launch_util.h"
+#include "lower.h"
+
+namespace dnnf {
+
+namespace thin {
+
+constexpr int THREADS = 256, ROWS = 32;          // rows per warp and step: 8 groups of 4 lanes x 4 rows
+
+template <int TN>
+struct RowIO {
+  static constexpr int VV = TN;
+  const GemmParams& p;
+  float accv[TN];
+  uint32_t row;
+  __device__ __forceinline__ uint32_t off(const TensorArg& a, int j) const {
+    return (uint32_t)a.base + row * (uint32_t)a.stride[1] + (uint32_t)(4 * j) * (uint32_t)a.stride[0];
+  }
+  __device__ __forceinline__ void load(int idx, float (&dst)[VV]) const {
+    const TensorArg& a = p.in[idx];
+#pragma unroll
+    for (int j = 0; j < TN / 4; ++j) {
+      float* d = &dst[4 * j];
+      if (a.stride[0] == 0) { float x = load_scalar<true>(a, off(a, j)); d[0] = d[1] = d[2] = d[3] = x; }
+      else load_vec4<true>(a, off(a, j), d);
+    }
+  }
+  __device__ __forceinline__ void anchor(float (&dst)[VV]) const {
+#pragma unroll
+    for (int v = 0; v < VV; ++v) dst[v] = accv[v];
+  }
+  __device__ __forceinline__ void store(int idx, const float (&val)[VV]) const {
+    const TensorArg& a = p.out[idx];
+#pragma unroll
+    for (int j = 0; j < TN / 4; ++j) store_vec4<true>(a, off(a, j), &val[4 * j], false);
+  }
+  __device__ __forceinline__ void row_reduce(int, float (&)[VV]) const {}
+};
+
+template <int TN, class SP>
+__global__ void __launch_bounds__(THREADS) conv_thin_kernel(const __grid_constant__ GemmParams p) {
+  extern __shared__ __align__(16) float ws[];    // [K rounded up to 16 / 4][4 x TN], zero past K; pitch: the four lanes of a
+  constexpr int PITCH = 4 * TN + 4;              // group read four different bank groups
+  pdl_launch_dependents();
+  const bool early = (p.static_mask & 1u) != 0;  // weights nobody writes: read while the previous kernel ends
+  if (!early) pdl_wait();
+  const int K16 = (p.K + 15) & ~15;
+  const float* W = reinterpret_cast<const float*>(p.B.ptr) + p.B.base;
+  for (int i = threadIdx.x * 4; i < K16 * TN; i += THREADS * 4)
+    *reinterpret_cast<float4*>(&ws[(i / (4 * TN)) * PITCH + i % (4 * TN)]) = i < p.K * TN ? __ldg(reinterpret_cast<const float4*>(W + i)) : make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
+  if (early) pdl_wait();
+  const float* X = reinterpret_cast<const float*>(p.A.ptr) + p.A.base;
+  const int lane = threadIdx.x & 31, g = lane >> 2, j = lane & 3;
+  const int64_t row0 = ((int64_t)blockIdx.x * (THREADS / 32) + (threadIdx.x >> 5)) * ROWS;
+  float acc[4][TN];
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+#pragma unroll
+    for (int v = 0; v < TN; ++v) acc[u][v] = 0.0f;
+  const float* xr[4];
+  bool ok[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int64_t m = row0 + u * 8 + g;
+    ok[u] = m < p.M;
+    xr[u] = X + (ok[u] ? m : 0) * p.A.stride_row;
+  }
+#pragma unroll 2
+  for (int k = j * 4; k < K16; k += 16) {
+    float4 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = ok[u] && k < p.K ? __ldg(reinterpret_cast<const float4*>(xr[u] + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+#pragma unroll
+      for (int n = 0; n < TN / 4; ++n) {
+        const float4 w = *reinterpret_cast<const float4*>(&ws[(k >> 2) * PITCH + e * TN + 4 * n]);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float xe = e == 0 ? x[u].x : e == 1 ? x[u].y : e == 2 ? x[u].z : x[u].w;
+          acc[u][4 * n] = fmaf(xe, w.x, acc[u][4 * n]); acc[u][4 * n + 1] = fmaf(xe, w.y, acc[u][4 * n + 1]);
+          acc[u][4 * n + 2] = fmaf(xe, w.z, acc[u][4 * n + 2]); acc[u][4 * n + 3] = fmaf(xe, w.w, acc[u][4 * n + 3]);
+        }
+      }
+  }
+  // lane j of a group keeps row u = j: bit 1 first (rows {0, 1} against {2, 3}), then bit 0
+  RowIO<TN> io{p};
+  const bool hi = (j & 2) != 0, odd = (j & 1) != 0;
+  float two[2][TN];
+#pragma unroll
+  for (int v = 0; v < TN; ++v) {
+    const float s0 = hi ? acc[0][v] : acc[2][v], s1 = hi ? acc[1][v] : acc[3][v];          // what the partner needs
+    const float r0 = __shfl_xor_sync(0xffffffffu, s0, 2), r1 = __shfl_xor_sync(0xffffffffu, s1, 2);
+    two[0][v] = (hi ? acc[2][v] : acc[0][v]) + r0;
+    two[1][v] = (hi ? acc[3][v] : acc[1][v]) + r1;
+  }
+#pragma unroll
+  for (int v = 0; v < TN; ++v) {
+    const float r = __shfl_xor_sync(0xffffffffu, odd ? two[0][v] : two[1][v], 1);
+    io.accv[v] = (odd ? two[1][v] : two[0][v]) + r;
+  }
+  const int64_t m = row0 + j * 8 + g;
+  if (m >= p.M) return;
+  io.row = (uint32_t)m;
+  run_program<TN, SP>(p.prog, io);
+}
+
+}  // namespace thin
+
+static const GemmParams& gp_of(const Launch& L) { return *reinterpret_cast<const GemmParams*>(L.blob.data()); }
+
+// From 4096 rows on (fewer are for the one-tile-per-CTA kernels).  K up to 128 at N = 4 (262144 x 128 x 4: 29.6 on split-TF32,
+// 27.6 here) and up to 32 at N = 8: past that the reads of the weights bind this kernel (524288 x 64 x 8: 32.5 against 38.6).
+bool conv_thin_eligible(const GemmParams& gp) {
+  if (plan_flag(DNNF_PLAN_NO_SMALL_CONV)) return false;
+  if ((gp.N != 4 && gp.N != 8) || gp.K % 4 || gp.K > (gp.N == 4 ? 128 : 32) || gp.M < 4096) return false;
+  if (gp.A.dtype != 0 || gp.B.dtype != 0) return false;
+  if (gp.batch_ext[0] * gp.batch_ext[1] != 1) return false;
+  if (gp.A.stride_col != 1 || gp.A.stride_row % 4 || gp.A.base % 4) return false;
+  if (gp.B.stride_col != 1 || gp.B.stride_row != gp.N || gp.B.base % 4) return false;
+  if (gp.n_nd != 1 || gp.m_nd != 1 || gp.b_nd != 1) return false;
+  // the chain reads and writes four neighbouring columns: 16-byte aligned wherever it walks along n
+  auto quad_ok = [](const TensorArg& a) { return a.dtype == 0 && (a.stride[0] == 0 || (a.stride[0] == 1 && a.base % 4 == 0 && a.stride[1] % 4 == 0)); };
+  for (int i = 0; i < gp.n_in; ++i) if (!quad_ok(gp.in[i]) || gp.in[i].mode == 2) return false;
+  for (int i = 0; i < gp.n_out; ++i) if (!quad_ok(gp.out[i]) || gp.out[i].stride[0] != 1) return false;
+  return true;
+}
+
+void conv_thin_plan(Launch& L) {
+  GemmParams& gp = *reinterpret_cast<GemmParams*>(L.blob.data());
+  L.variant = 9;
+  L.threads = thin::THREADS;
+  L.smem = (size_t)(((gp.K + 15) & ~15) / 4) * (4 * gp.N + 4) * 4;
+  const int rows = thin::ROWS * (thin::THREADS / 32);
+  L.grid = (gp.M + rows - 1) / rows;
+  L.static_id = StaticSet<ConvStatic>::find(gp.prog);
+}
+
+namespace {
+struct ThinLauncher {
+  const Launch& L; cudaStream_t st;
+  template <class SP> void run() {
+    if (gp_of(L).N == 4) launch_pdl(thin::conv_thin_kernel<4, SP>, L.grid, thin::THREADS, L.smem, st, gp_of(L));
+    else launch_pdl(thin::conv_thin_kernel<8, SP>, L.grid, thin::THREADS, L.smem, st, gp_of(L));
+  }
+};
+}  // namespace
+
+int conv_thin_launch(const Launch& L, cudaStream_t st) {
+  ThinLauncher F{L, st};
+  if (!(L.static_id > 0 && StaticSet<ConvStatic>::dispatch(L.static_id, F))) F.run<DynProg>();
+  return cudaGetLastError() == cudaSuccess ? 0 : 1;
+}
+
+}  // namespace dnnf

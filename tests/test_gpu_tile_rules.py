@@ -174,6 +174,26 @@ def test_head_merge_after_a_product_with_unit_dims_is_store_indexing(batch, head
     assert len([b for b in s.g.blocks() if b["family"] != "alias"]) == 1
 
 
+@pytest.mark.parametrize("mkn", [(4096, 4, 4), (4103, 16, 4), (8200, 20, 8), (4097, 32, 8), (5000, 128, 4)])
+@pytest.mark.parametrize("epi", ["none", "bias_tanh", "residual"])
+def test_thin_result_kernel(mkn, epi):
+    """fp32 products four or eight columns wide: rows that fill no warp, K that fills no round of the four lanes."""
+    m, k, n = mkn
+    g = graph()
+    g.ext("X", (m, k)); g.ext("Wt", (k, n), kind="weight")
+    ins = {"X": rnd((m, k), 970, -1, 1), "Wt": rnd((k, n), 971, -0.5, 0.5)}
+    t = g.add("MatMul", ["X", "Wt"])
+    if epi == "bias_tanh":
+        g.ext("b", (n,)); ins["b"] = rnd((n,), 972)
+        t = g.add("Tanh", [g.add("Add", [t, "b"])])
+    if epi == "residual":
+        g.ext("R", (m, n)); ins["R"] = rnd((m, n), 973, -1, 1)
+        t = g.add("Add", [t, "R"])
+    g.mark_output(t)
+    s = check(W.Workload(g, ins), RTOL_F32, FUSED, expect_blocks=1)
+    assert s.g.blocks()[0]["variant"] == 9
+
+
 @pytest.mark.parametrize("cfg", [(32, 14, 14, 384), (2, 56, 56, 144), (40, 7, 9, 960), (1, 120, 33, 100), (64, 15, 16, 20)])
 def test_dwconv_tiles_of_rows_columns_and_channel_blocks(cfg):
     n, h, w, c = cfg
