@@ -56,18 +56,6 @@ struct Params {
 };
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// Wait for the tensor-memory loads issued so far.  The loaded registers are named as read-write operands: without that
-// the compiler sees no dependence between the wait and later arithmetic on them, and may schedule that arithmetic
-// ahead of the wait when other work (the mask loads) sits between the load's issue and the wait.
-__device__ __forceinline__ void tc_ld_wait32(uint32_t (&r)[32]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]),
-                 "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]),
-                 "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]),
-                 "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-               :: "memory");
-}
-
 __device__ __forceinline__ float fast_exp2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
 template <int NC>
@@ -232,7 +220,7 @@ attention_kernel(const __grid_constant__ GemmParams pA, const __grid_constant__ 
         uint32_t raw[32];
         if (col0 + ch * 32 < sk16) {                       // (uniform over the warp)
           tc_ld32_issue(t_row + col0 + ch * 32, raw);
-          tc_ld_wait32(raw);
+          tc_ld_wait(raw);
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             const float v = fmaf(__uint_as_float(raw[j]), c, x[ch * 32 + j]);
@@ -291,7 +279,7 @@ attention_kernel(const __grid_constant__ GemmParams pA, const __grid_constant__ 
       for (int c0 = half * (D >> 1); c0 < (half + 1) * (D >> 1); c0 += 32) {
         uint32_t raw[32];
         tc_ld32_issue(t_row + q.o_col + c0, raw);
-        tc_ld_wait32(raw);
+        tc_ld_wait(raw);
         if (row_ok) {
 #pragma unroll
           for (int pc = 0; pc < 4; ++pc) {

@@ -31,7 +31,7 @@ namespace dnnf {
 namespace dwt {
 
 constexpr int THREADS = 256;
-constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // 1 s
+constexpr int kWaitPolls = 1 << 18;
 
 struct Params {
   CUtensorMap tmX;           // dims (C, W, H, N), box (cb, wt + 2, ht + 2, 1), no swizzle
@@ -55,16 +55,11 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ unsigned long long wall_ns() { unsigned long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
-// Bounded wait: false when the bound ran out (the caller records the failure and leaves).
+// Bounded wait: false when the polls ran out, a second at 4 us each (the caller records the failure and leaves).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = wall_ns();
-  for (;;) {
 #pragma unroll 1
-    for (int i = 0; i < 64; ++i) if (mbar_try(bar, parity)) return true;
-    if (wall_ns() - t0 > kWaitLimitNs) return false;
-  }
+  for (int i = 0; i < kWaitPolls; ++i) if (mbar_try(bar, parity)) return true;
+  return false;
 }
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, uint64_t* bar, int c0, int c1, int c2, int c3) {
   asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"

@@ -133,19 +133,21 @@ gemm_tc_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Gem
       if (!__all_sync(0xffffffffu, mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag))) { ok = false; break; }
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+      uint32_t accumulate = 0u;
       for (int kt = 0; kt < k_tiles; ++kt) {
         if (!__all_sync(0xffffffffu, mbar_wait(&full_bar[s], ph, abort_flag))) { ok = false; break; }
         // (no tcgen05 fence: TMA wrote the operands and the barrier orders its completion before the MMAs' reads)
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < TC_BK / 16; ++kk)
-            tc_mma_bf16(d_tmem, da_s + 2 * kk, db_s + dbk * kk, idesc, (kt | kk) ? 1u : 0u);
+            tc_mma_bf16(d_tmem, da_s + 2 * kk, db_s + dbk * kk, idesc, kk ? 1u : accumulate);
           tc_commit(&empty_bar[s]);          // frees the smem stage once these MMAs have read it
-          if (kt + 1 == k_tiles) tc_commit(&tfull_bar[acc]);   // accumulator complete
         }
+        accumulate = 1u;
         da_s += dstage; db_s += dstage;
         if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
       }
+      if (ok && elect_one()) tc_commit(&tfull_bar[acc]);   // accumulator complete
     }
   } else {
     // ---------------- epilogue warps ----------------
@@ -185,14 +187,12 @@ gemm_tc_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Gem
       for (int c = c_begin; c < c_end; c += 32) {
         const int n0 = tn * BN + c;
         if (n0 >= p.N) break;                  // uniform across the warp
-        if (q.debug & 4) continue;
         uint32_t raw[32];
         if (tcount == 0 && warp == 2 && lane == 0 && c == c_begin) TRACE(8);
         tc_ld32_issue(t_row + c, raw);
-        tc_ld_wait();
+        tc_ld_wait(raw);
         if (tcount == 0 && warp == 2 && lane == 0 && c == c_begin) TRACE(9);
         // transpose: lane = row  ->  lane = (row group, 4-column piece)
-        if (!(q.debug & 2)) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) stage[lane * 33 + j] = raw[j];
         __syncwarp();
@@ -201,10 +201,9 @@ gemm_tc_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Gem
 #pragma unroll
           for (int e = 0; e < 4; ++e) io.accv[i * 4 + e] = __uint_as_float(stage[((lane >> 3) + 4 * i) * 33 + (lane & 7) * 4 + e]);
         __syncwarp();
-        }
         if (tcount == 0 && warp == 2 && lane == 0 && c == c_begin) TRACE(10);
         io.n0 = (uint32_t)n0;
-        if (!(q.debug & 1)) run_program<32, SP, true>(p.prog, io);
+        run_program<32, SP, true>(p.prog, io);
         if (tcount == 0 && warp == 2 && lane == 0 && c == c_begin) TRACE(11);
       }
       tc_fence_before();
@@ -301,7 +300,6 @@ void tc_gemm_plan(Launch& L) {
   L.smem = (size_t)stages * stage_bytes + kSmemFixed;
   L.variant = 1;
   L.static_id = StaticSet<EpiStatic>::find(gp.prog);
-  tc.debug = dev_env("DNNF_GEMM_DEBUG") ? atoi(dev_env("DNNF_GEMM_DEBUG")) : 0;
 }
 
 // dims innermost first: {inner, outer, b0, b1}

@@ -336,7 +336,7 @@ gemm_tc2_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Pa
         for (int c = 0; c < chunks; ++c) {
           uint32_t raw[32];
           tc_ld32(t_row + c * 32, raw);
-          tc_ld_wait();
+          tc_ld_wait(raw);
 #pragma unroll
           for (int i = 0; i < 32; ++i) mine[(c * 32 + i) * 32 + lane] = __uint_as_float(raw[i]);     // a 128-byte line per instruction
         }
@@ -371,7 +371,7 @@ gemm_tc2_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Pa
         } else {
           uint32_t raw[32];
           tc_ld32(t_row + c * 32, raw);
-          tc_ld_wait();
+          tc_ld_wait(raw);
 #pragma unroll
           for (int i = 0; i < 32; ++i) io.accv[i] = __uint_as_float(raw[i]);
         }

@@ -55,8 +55,10 @@ namespace tf32 {
 #endif
 #ifdef DNNF_TRACE
 #define FACC(slot, v) do { if (blockIdx.x == 0 && p.status) atomicAdd(reinterpret_cast<unsigned long long*>(p.status) + 4 + (slot), (unsigned long long)(v)); } while (0)
+#define CLK() clock64()
 #else
 #define FACC(slot, v) do {} while (0)
+#define CLK() 0ll                              // (a read of the clock stays in the code even where its value is not used)
 #endif
 
 constexpr int EPI_WARPS = 8, CONV_WARPS = 4, THREADS = 64 + 32 * (EPI_WARPS + CONV_WARPS);
@@ -93,7 +95,6 @@ struct Params {
   int32_t dual;              // A_hi x [B_hi | B_lo] in one MMA (two accumulator ranges)
   int32_t b_dense;           // B is a dense row-major [K x N] block: fetched with one bulk copy
   int32_t fast_epi;          // the fast epilogue form applies
-  int32_t debug;             // ablation switches (development only)
   int32_t epi_bytes;         // chunk buffers / transpose staging / raw B
   int32_t chunks_per_warp;   // fast epilogue: chunk buffers of one warp
   FastDiv fd_n, fd_npad, fd_kpad;   // element index of B -> (k, n)
@@ -101,26 +102,6 @@ struct Params {
   int8_t slot[kMaxIn];       // fast form: staged-vector slot of epilogue input i, or -1 for a dense operand
 };
 
-#ifdef DNNF_TF32_POLL
-// non-suspending poll
-__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
-               : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_poll(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_test(bar, parity)) return true;
-  const unsigned long long t0 = wall_ns();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 256; ++i) if (mbar_test(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (wall_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; return false; }
-  }
-}
-#define mbar_wait mbar_wait_poll
-#endif
 // Fast epilogue IO: a lane owns 32 consecutive columns [c, c+32) of its own row.
 struct RowEpiIO {
   static constexpr int VV = 32;
@@ -244,7 +225,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int n_epi = q.epi_warps, conv_sets = (EPI_WARPS + CONV_WARPS - n_epi) / 4;   // converter sets take chunks in turn
   const int rb = q.rb, units = BM / rb;                            // a raw block holds rb rows; `units` blocks per tile
-  const long long t_begin = clock64();
+  const long long t_begin = CLK();
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(&raw_bar[s], 1); mbar_init(&empty_bar[s], (uint32_t)(rb / 32 * conv_sets)); }
     for (int s = 0; s < a_stages; ++s) { mbar_init(&conv_bar[s], 4); mbar_init(&afree_bar[s], 1); }
@@ -278,7 +259,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     bool ok = true;
     for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
       for (int u = 0; u < units; ++u) {
-        { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph ^ 1, abort_flag))) { ok = false; break; } if (lane == 0) FACC(1, clock64() - t0); }
+        { long long t0 = CLK(); if (!__all_sync(0xffffffffu, mbar_wait(&empty_bar[s], ph ^ 1, abort_flag))) { ok = false; break; } if (lane == 0) FACC(1, CLK() - t0); }
         if (elect_one()) {
           mbar_expect_tx(&raw_bar[s], (uint32_t)(rb * q.pitch * 4));
           tma_load_2d(ring + (size_t)s * q.unit_stride, &q.tmA, &raw_bar[s], 0, tile * BM + u * rb);
@@ -353,7 +334,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     }
     fence_async_smem();
     asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
-    if (tid == 0) FACC(0, clock64() - t_begin);
+    if (tid == 0) FACC(0, CLK() - t_begin);
   }
 
   if (warp == 1) {
@@ -370,23 +351,22 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++tcount) {
       const int acc = tcount & 1;
       const uint32_t aph = (tcount >> 1) & 1;
-      { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag))) { ok = false; break; } if (lane == 0) FACC(2, clock64() - t0); }
+      { long long t0 = CLK(); if (!__all_sync(0xffffffffu, mbar_wait(&tempty_bar[acc], aph ^ 1, abort_flag))) { ok = false; break; } if (lane == 0) FACC(2, CLK() - t0); }
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * acc_cols);
-      const long long t_tile = clock64();
+      const long long t_tile = CLK();
       uint64_t dbh = db0;
       int k_left = p.K;
       for (int kc = 0; kc < k_chunks; ++kc, k_left -= BK, dbh += atom_bytes >> 4) {
-        { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&conv_bar[s], ph, abort_flag))) { ok = false; break; } if (lane == 0) FACC3(3, clock64() - t0); }
+        { long long t0 = CLK(); if (!__all_sync(0xffffffffu, mbar_wait(&conv_bar[s], ph, abort_flag))) { ok = false; break; } if (lane == 0) FACC3(3, CLK() - t0); }
         tc_fence_after();
-        const long long t_issue = clock64();
+        const long long t_issue = CLK();
         const int ksteps = min(BK, k_left + 7) >> 3;                   // 8 tf32 per MMA
         const uint32_t a_hi = tmem_base + a_cols0 + (uint32_t)(s * kAStageCols), a_lo = a_hi + BK;
         // B descriptors advance by 32 bytes (2 units of 16) per k-step inside the swizzled atom
         const uint64_t dbl = dbh + (lo_off >> 4);
         if (elect_one()) {
-          if (q.debug & 2) {
-          } else if (dual) {
+          if (dual) {
 #pragma unroll
             for (int kk = 0; kk < BK / 8; ++kk) {
               if (kk < ksteps) {
@@ -405,14 +385,14 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
             }
           }
           tc_commit(&afree_bar[s]);          // frees the A stage once these MMAs have read it
-          if (kc + 1 == k_chunks) tc_commit(&tfull_bar[acc]);  // accumulator complete
         }
         if (++s == a_stages) { s = 0; ph ^= 1; }
-        if (lane == 0) FACC3(4, clock64() - t_issue);
+        if (lane == 0) FACC3(4, CLK() - t_issue);
       }
-      if (lane == 0) FACC(10, clock64() - t_tile);
+      if (ok && elect_one()) tc_commit(&tfull_bar[acc]);       // accumulator complete
+      if (lane == 0) FACC(10, CLK() - t_tile);
     }
-    if (lane == 0) FACC(11, clock64() - t_begin);
+    if (lane == 0) FACC(11, CLK() - t_begin);
   } else if (warp >= 2 && warp < 2 + n_epi) {
     // ---------------- epilogue warps ----------------
     const int sub = warp & 3;                 // TMEM sub-partition this warp may read
@@ -423,10 +403,9 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++tcount) {
       const int acc = tcount & 1;
       const uint32_t aph = (tcount >> 1) & 1;
-      { long long t0 = clock64(); if (!mbar_wait(&tfull_bar[acc], aph, abort_flag)) { ok = false; break; } if (warp == 2 && lane == 0) FACC(5, clock64() - t0); }
-      const long long t_epi = clock64();
+      { long long t0 = CLK(); if (!mbar_wait(&tfull_bar[acc], aph, abort_flag)) { ok = false; break; } if (warp == 2 && lane == 0) FACC(5, CLK() - t0); }
+      const long long t_epi = CLK();
       tc_fence_after();
-      if (q.debug & 4) { __syncwarp(); if (lane == 0) mbar_arrive(&tempty_bar[acc]); continue; }
       const uint32_t t_row = tmem_base + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * acc_cols);
       bool released = false;
       if (kFast) {
@@ -439,8 +418,8 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
         // One chunk buffer per 32-column chunk of this warp: the tile's stores are issued together at its end, and the
         // wait for the buffers (the previous tile's stores have read them) comes a whole tile after they were issued.
         // (With two buffers per warp, every chunk waited for the store of two chunks earlier: 1100 cycles per chunk.)
-        { const long long t0 = clock64(); if (lane == 0) tma_store_wait_read0();
-        __syncwarp(); if (warp == 2 && lane == 0) FACC(14, clock64() - t0); }
+        { const long long t0 = CLK(); if (lane == 0) tma_store_wait_read0();
+        __syncwarp(); if (warp == 2 && lane == 0) FACC(14, CLK() - t0); }
         uint8_t* my_chunks = epi + (size_t)(warp - 2) * q.chunks_per_warp * kChunkBytes;
         int slot = 0;
         if (p.N <= 8) {                                   // one narrow chunk (cgroup 0 only: four epilogue warps)
@@ -448,12 +427,12 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
           io8.lane = lane; io8.vec_s = vec_s; io8.row_ok = io.row_ok; io8.row = io.row;
           uint32_t raw[8];
           tc_ld8_issue(t_row, raw);
-          tc_ld_wait();
+          tc_ld_wait(raw);
 #pragma unroll
           for (int j = 0; j < 8; ++j) io8.accv[j] = __uint_as_float(raw[j]);
           for (int r = 1; r < nranges; ++r) {
             tc_ld8_issue(t_row + r * NP, raw);
-            tc_ld_wait();
+            tc_ld_wait(raw);
 #pragma unroll
             for (int j = 0; j < 8; ++j) io8.accv[j] += __uint_as_float(raw[j]);
           }
@@ -462,22 +441,22 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
         } else
         for (int c = cgroup * 32; c < n_here; c += cstep, ++slot) {
           uint32_t raw[32];
-          const long long t0 = clock64();
+          const long long t0 = CLK();
           tc_ld32_issue(t_row + c, raw);
-          tc_ld_wait();
+          tc_ld_wait(raw);
 #pragma unroll
           for (int j = 0; j < 32; ++j) io.accv[j] = __uint_as_float(raw[j]);
           for (int r = 1; r < nranges; ++r) {
             tc_ld32_issue(t_row + r * NP + c, raw);
-            tc_ld_wait();
+            tc_ld_wait(raw);
 #pragma unroll
             for (int j = 0; j < 32; ++j) io.accv[j] += __uint_as_float(raw[j]);
           }
-          const long long t1 = clock64();
+          const long long t1 = CLK();
           io.c = c; io.n = n_base + c;
           io.chunk = my_chunks + slot * kChunkBytes;
           run_program<32, SP, false>(p.prog, io);
-          if (warp == 2 && lane == 0) { FACC(12, t1 - t0); FACC(13, clock64() - t1); }
+          if (warp == 2 && lane == 0) { FACC(12, t1 - t0); FACC(13, CLK() - t1); }
         }
         // the accumulator stage is free as soon as it has been read
         tc_fence_before();
@@ -512,11 +491,11 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
         for (int c = cgroup * 32; c < n_here; c += cstep) {
           uint32_t raw[32];
           tc_ld32_issue(t_row + c, raw);
-          tc_ld_wait();
+          tc_ld_wait(raw);
           for (int r = 1; r < nranges; ++r) {
             uint32_t raw2[32];
             tc_ld32_issue(t_row + r * NP + c, raw2);
-            tc_ld_wait();
+            tc_ld_wait(raw2);
 #pragma unroll
             for (int j = 0; j < 32; ++j) raw[j] = __float_as_uint(__uint_as_float(raw[j]) + __uint_as_float(raw2[j]));
           }
@@ -538,7 +517,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
         __syncwarp();
         if (lane == 0) mbar_arrive(&tempty_bar[acc]);
       }
-      if (warp == 2 && lane == 0) FACC(6, clock64() - t_epi);
+      if (warp == 2 && lane == 0) FACC(6, CLK() - t_epi);
     }
     if (kFast && lane == 0) tma_store_wait_all();     // shared memory must outlive the last stores' reads
     (void)nstore;
@@ -555,7 +534,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     int as = 0, turn = 0; uint32_t aph = 0;
     for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step) {
       // (votes keep the warp together: the tensor-memory stores below are warp-wide)
-      { long long t0 = clock64(); if (!__all_sync(0xffffffffu, mbar_wait(&raw_bar[s], rph, abort_flag))) { ok = false; break; } if (warp == 13 && lane == 0) FACC(7, clock64() - t0); }
+      { long long t0 = CLK(); if (!__all_sync(0xffffffffu, mbar_wait(&raw_bar[s], rph, abort_flag))) { ok = false; break; } if (warp == 13 && lane == 0) FACC(7, CLK() - t0); }
       const float4* src = reinterpret_cast<const float4*>(ring + (size_t)s * q.unit_stride) + row * pieces;
       for (int kc = 0; kc < k_chunks; ++kc) {
         const bool mine = turn == set;
@@ -565,41 +544,38 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
           if (++as == a_stages) { as = 0; aph ^= 1; }
           continue;
         }
-        const long long t_cv = clock64();
+        const long long t_cv = CLK();
         uint32_t hi[32], lo[32];
-        if (!(q.debug & 1)) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int pc = kc * 8 + j;
-            const float4 x = pc < pieces ? src[pc] : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float xs[4] = {x.x, x.y, x.z, x.w};
+        for (int j = 0; j < 8; ++j) {
+          const int pc = kc * 8 + j;
+          const float4 x = pc < pieces ? src[pc] : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float xs[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              // hi = x cut to TF32 precision by a mask, lo = x - hi (exact in fp32); the tensor core reads the upper 19
-              // bits of lo, i.e. cuts it once more: |a - (hi + lo')| < 2^-20 |a|.  Two full-rate instructions per value
-              // instead of two conversions and a subtraction (7 % of the 144 -> 24 block's time).
-              const uint32_t hb = __float_as_uint(xs[e]) & 0xffffe000u;
-              hi[4 * j + e] = hb;
-              lo[4 * j + e] = __float_as_uint(xs[e] - __uint_as_float(hb));
-            }
+          for (int e = 0; e < 4; ++e) {
+            // hi = x cut to TF32 precision by a mask, lo = x - hi (exact in fp32); the tensor core reads the upper 19
+            // bits of lo, i.e. cuts it once more: |a - (hi + lo')| < 2^-20 |a|.  Two full-rate instructions per value
+            // instead of two conversions and a subtraction (7 % of the 144 -> 24 block's time).
+            const uint32_t hb = __float_as_uint(xs[e]) & 0xffffe000u;
+            hi[4 * j + e] = hb;
+            lo[4 * j + e] = __float_as_uint(xs[e] - __uint_as_float(hb));
           }
         }
-        if (kc == k_chunks - 1) {                                // the raw block is in registers
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&empty_bar[s]);
-        }
         if (!__all_sync(0xffffffffu, mbar_wait(&afree_bar[as], aph ^ 1, abort_flag))) { ok = false; break; }
-        if (!(q.debug & 1)) {
-          tc_fence_after();
-          const uint32_t t_a = tmem_base + ((uint32_t)(sub * 32) << 16) + a_cols0 + (uint32_t)(as * kAStageCols);
-          tc_st32(t_a, hi);
-          tc_st32(t_a + BK, lo);
-          tc_st_wait();
-          tc_fence_before();
-        }
+        tc_fence_after();
+        const uint32_t t_a = tmem_base + ((uint32_t)(sub * 32) << 16) + a_cols0 + (uint32_t)(as * kAStageCols);
+        tc_st32(t_a, hi);
+        tc_st32(t_a + BK, lo);
+        tc_st_wait();
+        tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&conv_bar[as]);
-        if (warp == 13 && lane == 0) FACC(8, clock64() - t_cv);
+        if (lane == 0) {
+          // The raw block is free once its values have been USED: a shared-memory load that was issued before the arrival may still
+          // wait behind the residual's global loads when the next block lands (rows of two blocks were seen mixed).
+          if (kc == k_chunks - 1) mbar_arrive(&empty_bar[s]);
+          mbar_arrive(&conv_bar[as]);
+        }
+        if (warp == 13 && lane == 0) FACC(8, CLK() - t_cv);
         if (++as == a_stages) { as = 0; aph ^= 1; }
       }
       s += units;
@@ -611,7 +587,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   __syncwarp();
   tc_fence_before();
   __syncthreads();
-  if (threadIdx.x == 0) FACC(9, clock64() - t_begin);
+  if (threadIdx.x == 0) FACC(9, CLK() - t_begin);
   if (*abort_flag) {
     if (threadIdx.x == 0 && p.status) { atomicExch(&p.status[0], DNNF_ERR_TIMEOUT); atomicExch(&p.status[1], p.block_index); }
     // give copies that are still in flight time to land before shared memory is released
@@ -693,7 +669,6 @@ void tf32_gemm_plan(Launch& L) {
   L.early_reads = gp.static_mask != 0;
   q.fd_n = make_fastdiv((uint32_t)gp.N); q.fd_npad = make_fastdiv((uint32_t)q.npad); q.fd_kpad = make_fastdiv((uint32_t)(q.k_chunks * tf32::BK));
   q.epi_warps = (PN <= 32 && !dev_env("DNNF_TF32_EPI8")) ? 4 : 8;
-  q.debug = dev_env("DNNF_TF32_DEBUG") ? atoi(dev_env("DNNF_TF32_DEBUG")) : 0;
   gp.tiles_m = (gp.M + tf32::BM - 1) / tf32::BM;
   gp.tiles_n = parts;
   q.total_tiles = gp.tiles_m;
@@ -709,7 +684,9 @@ void tf32_gemm_plan(Launch& L) {
   const int ring_budget = tf32::kSmemMax - fixed - tf32_b_bytes_of(PN, gp.K);
   q.rb = 32;                                                 // one block per converter warp
   q.unit_stride = (q.rb * q.pitch * 4 + 1023) / 1024 * 1024;
-  q.stages = std::min(tf32::kMaxStages, ring_budget / q.unit_stride);
+  // A multiple of a tile's four blocks: a stage then always holds the same converter warp's rows.  With any other count a warp could
+  // come to a stage whose last block, another warp's, had not landed yet, and take the phase before that for its own.
+  q.stages = std::min(tf32::kMaxStages, ring_budget / q.unit_stride) / 4 * 4;
   q.a_stages = std::min(6, (512 - 2 * (q.dual ? 2 : 1) * q.npad) / tf32::kAStageCols);
   L.smem = (size_t)tf32_b_bytes_of(PN, gp.K) + (size_t)q.stages * q.unit_stride + fixed;
   q.b_dense = parts == 1 && gp.B.stride_col == 1 && gp.B.stride_row == gp.N && gp.N % 4 == 0 && gp.B.base % 4 == 0 &&

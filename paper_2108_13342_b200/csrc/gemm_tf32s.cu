@@ -257,16 +257,15 @@ gemm_tf32s_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ 
 #pragma unroll
           for (int e = 0; e < 4; ++e) lo[4 * j + e] = __float_as_uint(xs[e] - __uint_as_float(__float_as_uint(xs[e]) & 0xffffe000u));
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&rfree_bar[rs]);
-        if (++rs == raw_stages) { rs = 0; rph ^= 1; }
         if (!__all_sync(0xffffffffu, mbar_wait(&free_bar[s], ph ^ 1, abort_flag))) break;
         tc_fence_after();
         tc_st32(t_lane + (uint32_t)(s * BK), lo);
         tc_st_wait();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&conv_bar[s]);
+        // (the raw tile is released when its values have been used: a load that was only issued may come after the next tile)
+        if (lane == 0) { mbar_arrive(&rfree_bar[rs]); mbar_arrive(&conv_bar[s]); }
+        if (++rs == raw_stages) { rs = 0; rph ^= 1; }
         if (++s == stages) { s = 0; ph ^= 1; }
       }
     } else {
@@ -294,9 +293,6 @@ gemm_tf32s_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ 
 #pragma unroll
               for (int e = 0; e < 4; ++e) v[i][e] = src[i * kstride + e * BN];
           }
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&rfree_bar[rs]);
-          if (++rs == raw_stages) { rs = 0; rph ^= 1; }
           if (!__all_sync(0xffffffffu, mbar_wait(&free_bar[s], ph ^ 1, abort_flag))) break;
           const uint32_t hi_off = (chain & 1) ? lo_off : 0u;         // (an odd chain has the lo image in front)
           uint8_t* bh = smem + (size_t)s * b_stage;
@@ -314,7 +310,8 @@ gemm_tf32s_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ 
           }
           fence_async_smem();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&conv_bar[s]);
+          if (lane == 0) { mbar_arrive(&rfree_bar[rs]); mbar_arrive(&conv_bar[s]); }
+          if (++rs == raw_stages) { rs = 0; rph ^= 1; }
           if (++s == stages) { s = 0; ph ^= 1; }
           if (++chain == q.chains) chain = 0;
         }
@@ -380,12 +377,12 @@ gemm_tf32s_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ 
         for (int c = half * 32; c < BN && n0 + c < p.N; c += 64) {
           uint32_t r[32];
           tc_ld32_issue(t_row + c, r);                             // (columns past BN are past N as well: never used)
-          tc_ld_wait();
+          tc_ld_wait(r);
 #pragma unroll
           for (int j = 0; j < 32; ++j) stage[lane * 33 + j] = r[j];
           for (int rg = 1; rg < q.ranges; ++rg) {
             tc_ld32_issue(t_row + rg * BN + c, r);
-            tc_ld_wait();
+            tc_ld_wait(r);
 #pragma unroll
             for (int j = 0; j < 32; ++j) stage[lane * 33 + j] = __float_as_uint(__uint_as_float(stage[lane * 33 + j]) + __uint_as_float(r[j]));
           }

@@ -30,6 +30,7 @@ namespace tc2 {
 constexpr int BM = 128, BK = 64, EPI_WARPS = 8, THREADS = 64 + 32 * EPI_WARPS;
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // 1 s
 constexpr int kFastPolls = 2048;                             // polls of a barrier before the wall clock is consulted
+constexpr int kWaitPolls = 1 << 18;
 constexpr int kSmemMax = 227 * 1024;
 constexpr int kBiasFloats = 128;                             // per warp, per row-invariant operand
 constexpr int kMaxVec = 2;                                   // row-invariant operands staged in shared memory
@@ -65,21 +66,13 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 __device__ __forceinline__ unsigned long long wall_ns() { unsigned long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
-// Bounded wait: gives up after kWaitLimitNs of wall-clock time (or as soon as another role of the
-// CTA gave up), sets the CTA's abort flag and returns false.
+// Bounded wait: false, with the CTA's abort flag set, once the polls ran out.  A poll that fails has been suspended for 4 us by
+// the hardware, so kWaitPolls of them are a second; nothing else stands in the loop (tc_common.cuh says what it would cost).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try(bar, parity)) return true;
-  // Fast phase: the common case is a wait of well under a microsecond.  Reading the global timer costs about as much
-  // as a whole pipeline step of the issuing threads, so the clock is consulted only after this many polls.
 #pragma unroll 1
-  for (int i = 0; i < kFastPolls; ++i) if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = wall_ns();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 64; ++i) if (mbar_try(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (wall_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; return false; }
-  }
+  for (int i = 0; i < kWaitPolls; ++i) if (mbar_try(bar, parity)) return true;
+  *abort_flag = 1;
+  return false;
 }
 // Operand load of a CTA pair: the bytes land in THIS CTA's shared memory, the completion is
 // counted on the LEADER's barrier (cluster address), so the MMA thread waits on one barrier only.
@@ -118,7 +111,14 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
                  "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
                : "r"(taddr));
 }
-__device__ __forceinline__ void tc_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// (the loaded registers are operands of the wait: no arithmetic on them may move in front of it)
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                 "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) :: "memory");
+}
 
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
   uint64_t d = 0;

@@ -12,7 +12,6 @@
 
 namespace dnnf {
 
-constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // 1 s
 constexpr int kStageWords = 32 * 33;                       // per epilogue warp: 32 rows x (32 + 1 pad) words
 
 // ---- PTX wrappers -------------------------------------------------------------------------
@@ -33,19 +32,16 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded wait.  Returns false when the bound ran out or another role already gave up.
-__device__ __forceinline__ unsigned long long wall_ns() { unsigned long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
-// Bounded wait: gives up after kWaitLimitNs of wall-clock time (or as soon as another role of the
-// CTA gave up), sets the CTA's abort flag and returns false.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, unsigned long long limit_ns = kWaitLimitNs) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = wall_ns();
-  for (;;) {
+// Bounded wait: false, with the CTA's abort flag set, once the polls ran out.  A poll that fails has been suspended for 4 us by
+// the hardware (measured on a barrier nobody signals, with any hint), so kWaitPolls of them are a second.  Nothing else stands in
+// the loop: with a look at the timer and at the abort flag inlined into every wait (or a call to such code), the warp that issues
+// the MMAs of a 128 x 64 tile took 390 instead of 280 cycles per k-tile.
+constexpr int kWaitPolls = 1 << 18;
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int polls = kWaitPolls) {
 #pragma unroll 1
-    for (int i = 0; i < 64; ++i) if (mbar_try(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (wall_ns() - t0 > limit_ns) { *abort_flag = 1; return false; }
-  }
+  for (int i = 0; i < polls; ++i) if (mbar_try(bar, parity)) return true;
+  *abort_flag = 1;
+  return false;
 }
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, uint64_t* bar, int c0, int c1, int c2, int c3) {
   asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
@@ -78,7 +74,24 @@ __device__ __forceinline__ void tc_ld8_issue(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr));
 }
-__device__ __forceinline__ void tc_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// Wait for the tensor-memory loads issued so far.  The loaded registers are operands of the wait: without that the compiler sees no
+// dependence between it and arithmetic on them, and may place that arithmetic (a scale next to its load) in front of the wait.
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]) :: "memory");
+}
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]) :: "memory");
+}
+__device__ __forceinline__ void tc_ld_wait(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                 "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]) :: "memory");
+}
 
 // Shared-memory matrix descriptor (sm_100 format: version 1, 128-byte swizzle).
 //  K-major tile  [rows][64 bf16]: rows 128 B apart, 8-row groups 1024 B apart (SBO); LBO unused.
