@@ -18,12 +18,15 @@
 // columns at a time -> bf16 -> swizzled 32 x 32 chunk -> TMA store.  With four warps and 32 columns at a time the epilogue
 // was the longer half of these kernels: 248 x 2304 x 768 + bias 6.1 -> 5.4 us, 248 x 768 x 768 5.5 -> 4.8, 248 x 3072 x 768 +
 // GELU 6.8 -> 6.0, 1024 x 768 x 768 6.0 -> 5.4.
+// Tile widths: 64, 128 or 192 columns, by counted time (tile_us): a k-tile costs a CTA 0.145, 0.2 or 0.235 us, so wide tiles are for
+// the problems whose narrow ones would share SMs (1024 x 3072 x 768 + GELU: 192 tiles of 128 columns 10.8 us, 128 of 192 8.9).
+// The issuer's and the producers' loops hold nothing but their wait, their requests and their commit: conditional commits, a branch
+// on B's order, and the timer and abort flag inside the wait made a k-tile of 64 columns cost 500 cycles instead of 280
+// (1024 x 768 x 3072 unsplit 12.4 -> 10.0 us, 248 x 768 x 768 5.2 -> 4.6).  The k-tiles of a weight beyond the ring go into L2 before
+// the wait on the previous kernel: in a chain of layers the weights come from DRAM (twelve decoder layers 600 -> 568 us).
 // Long K, few tiles: the k-tiles of a tile are shared by three or four CTAs that meet in the workspace (kMode 2): every epilogue
-// warp writes its partial sums to scratch and bumps its part's counter; the warp whose bump is the last adds all slices in
-// slice order and finishes.  Nobody waits for anybody, no cluster is launched, and the set-up of the CTAs overlaps the previous
-// kernel: 248 x 768 x 3072 14.0 (one CTA per tile) -> 10.5 us, 1024 x 768 x 3072 13.7 (CTA pairs) -> 12.9.  About 5 us of that is the hand-over (write,
-// fence, counter, read back in two rounds); 128-column tiles (16.5 us) or more slices (18.6 us with 4) lose, reading the
-// partial sums as float4, three slices at once, costs more registers than the 80 a thread has here (14.8 us).
+// warp hands its partial sums over, the last to arrive fetches the others' with one bulk copy per slice into the idle operand ring
+// and adds all in slice order.  248 x 768 x 3072: 14.0 us as one CTA per tile, 10.5 with plain loads of all slices, 8.5 now.
 // Every wait is bounded; on expiry the CTA records DNNF_ERR_TIMEOUT and releases tensor memory.
 //
 // Every TMA load in this file is a plain per-CTA load; no clusters are used.
@@ -50,6 +53,7 @@ constexpr int kChunkB = 32 * 64;                                     // 32 rows 
 constexpr int kVecBytes = kEpiWarps * kMaxVec * kBiasFloats * 4;     // staged row-invariant operands, per warp
 constexpr int kBarBytes = 256;
 constexpr int kSmemTwoPerSm = 112 * 1024;                            // two CTAs of this size fit one SM
+constexpr int kSmemOnePerSm = 136 * 1024;                            // three stages of a 192-column tile
 
 struct Params {
   CUtensorMap tmA, tmB, tmD;
@@ -57,6 +61,8 @@ struct Params {
   int32_t c_input;           // index of the epilogue input that is a full tile, or -1
   int32_t stages;
   int32_t tail_off;          // staged vectors, then barriers
+  int32_t b_blocks;          // a row-major B seen as [N / 64 blocks][K][64 columns]: a stage is one request
+  int32_t b_second;          // where 64 does not divide N: one request per 64 columns, two of them
   int32_t b_static;          // B is never written by a kernel of the graph
   int32_t tmem_cols;
   int32_t ksplit, kt_per;    // CTAs that share a tile (a cluster's, or through the workspace) and the k-tiles each of them takes
@@ -82,16 +88,30 @@ __device__ __forceinline__ bool mbar_try_cta(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 __device__ __forceinline__ bool mbar_wait_cta(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_cta(bar, parity)) return true;
 #pragma unroll 1
-  for (int i = 0; i < kFastPolls; ++i) if (mbar_try_cta(bar, parity)) return true;
-  const unsigned long long t0 = wall_ns();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 64; ++i) if (mbar_try_cta(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (wall_ns() - t0 > kWaitLimitNs) { *abort_flag = 1; return false; }
-  }
+  for (int i = 0; i < kWaitPolls; ++i) if (mbar_try_cta(bar, parity)) return true;
+  *abort_flag = 1;
+  return false;
+}
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, uint64_t* bar, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+               ::"r"(smem_u32(dst)), "l"(tm), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2) : "memory");
+}
+// counter += 1, ordered after what this warp has written and before what it reads next
+__device__ __forceinline__ int arrive_acq_rel(int32_t* counter) {
+  int old;
+  asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
+  return old;
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void l2_prefetch_2d(const CUtensorMap* tm, int c0, int c1) {
+  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tm), "r"(c0), "r"(c1) : "memory");
+}
+__device__ __forceinline__ void l2_prefetch_3d(const CUtensorMap* tm, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.prefetch.tensor.3d.L2.global.tile [%0, {%1, %2, %3}];" ::"l"(tm), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
@@ -116,16 +136,16 @@ struct TileIO {
   const GemmParams& p;
   float accv[16];
   uint4 res[2];              // the full-tile operand's 16 values of this row
-  const float* vec_s;        // staged row-invariant operands of this warp: [kMaxVec][kBiasFloats], indexed by tile column
+  const float* vec_s;        // staged row-invariant operands of this warp's columns: [kMaxVec][kBiasFloats]
   uint8_t* chunk;            // chunk buffer of this warp
-  int c_input, col;          // first tile column of the 16
+  int c_input, vcol;         // first of the 16 columns among those staged
   int n;                     // its global column
   int lane, h;               // half of the chunk
   uint32_t out_off;          // element offset of (row, column 0) in the result
   bool row_ok;
   __device__ __forceinline__ void load(int idx, float (&dst)[VV]) const {
     if (idx == c_input) { unpack_bf16(res[0], dst); unpack_bf16(res[1], dst + 8); return; }
-    const float* s = vec_s + p.in[idx].mode * kBiasFloats + col;     // every lane reads the same words: broadcast
+    const float* s = vec_s + p.in[idx].mode * kBiasFloats + vcol;    // every lane reads the same words: broadcast
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       float4 w = *reinterpret_cast<const float4*>(s + 4 * j);
@@ -166,7 +186,9 @@ __device__ __forceinline__ void st_cluster_f4(uint32_t cluster_addr, float4 v) {
 // into CTA j's operand ring (idle by then), and CTA j adds them to its own accumulator, runs the epilogue program on
 // its slice and stores it.  Two cluster barriers frame the exchange: all main loops done (the rings are free), all
 // partial sums written.  The main loop shrinks S-fold, and so does each CTA's epilogue.
-template <class SP, int kMode>          // 0: a CTA per tile, 1: cluster split over K, 2: split over K through the workspace
+// kMode 0: a CTA per tile, 1: cluster split over K, 2: split over K through the workspace.  kBK: B is K-major (a branch on it, or a
+// loop over the boxes of a row-major B, beside the requests costs the producers as much as a request).
+template <class SP, int kMode, bool kBK>
 __global__ void __launch_bounds__(kThreads, 2)
 gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Params q) {
   constexpr bool kSplit = kMode == 1;
@@ -178,7 +200,8 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(tail + kVecBytes);   // [stages] bytes of one stage
   uint64_t* empty_bar = full_bar + 8;         // [stages] 1 arrival (commit)
   uint64_t* tfull_bar = empty_bar + 8;        // accumulator complete
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfull_bar + 1);
+  uint64_t* recv_bar = tfull_bar + 1;         // [epilogue warps] the other slices' partial sums have arrived
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(recv_bar + kEpiWarps);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
@@ -186,6 +209,7 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
     mbar_init(tfull_bar, 1);
+    if (kMode == 2) for (int w = 0; w < kEpiWarps; ++w) mbar_init(&recv_bar[w], 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -217,12 +241,15 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     // ---------------- TMA producers: warp j loads the k-tiles j, j+2, j+4, ... ----------------
     // The whole warp walks the loop, one elected lane issues.  Two producers on alternate k-tiles keep the
     // loads off the critical path: a k-tile of three requests costs its producer about as much as the issuer's four MMAs.
+    const int bx = q.b_blocks ? 0 : n0, bz = q.b_blocks ? n0 >> 6 : 0;
+    const bool second_box = q.b_second != 0;
     auto load_b = [&](int s, int kt) {
       uint8_t* sb = smem + (size_t)s * stage_bytes + a_bytes;
-      if (q.b_kmajor) {
+      if (kBK) {
         tma_load_2d(sb, &q.tmB, &full_bar[s], (kt0 + kt) * BK, n0);
       } else {
-        for (int j = 0; j < BN / 64; ++j) tma_load_2d(sb + j * (64 * BK * 2), &q.tmB, &full_bar[s], n0 + j * 64, (kt0 + kt) * BK);
+        tma_load_3d(sb, &q.tmB, &full_bar[s], bx, (kt0 + kt) * BK, bz);
+        if (second_box) tma_load_3d(sb + 64 * BK * 2, &q.tmB, &full_bar[s], bx + 64, (kt0 + kt) * BK, bz);
       }
     };
     auto load_a = [&](int s, int kt) { tma_load_2d(smem + (size_t)s * stage_bytes, &q.tmA, &full_bar[s], (kt0 + kt) * BK, m0); };
@@ -258,26 +285,28 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     // ---------------- MMA issuer ----------------
     // (No tcgen05 fence inside the loop: the operands were written by TMA, whose completion the barrier itself orders
     // before the MMAs' reads.)
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((q.b_kmajor ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) |
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((kBK ? 0u : 1u) << 16) | ((uint32_t)(BN >> 3) << 17) |
                            ((uint32_t)(BM >> 4) << 24);
     const uint64_t da0 = make_desc(smem_u32(smem), 16, 1024);
-    const uint64_t db0 = q.b_kmajor ? make_desc(smem_u32(smem) + a_bytes, 16, 1024) : make_desc(smem_u32(smem) + a_bytes, 64 * BK * 2, 1024);
-    const uint64_t dstage = stage_bytes >> 4, dbk = q.b_kmajor ? 2 : 128;
+    const uint64_t db0 = kBK ? make_desc(smem_u32(smem) + a_bytes, 16, 1024) : make_desc(smem_u32(smem) + a_bytes, 64 * BK * 2, 1024);
+    const uint64_t dstage = stage_bytes >> 4, dbk = kBK ? 2 : 128;
     uint64_t da_s = da0, db_s = db0;
-    int s = 0; uint32_t ph = 0;
+    // Straight through, the same for every k-tile: a commit on a condition, or the last one inside the loop, costs the issuer
+    // more cycles than the MMAs take.
+    int s = 0; uint32_t ph = 0, accumulate = 0u;
     for (int kt = 0; kt < k_tiles; ++kt) {
       if (!__all_sync(0xffffffffu, mbar_wait_cta(&full_bar[s], ph, abort_flag))) break;
-      if (kt == 0 && lane == 0) TSTAMP(3);
-      if (kt == k_tiles - 1 && lane == 0) TSTAMP(4);
       if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < BK / 16; ++kk) tc_mma1(tmem_base, da_s + 2 * kk, db_s + dbk * kk, idesc, (kt | kk) ? 1u : 0u);
-        if (kt + stages < k_tiles) tc_commit1(&empty_bar[s]);         // only a stage that is refilled needs the signal
-        if (kt + 1 == k_tiles) tc_commit1(tfull_bar);                 // accumulator complete
+        for (int kk = 0; kk < BK / 16; ++kk) tc_mma1(tmem_base, da_s + 2 * kk, db_s + dbk * kk, idesc, kk ? 1u : accumulate);
+        tc_commit1(&empty_bar[s]);
       }
+      accumulate = 1u;
       da_s += dstage; db_s += dstage;
       if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
     }
+    if (lane == 0) TSTAMP(4);
+    if (elect_one()) tc_commit1(tfull_bar);                            // accumulator complete
     if (kSplit) { __syncwarp(); cluster_sync(); cluster_sync(); }
   } else {
     // ---------------- epilogue warps 3..10: a warp may read the tensor-memory lanes 32 (warp % 4) .. + 31 ----------------
@@ -286,12 +315,13 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     uint8_t* cbuf = smem + (size_t)ew * (half_cols >> 5) * kChunkB;      // (the operand ring is idle by then)
     float* vec_s = reinterpret_cast<float*>(tail) + ew * (kMaxVec * kBiasFloats);
     const int m = m0 + sub * 32 + lane;
+    const int v_first = kSplit ? 0 : half * half_cols, v_cols = kSplit ? BN : half_cols;     // columns of the tile that this warp may need
     auto stage_vectors = [&](bool want_static) {
       for (int k = 0; k < p.n_in; ++k) {
         const TensorArg& a = p.in[k];
         if (k == q.c_input || (((p.static_mask >> (1 + k)) & 1u) != 0) != want_static) continue;
-        for (int c = lane; c < BN; c += 32) {
-          const int n = n0 + c;
+        for (int c = lane; c < v_cols; c += 32) {
+          const int n = n0 + v_first + c;
           vec_s[a.mode * kBiasFloats + c] = n < p.N ? load_scalar<false>(a, (uint32_t)a.base + (uint32_t)n * (uint32_t)a.stride[0]) : 0.0f;
         }
       }
@@ -308,6 +338,19 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
       }
     };
     stage_vectors(true);
+    // The k-tiles of a weight beyond the ring's first ones go into L2 while the previous kernel runs: from DRAM, a ring of four
+    // stages is a microsecond's latency every four k-tiles.  The CTAs of a column of tiles and their epilogue warps take turns.
+    if (q.b_static)
+      for (int kt = stages + tm * kEpiWarps + ew; kt < k_tiles; kt += p.tiles_m * kEpiWarps)
+        if (elect_one()) {
+          if (kBK) {
+            l2_prefetch_2d(&q.tmB, (kt0 + kt) * BK, n0);
+          } else {
+            l2_prefetch_3d(&q.tmB, q.b_blocks ? 0 : n0, (kt0 + kt) * BK, q.b_blocks ? n0 >> 6 : 0);
+            if (q.b_second) l2_prefetch_3d(&q.tmB, n0 + 64, (kt0 + kt) * BK, 0);
+          }
+        }
+    __syncwarp();
     pdl_wait();
     stage_vectors(false);
     uint4 res[4];
@@ -349,8 +392,8 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
         io.out_off = (uint32_t)p.out[0].base + mm * (uint32_t)p.out[0].stride[1];
         const float4* rcv = reinterpret_cast<const float4*>(smem);
         for (int c = half * 16; c < slice; c += 32) {
-          io.col = rank * slice + c;
-          io.n = n0 + io.col;
+          io.vcol = rank * slice + c;
+          io.n = n0 + io.vcol;
           if (q.c_input >= 0) {
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
@@ -359,7 +402,7 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
             }
           }
           uint32_t raw[16];
-          ld16(t_row + io.col, raw);
+          ld16(t_row + io.vcol, raw);
 #pragma unroll
           for (int i = 0; i < 16; ++i) io.accv[i] = __uint_as_float(raw[i]);
           for (int sl = 0; sl < S - 1; ++sl) {
@@ -376,10 +419,11 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     } else if (ok) {
       tc_fence_after();
       bool finish = true;
-      const float* parts = nullptr;
+      uint8_t* recv = smem + (size_t)ew * (size_t)((S - 1) * half_cols * 128);          // the other slices' partial sums (the operand ring is idle by then)
       if (kMode == 2) {
         const uint32_t unit = (uint32_t)tile * kEpiWarps + (uint32_t)ew;
-        float* mine = q.scratch + ((size_t)unit * S + rank) * (size_t)(half_cols * 32) + lane;
+        float* base = q.scratch + (size_t)unit * S * (size_t)(half_cols * 32);
+        float* mine = base + (size_t)rank * (size_t)(half_cols * 32) + lane;
 #pragma unroll 1
         for (int c = 0; c < half_cols; c += 16) {
           uint32_t raw[16];
@@ -387,48 +431,56 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
 #pragma unroll
           for (int i = 0; i < 16; ++i) mine[(c + i) * 32] = __uint_as_float(raw[i]);      // a 128-byte line per instruction
         }
-        __threadfence();                         // this lane's partial sums are visible before the counter moves
+        asm volatile("fence.proxy.async;" ::: "memory");        // (they are read by a bulk copy)
         __syncwarp();
         int old = 0;
-        if (lane == 0) old = atomicAdd(&q.counters[unit], 1);
+        if (lane == 0) old = arrive_acq_rel(&q.counters[unit]);  // the warp's partial sums are visible before the counter moves
         old = __shfl_sync(0xffffffffu, old, 0);
         finish = old == S - 1;                   // else somebody else finishes this part (uniform over the warp)
         if (finish) {
-          if (lane == 0) q.counters[unit] = 0;   // all slices have arrived: ready for the next run
-          __threadfence();
-          parts = q.scratch + (size_t)unit * S * (size_t)(half_cols * 32) + lane;
+          if (lane == 0) {
+            q.counters[unit] = 0;                // all slices have arrived: ready for the next run
+            asm volatile("fence.proxy.async;" ::: "memory");
+            const uint32_t bytes = (uint32_t)half_cols * 128u;
+            mbar_expect_tx(&recv_bar[ew], (uint32_t)(S - 1) * bytes);
+            for (int sl = 0, slot = 0; sl < S; ++sl)
+              if (sl != rank) bulk_load(recv + (size_t)(slot++) * bytes, base + (size_t)sl * (size_t)(half_cols * 32), bytes, &recv_bar[ew]);
+          }
+          __syncwarp();
+          finish = __all_sync(0xffffffffu, mbar_wait_cta(&recv_bar[ew], 0, abort_flag));
         }
       }
       for (int c = 0; finish && c < half_cols; c += 32) {
         const int col = half * half_cols + c;
         if (n0 + col >= p.N) break;                                // (uniform over the warp)
-        io.chunk = cbuf + (c >> 5) * kChunkB;
+        io.chunk = kMode == 2 ? recv + c * 128 : cbuf + (c >> 5) * kChunkB;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
+          uint32_t raw[16];
+          ld16(t_row + col + 16 * h, raw);
           if (kMode == 2) {
-            // slices in order, two slices' loads in flight (written by other SMs: read from L2)
+            // slices in order, this CTA's own in its place
+            const float* o = reinterpret_cast<const float*>(recv) + (c + 16 * h) * 32 + lane;
 #pragma unroll
             for (int i = 0; i < 16; ++i) io.accv[i] = 0.0f;
-            for (int sl = 0; sl < S; sl += 2) {
-              const float* o = parts + (size_t)sl * (size_t)(half_cols * 32) + (c + 16 * h) * 32;
-              const bool two = sl + 1 < S;
-              float v0[16], v1[16];
+            for (int sl = 0; sl < S; ++sl) {
+              if (sl == rank) {
 #pragma unroll
-              for (int i = 0; i < 16; ++i) v0[i] = __ldcg(o + i * 32);
+                for (int i = 0; i < 16; ++i) io.accv[i] += __uint_as_float(raw[i]);
+              } else {
 #pragma unroll
-              for (int i = 0; i < 16; ++i) v1[i] = two ? __ldcg(o + half_cols * 32 + i * 32) : 0.0f;
-#pragma unroll
-              for (int i = 0; i < 16; ++i) io.accv[i] = (io.accv[i] + v0[i]) + v1[i];
+                for (int i = 0; i < 16; ++i) io.accv[i] += o[i * 32];
+                o += half_cols * 32;
+              }
             }
+            __syncwarp();                        // (the chunk buffer lies on columns that everybody has read now)
           } else {
-            uint32_t raw[16];
-            ld16(t_row + col + 16 * h, raw);
 #pragma unroll
             for (int i = 0; i < 16; ++i) io.accv[i] = __uint_as_float(raw[i]);
           }
           io.res[0] = res[2 * h]; io.res[1] = res[2 * h + 1];
           if (h == 1 && q.c_input >= 0 && c + 32 < half_cols) fetch_residual(n0 + col + 32, res);
-          io.col = col + 16 * h; io.n = n0 + io.col; io.h = h;
+          io.vcol = c + 16 * h; io.n = n0 + col + 16 * h; io.h = h;
           run_program<16, SP, true>(p.prog, io);
         }
         fence_async_smem();
@@ -498,16 +550,48 @@ static int ws_slices(const GemmParams& gp) {
   return s >= 3 ? (int)s : 1;
 }
 
-// Measured on the projection and feed-forward shapes of a 1024-token encoder layer: a k-tile costs a CTA about 0.22 us
-// whatever the tile's size, so a problem with few 256 x 256 tiles and a short K finishes sooner as many small tiles
-// (1024 x 768 x 768: 5.4 against 7.8 us; 1024 x 2304 x 768: 7.4 against 8.1; 1024 x 3072 x 768: 10.1 against 11.1); with a long K
-// only where CTAs can share its k-tiles through the workspace.
+// Microseconds of an unsplit problem with tiles of 128 x bn: set-up, and the k-tiles and epilogues of the CTAs that share an SM one
+// after the other (rows x N x K, measured / counted: 1024 x 768 x 768 in 64 columns 4.8 / 4.8, 128 6.0 / 6.0, 192 7.3 / 7.2;
+// 1024 x 768 x 3072 in 64 columns 10.0 / 10.0; 4096 x 768 x 768 in 128 columns, two CTAs per SM, 8.8 / 9.3).  A third CTA of an SM
+// starts when another has left.
+static double tile_us(const GemmParams& gp, int bn) {
+  const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
+  const int64_t tiles = (int64_t)((gp.M + tc2::BM - 1) / tc2::BM) * ((gp.N + bn - 1) / bn);
+  const double c = (double)((tiles + sm_count() - 1) / sm_count());
+  const double k_us = bn == 64 ? 0.145 : bn == 128 ? 0.2 : 0.235, epi_us = bn == 64 ? 0.3 : bn == 128 ? 0.85 : 1.6;
+  return 2.75 + c * (k_tiles * k_us + epi_us) + (c > 2 ? 1.5 * (c - 2) : 0.0);
+}
+// 192 columns only while every tile has an SM to itself (its ring leaves no room for a second CTA) and 64 divides N (one request for B).
+static int tile_columns(const GemmParams& gp) {
+  const int64_t tiles_m = (gp.M + tc2::BM - 1) / tc2::BM;
+  int best = 64;
+  if (gp.N > 64 && tile_us(gp, 128) < tile_us(gp, best)) best = 128;
+  if (gp.N > 128 && gp.N % 64 == 0 && tiles_m * ((gp.N + 191) / 192) <= sm_count() && tile_us(gp, 192) < tile_us(gp, best)) best = 192;
+  return best;
+}
+// The same for the CTA-pair kernel: one wave of 256-row tiles after the other, the last epilogue on its own (512 x 768 x 768 7.2 / 7.2,
+// 2048 x 384 x 1536 9.6 / 9.6, 4096 x 2304 x 768 14.9 / 15.8).
+static double pair_us(const GemmParams& gp) {
+  const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
+  double best = 0.0;
+  for (int bn : {256, 192, 128}) {
+    const int64_t tiles = (int64_t)((gp.M + 255) / 256) * ((gp.N + bn - 1) / bn);
+    const double waves = (double)((tiles + sm_count() / 2 - 1) / (sm_count() / 2));
+    const double main_us = k_tiles * (bn == 256 ? 0.28 : bn == 192 ? 0.24 : 0.2), epi_us = bn == 256 ? 2.3 : bn == 192 ? 1.7 : 1.15;
+    const double us = 3.6 + waves * std::max(main_us, epi_us) + epi_us + 0.9 * (waves - 1);
+    if (best == 0.0 || us < best) best = us;
+  }
+  return best;
+}
+
+// Against the CTA-pair kernel: whichever the counts say is the faster (1024 x 768 x 768 4.8 against 7.2 us, 2048 x 2304 x 768 8.9 / 11.3,
+// 2048 x 768 x 3072 13.4 / 15.2, 4096 x 768 x 3072 16.8 / 17.8; 4096 x 2304 x 768 16.9 / 14.9).
 bool tile_gemm_preferred(const GemmParams& gp) {
   if (plan_flag(DNNF_PLAN_NO_TILE_GEMM)) return false;
   if (dev_env("DNNF_GEMM_TILE")) return atoi(dev_env("DNNF_GEMM_TILE")) != 0;
-  const int64_t pair_tiles = (int64_t)((gp.M + 255) / 256) * ((gp.N + 255) / 256);
-  const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
-  return pair_tiles < sm_count() / 2 && (k_tiles <= 16 || plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K) || ws_slices(gp) > 1);
+  if (ws_slices(gp) > 1) return true;
+  if (plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K)) return (int64_t)((gp.M + 255) / 256) * ((gp.N + 255) / 256) < sm_count() / 2;
+  return tile_us(gp, tile_columns(gp)) < pair_us(gp);
 }
 
 void tile_gemm_plan(Launch& L) {
@@ -517,10 +601,9 @@ void tile_gemm_plan(Launch& L) {
   q.k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
   const int tiles_m = (gp.M + tc2::BM - 1) / tc2::BM;
   const int sms = sm_count();
-  // N tile: 128 columns unless that leaves most of the machine without a CTA (an MMA costs its issuer the same 60
-  // cycles whatever its width); with the cluster split the CTAs come from the split instead
-  int best_bn = (gp.N > 64 && (plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K) || (int64_t)tiles_m * ((gp.N + 127) / 128) >= 96)) ? 128 : 64;
-  if (dev_env("DNNF_TILE_BN")) best_bn = atoi(dev_env("DNNF_TILE_BN")) == 128 ? 128 : 64;
+  // (with the cluster split the CTAs come from the split instead)
+  int best_bn = plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K) ? (gp.N > 64 ? 128 : 64) : tile_columns(gp);
+  if (dev_env("DNNF_TILE_BN")) best_bn = atoi(dev_env("DNNF_TILE_BN"));
   q.bn = best_bn;
   q.tiles_n = (gp.N + q.bn - 1) / q.bn;
   q.fd_tiles_n = make_fastdiv((uint32_t)q.tiles_n);
@@ -559,16 +642,19 @@ void tile_gemm_plan(Launch& L) {
     else { q.c_input = i; gp.in[i].mode = 0; }
   }
   q.b_static = (gp.static_mask & 1u) ? 1 : 0;
+  q.b_blocks = gp.N % 64 == 0 ? 1 : 0;
+  q.b_second = !q.b_blocks && q.bn == 128 ? 1 : 0;
   L.early_reads = gp.static_mask != 0;
   const int stage_bytes = tc2::BM * tc2::BK * 2 + q.bn * tc2::BK * 2;
   const int fixed = 1024 + tile::kVecBytes + tile::kBarBytes;
-  int budget = tile::kSmemTwoPerSm;
+  int budget = q.bn > 128 ? tile::kSmemOnePerSm : tile::kSmemTwoPerSm;
   if (dev_env("DNNF_TILE_SMEM")) budget = atoi(dev_env("DNNF_TILE_SMEM")) * 1024;
   q.stages = std::max(2, std::min({8, q.kt_per, (budget - fixed) / stage_bytes}));
   int ring = q.stages * stage_bytes;                               // (the chunk buffers, 128 x bn bf16, are never more than that)
-  if (S > 1 && !q.ws_split) ring = std::max(ring, (S - 1) * (q.bn / S / 4) * tc2::BM * 16);          // the ring doubles as the receive buffer
+  if (q.ws_split) ring = std::max(ring, tile::kEpiWarps * (S - 1) * (q.bn / 2) * 128);               // the ring doubles as the receive buffer
+  if (S > 1 && !q.ws_split) ring = std::max(ring, (S - 1) * (q.bn / S / 4) * tc2::BM * 16);          // (here too)
   q.tail_off = ring;
-  q.tmem_cols = q.bn < 32 ? 32 : q.bn;
+  q.tmem_cols = q.bn <= 64 ? 64 : q.bn <= 128 ? 128 : 256;
   L.counter_bytes = q.ws_split ? tiles * tile::kEpiWarps * 4 : 0;
   L.scratch_bytes = q.ws_split ? tiles * S * tc2::BM * q.bn * 4 : 0;
   L.grid = (int)(tiles * S);
@@ -595,7 +681,12 @@ bool tile_gemm_prepare(Launch& L, std::string& err) {
   if (((uintptr_t)a & 15) || ((uintptr_t)b & 15) || ((uintptr_t)d & 15)) { err = "GEMM operand is not 16-byte aligned"; return false; }
   if (!encode2d(&q.tmA, a, gp.K, gp.M, gp.A.stride_row, tc2::BK, tc2::BM, err)) return false;
   if (q.b_kmajor) { if (!encode2d(&q.tmB, b, gp.K, gp.N, gp.B.stride_col, tc2::BK, q.bn, err)) return false; }
-  else { if (!encode2d(&q.tmB, b, gp.N, gp.K, gp.B.stride_row, 64, tc2::BK, err)) return false; }
+  else {
+    cuuint64_t dims[3] = {(cuuint64_t)(q.b_blocks ? 64 : gp.N), (cuuint64_t)gp.K, (cuuint64_t)(q.b_blocks ? gp.N / 64 : 1)};
+    cuuint64_t strides[2] = {(cuuint64_t)gp.B.stride_row * 2, 128};
+    cuuint32_t box[3] = {64, (cuuint32_t)tc2::BK, (cuuint32_t)(q.b_blocks ? q.bn / 64 : 1)};
+    if (!tma_encode(&q.tmB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, b, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B, err)) return false;
+  }
   if (!encode2d(&q.tmD, d, gp.N, gp.M, gp.out[0].stride[1], 32, 32, err, CU_TENSOR_MAP_SWIZZLE_64B)) return false;
   if (q.c_input >= 0 && ((uintptr_t)(reinterpret_cast<uint16_t*>(gp.in[q.c_input].ptr) + gp.in[q.c_input].base) & 15)) {
     err = "epilogue operand is not 16-byte aligned"; return false;
@@ -605,17 +696,20 @@ bool tile_gemm_prepare(Launch& L, std::string& err) {
 
 struct TileLauncher {
   const Launch& L; cudaStream_t st; cudaError_t rc;
-  template <class SP, int kMode> void plain() {
+  template <class SP, int kMode, bool kBK> void plain() {
     static PerDeviceOnce once;       // per instantiation
-    if (once.first_use()) cudaFuncSetAttribute(tile::gemm_tile_kernel<SP, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    rc = launch_pdl(tile::gemm_tile_kernel<SP, kMode>, dim3(L.grid), dim3(tile::kThreads), L.smem, st, gp_of(L), tl_of(L));
+    if (once.first_use()) cudaFuncSetAttribute(tile::gemm_tile_kernel<SP, kMode, kBK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    rc = launch_pdl(tile::gemm_tile_kernel<SP, kMode, kBK>, dim3(L.grid), dim3(tile::kThreads), L.smem, st, gp_of(L), tl_of(L));
   }
   template <class SP> void run() {
+    if (tl_of(L).b_kmajor) major<SP, true>(); else major<SP, false>();
+  }
+  template <class SP, bool kBK> void major() {
     const int S = tl_of(L).ksplit;
-    if (S <= 1) { plain<SP, 0>(); return; }
-    if (tl_of(L).ws_split) { plain<SP, 2>(); return; }
+    if (S <= 1) { plain<SP, 0, kBK>(); return; }
+    if (tl_of(L).ws_split) { plain<SP, 2, kBK>(); return; }
     static PerDeviceOnce once;
-    if (once.first_use()) cudaFuncSetAttribute(tile::gemm_tile_kernel<SP, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    if (once.first_use()) cudaFuncSetAttribute(tile::gemm_tile_kernel<SP, 1, kBK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(L.grid); cfg.blockDim = dim3(tile::kThreads); cfg.dynamicSmemBytes = L.smem; cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -624,7 +718,7 @@ struct TileLauncher {
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    rc = cudaLaunchKernelEx(&cfg, tile::gemm_tile_kernel<SP, 1>, gp_of(L), tl_of(L));
+    rc = cudaLaunchKernelEx(&cfg, tile::gemm_tile_kernel<SP, 1, kBK>, gp_of(L), tl_of(L));
   }
 };
 

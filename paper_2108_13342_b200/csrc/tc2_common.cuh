@@ -28,8 +28,6 @@ namespace tc2 {
 #endif
 
 constexpr int BM = 128, BK = 64, EPI_WARPS = 8, THREADS = 64 + 32 * EPI_WARPS;
-constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // 1 s
-constexpr int kFastPolls = 2048;                             // polls of a barrier before the wall clock is consulted
 constexpr int kWaitPolls = 1 << 18;
 constexpr int kSmemMax = 227 * 1024;
 constexpr int kBiasFloats = 128;                             // per warp, per row-invariant operand
