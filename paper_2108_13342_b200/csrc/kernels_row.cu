@@ -16,6 +16,9 @@ int launch_row_h(const Launch& L, cudaStream_t st);
 int launch_row_i(const Launch& L, cudaStream_t st);
 int launch_row_j(const Launch& L, cudaStream_t st);
 int launch_row_k(const Launch& L, cudaStream_t st);
+int launch_row_l(const Launch& L, cudaStream_t st);
+int launch_row_shift(const Launch& L, cudaStream_t st);
+bool finalize_row_shift(Launch& L);
 
 // variant encoding: V * 100000 + NV * 1000 + WPR * 10 + RPW
 int launch_row(const Launch& L, cudaStream_t st) {
@@ -31,6 +34,8 @@ int launch_row(const Launch& L, cudaStream_t st) {
   if (rc == 2) rc = launch_row_i(L, st);
   if (rc == 2) rc = launch_row_j(L, st);
   if (rc == 2) rc = launch_row_k(L, st);
+  if (rc == 2) rc = launch_row_l(L, st);
+  if (rc == 2) rc = launch_row_shift(L, st);
   return rc;
 }
 
@@ -50,6 +55,7 @@ bool finalize_row(Launch& L) {
   // 148 * 32 for a lone 1024-row launch.
   static const long target = dev_env("DNNF_ROW_TARGET_WARPS") ? atol(dev_env("DNNF_ROW_TARGET_WARPS")) : 4000L;
   static const long split_target = dev_env("DNNF_ROW_SPLIT_TARGET") ? atol(dev_env("DNNF_ROW_SPLIT_TARGET")) : 4000L;   // (2000 is 3 % better when independent blocks overlap, 20 % worse for a lone 1024-row launch)
+  if (V == 1 && finalize_row_shift(L)) return true;
   if (V == 4) {
     const int vectors = (Lr + 3) / 4;
     auto fit = [&](int w) { int need = (vectors + 32 * w - 1) / (32 * w); return need; };   // vectors per lane with w warps per row
@@ -85,7 +91,7 @@ bool finalize_row(Launch& L) {
   int64_t warps = (p.rows + rpw - 1) / rpw;
   L.grid = wpr > 1 ? (int)p.rows : (int)((warps + kRowWarpsPerCta - 1) / kRowWarpsPerCta);
   L.threads = wpr > 1 ? 32 * wpr : 32 * kRowWarpsPerCta;
-  L.static_id = (V == 4 ? (wpr < 8 || nv == 1) : nv < 32) ? StaticSet<RowStatic>::find(p.prog) : 0;
+  L.static_id = V == 4 || nv < 32 ? StaticSet<RowStatic>::find(p.prog) : 0;
   set_fastdiv(p.it);
   return true;
 }
