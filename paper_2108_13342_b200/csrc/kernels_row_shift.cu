@@ -11,7 +11,7 @@ namespace dnnf {
 
 namespace {
 
-// LPR lanes share a row (8, 32 or a CTA of 256), each with NV vectors of four.
+// LPR lanes share a row, each with NV vectors of four.
 template <int NV, int LPR>
 struct ShiftIO {
   static constexpr int VV = 4 * NV;
@@ -21,6 +21,9 @@ struct ShiftIO {
   int lane_in_row, m;
   float* xchg;                     // shared memory, 2 x 8 floats (LPR == 256)
   mutable int xslot = 0;
+  // Vectors that can reach past an end of the row: the first, and the last two (with no form for seven vectors, three of eight).
+  // The ones between lie in the row whole, and so does the window of eight that an operand of another alignment is read through.
+  static constexpr bool edge(int j) { return j == 0 || j >= NV - (NV == 8 ? 3 : 2); }
   __device__ __forceinline__ int col(int j) const { return 4 * (j * LPR + lane_in_row) - m; }
   __device__ __forceinline__ bool valid(int c) const { return (unsigned)c < (unsigned)p.L; }
   __device__ __forceinline__ const float* row_ptr(const TensorArg& a) const {
@@ -30,6 +33,10 @@ struct ShiftIO {
     return reinterpret_cast<const float*>(a.ptr) + off;
   }
   static __device__ __forceinline__ int misalignment(const float* q) { return (int)((reinterpret_cast<uintptr_t>(q) >> 2) & 3); }
+  __device__ __forceinline__ void masked(const float* q, int c, float* d) const {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) d[v] = row_ok && valid(c + v) ? __ldg(q + c + v) : 0.0f;
+  }
   __device__ __forceinline__ void load(int idx, float (&dst)[VV]) const {
     const TensorArg& a = p.in[idx];
     const float* q = row_ptr(a);
@@ -39,17 +46,38 @@ struct ShiftIO {
       for (int e = 0; e < VV; ++e) dst[e] = x;
       return;
     }
-    const bool same = misalignment(q) == m;
+    const int by = (misalignment(q) - m) & 3;      // this operand's vectors lie `by` elements earlier (the same for a warp but where rows share one)
+    if (by == 0) {
+#pragma unroll
+      for (int j = 0; j < NV; ++j) {
+        const int c = col(j);
+        float* d = &dst[4 * j];
+        if (row_ok && (!edge(j) || (c >= 0 && c + 4 <= p.L))) {
+          const float4 w = __ldg(reinterpret_cast<const float4*>(q + c));
+          d[0] = w.x; d[1] = w.y; d[2] = w.z; d[3] = w.w;
+        } else {
+          masked(q, c, d);
+        }
+      }
+      return;
+    }
+    if (LPR < 32) {
+#pragma unroll
+      for (int j = 0; j < NV; ++j) masked(q, col(j), &dst[4 * j]);
+      return;
+    }
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       const int c = col(j);
       float* d = &dst[4 * j];
-      if (same && row_ok && c >= 0 && c + 4 <= p.L) {
-        const float4 w = __ldg(reinterpret_cast<const float4*>(q + c));
-        d[0] = w.x; d[1] = w.y; d[2] = w.z; d[3] = w.w;
+      if (row_ok && (!edge(j) || (c >= by && c + 8 <= p.L))) {
+        const float4 u = __ldg(reinterpret_cast<const float4*>(q + c - by)), w = __ldg(reinterpret_cast<const float4*>(q + c - by) + 1);
+        d[0] = by == 1 ? u.y : by == 2 ? u.z : u.w;
+        d[1] = by == 1 ? u.z : by == 2 ? u.w : w.x;
+        d[2] = by == 1 ? u.w : by == 2 ? w.x : w.y;
+        d[3] = by == 1 ? w.x : by == 2 ? w.y : w.z;
       } else {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) d[v] = row_ok && valid(c + v) ? __ldg(q + c + v) : 0.0f;
+        masked(q, c, d);
       }
     }
   }
@@ -64,7 +92,7 @@ struct ShiftIO {
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       const int c = col(j);
-      if (same && c >= 0 && c + 4 <= p.L) {
+      if (same && (!edge(j) || (c >= 0 && c + 4 <= p.L))) {
         *reinterpret_cast<float4*>(q + c) = make_float4(val[4 * j], val[4 * j + 1], val[4 * j + 2], val[4 * j + 3]);
       } else {
 #pragma unroll
@@ -74,14 +102,19 @@ struct ShiftIO {
   }
   __device__ __forceinline__ void row_reduce(int op, float (&acc)[VV]) const {
     pdl_launch_dependents();         // (the row's loads have been issued)
-    float red = op == M_ROWMAX ? -CUDART_INF_F : (op == M_ROWPROD ? 1.0f : 0.0f);
-    auto join = [&](float x) { if (op == M_ROWMAX) red = fmaxf(red, x); else if (op == M_ROWPROD) red *= x; else red += x; };
+    const float none = op == M_ROWMAX ? -CUDART_INF_F : (op == M_ROWPROD ? 1.0f : 0.0f);
+    auto join = [&](float& r, float x) { if (op == M_ROWMAX) r = fmaxf(r, x); else if (op == M_ROWPROD) r *= x; else r += x; };
+    float part[4] = {none, none, none, none};          // four chains instead of one
 #pragma unroll
-    for (int j = 0; j < NV; ++j)
+    for (int j = 0; j < NV; ++j) {
+      const int c = col(j);
 #pragma unroll
-      for (int v = 0; v < 4; ++v) if (valid(col(j) + v)) join(acc[4 * j + v]);
+      for (int v = 0; v < 4; ++v) join(part[v], !edge(j) || valid(c + v) ? acc[4 * j + v] : none);
+    }
+    join(part[0], part[1]); join(part[2], part[3]); join(part[0], part[2]);
+    float red = part[0];
 #pragma unroll
-    for (int o = (LPR < 32 ? LPR : 32) / 2; o > 0; o >>= 1) join(__shfl_xor_sync(0xffffffffu, red, o));
+    for (int o = (LPR < 32 ? LPR : 32) / 2; o > 0; o >>= 1) join(red, __shfl_xor_sync(0xffffffffu, red, o));
     if (LPR > 32) {
       // two exchange areas used in turn: the barrier of this exchange also tells that everybody has read the one before
       float* x = xchg + xslot * (LPR / 32);
@@ -90,7 +123,7 @@ struct ShiftIO {
       __syncthreads();
       red = x[0];
 #pragma unroll
-      for (int w = 1; w < LPR / 32; ++w) join(x[w]);
+      for (int w = 1; w < LPR / 32; ++w) join(red, x[w]);
     }
     const float x = op == M_ROWMEAN ? red * p.inv_L : red;
 #pragma unroll
@@ -143,33 +176,25 @@ int launch_row_shift(const Launch& L, cudaStream_t st) {
   switch (L.variant) {
     case 901008: return launch_shift<1, 8>(L, st);
     case 902008: return launch_shift<2, 8>(L, st);
+    case 903008: return launch_shift<3, 8>(L, st);
     case 904008: return launch_shift<4, 8>(L, st);
-    case 902032: return launch_shift<2, 32>(L, st);
-    case 904032: return launch_shift<4, 32>(L, st);
-    case 908032: return launch_shift<8, 32>(L, st);
-    case 901256: return launch_shift<1, 256>(L, st);
-    case 902256: return launch_shift<2, 256>(L, st);
-    case 904256: return launch_shift<4, 256>(L, st);
-    case 908256: return launch_shift<8, 256>(L, st);
     default: return 2;
   }
 }
 
-// The lanes of a row: the fewest that hold it in eight vectors, a CTA for longer ones.  With few rows (up to three per SM) of more
-// than 128 elements a CTA shares each, as in the element-wise form.
+// Rows of up to 122 elements, four to a warp: 64 x 12 x 61 x 61 masked softmax 13.5 -> 6.5 us, 131072 x 93 LayerNorm + GELU 38.6.  Longer
+// ones stay with one element per lane and load: with a warp or a CTA to a row the branches between the loads serialise them
+// (8000 x 4095 91 -> 150 us, 32 x 12 x 317 x 317 80.8 -> 84.6).
 bool finalize_row_shift(Launch& L) {
   RowParams& p = L.row;
-  L.static_id = StaticSet<RowStatic>::find(p.prog);
-  if (!L.static_id) return false;
+  const int vectors = (p.L + 6) / 4;                             // up to three elements in front of the row
+  if (vectors > 32) return false;
   for (int i = 0; i < p.n_in; ++i) if (p.in[i].dtype != 0) return false;
   for (int i = 0; i < p.n_out; ++i) if (p.out[i].dtype != 0 || p.out[i].stride[0] != 1) return false;
   if (p.in[0].stride[0] != 1) return false;
-  const int vectors = (p.L + 6) / 4;                             // up to three elements in front of the row
-  int nv = 0, lpr = 0;
-  if (vectors <= 32) { lpr = 8; nv = vectors <= 8 ? 1 : vectors <= 16 ? 2 : 4; }
-  else if (vectors <= 256 && p.rows > 3L * sm_count()) { lpr = 32; nv = vectors <= 64 ? 2 : vectors <= 128 ? 4 : 8; }
-  else { lpr = 256; nv = vectors <= 256 ? 1 : vectors <= 512 ? 2 : vectors <= 1024 ? 4 : 8; }
-  if (vectors > nv * lpr) return false;
+  L.static_id = StaticSet<RowStatic>::find(p.prog);
+  if (!L.static_id) return false;
+  const int lpr = 8, nv = (vectors + lpr - 1) / lpr;
   L.variant = 900000 + nv * 1000 + lpr;
   const int64_t rows_per_cta = lpr > 32 ? 1 : 32 * kRowWarpsPerCta / lpr;
   L.grid = (int)((p.rows + rows_per_cta - 1) / rows_per_cta);
