@@ -411,6 +411,11 @@ DNNF_API int dnnf_status(dnnf_graph* g, int* device_status, int* block);
  * reports DNNF_ERR_TIMEOUT from block -2; the caller then clears the workspace's first dnnf_workspace_zero_bytes bytes
  * and the graph runs as before.  Needs a bound workspace; nothing faults, traps or hangs. */
 DNNF_API int dnnf_selftest_wait_expiry(dnnf_graph* g, uint64_t limit_ns, void* cuda_stream);
+/* The same with one of the framework's own kernels: block `block`, which has to run on the one-tile-per-CTA bf16 GEMM kernel and
+ * to have run before, is launched with a descriptor that brings one row of its first operand less than the kernel waits for.  Its
+ * waits run out after a second; it must then store nothing, leave the workspace's counters as they were and report DNNF_ERR_TIMEOUT
+ * from that block.  Every copy stays inside the operand and the kernel's shared memory; nothing faults, traps or hangs. */
+DNNF_API int dnnf_selftest_lost_copy(dnnf_graph* g, int block, void* cuda_stream);
 /* Number of kernels one dnnf_run launches. */
 DNNF_API int dnnf_launch_count(const dnnf_graph* g, int* n);
 

@@ -23,6 +23,7 @@ int profile_measure(Graph& g, void* scratch, size_t scratch_bytes, void* stream,
 static int fail(dnnf_graph* g, int code, const char* msg) { if (g) g->g.err = msg; return code; }
 
 namespace dnnf { int selftest_wait_expiry(Graph& g, unsigned long long limit_ns, void* stream); }
+namespace dnnf { int selftest_lost_copy(Graph& g, int block, void* stream); }
 
 extern "C" {
 
@@ -445,6 +446,11 @@ int dnnf_block_info(const dnnf_graph* g, int bi, dnnf_block_desc* out) {
 int dnnf_selftest_wait_expiry(dnnf_graph* g, uint64_t limit_ns, void* stream) {
   if (!g) return DNNF_ERR_INVALID_ARG;
   return dnnf::selftest_wait_expiry(g->g, limit_ns, stream);
+}
+
+int dnnf_selftest_lost_copy(dnnf_graph* g, int block, void* stream) {
+  if (!g) return DNNF_ERR_INVALID_ARG;
+  return dnnf::selftest_lost_copy(g->g, block, stream);
 }
 
 int dnnf_block_tensors(const dnnf_graph* g, int bi, int* in_ids, int cap_in, int* n_in, int* out_ids, int cap_out, int* n_out) {

@@ -294,8 +294,9 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     // Straight through, the same for every k-tile: a commit on a condition, or the last one inside the loop, costs the issuer
     // more cycles than the MMAs take.
     int s = 0; uint32_t ph = 0, accumulate = 0u;
+    bool ok = true;
     for (int kt = 0; kt < k_tiles; ++kt) {
-      if (!__all_sync(0xffffffffu, mbar_wait_cta(&full_bar[s], ph, abort_flag))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait_cta(&full_bar[s], ph, abort_flag))) { ok = false; break; }
       if (elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < BK / 16; ++kk) tc_mma1(tmem_base, da_s + 2 * kk, db_s + dbk * kk, idesc, kk ? 1u : accumulate);
@@ -306,7 +307,7 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
       if (++s == stages) { s = 0; ph ^= 1; da_s = da0; db_s = db0; }
     }
     if (lane == 0) TSTAMP(4);
-    if (elect_one()) tc_commit1(tfull_bar);                            // accumulator complete
+    if (ok && elect_one()) tc_commit1(tfull_bar);                      // accumulator complete (after a wait that ran out it never is)
     if (kSplit) { __syncwarp(); cluster_sync(); cluster_sync(); }
   } else {
     // ---------------- epilogue warps 3..10: a warp may read the tensor-memory lanes 32 (warp % 4) .. + 31 ----------------
@@ -733,6 +734,20 @@ int tile_gemm_launch(const Launch& L, cudaStream_t st) {
   TileLauncher F{L, st, cudaSuccess};
   if (!(L.static_id > 0 && StaticSet<Epi2Static>::dispatch(L.static_id, F))) F.run<DynProg>();
   return (F.rc == cudaSuccess && cudaGetLastError() == cudaSuccess) ? 0 : 1;
+}
+
+// Launch of the block with a descriptor that brings one row of A less than the kernel waits for, as a lost copy would: the waits
+// for the operands run out.  The caller's launch is left as it is.
+int tile_gemm_lose_a_row(Launch L, void* status_words, int block_index, cudaStream_t st, std::string& err) {
+  if (L.variant != 5 || !L.tc_ready) { err = "the block does not run, or has not yet run, on the one-tile-per-CTA GEMM kernel"; return DNNF_ERR_INVALID_ARG; }
+  GemmParams& gp = gp_of(L);
+  gp.status = reinterpret_cast<int32_t*>(status_words);
+  gp.block_index = block_index;
+  gp.ordered = 1;
+  if (!encode2d(&tl_of(L).tmA, reinterpret_cast<uint16_t*>(gp.A.ptr) + gp.A.base, gp.K, gp.M, gp.A.stride_row, tc2::BK, tc2::BM - 1, err)) return DNNF_ERR_CUDA;
+  tile_set_scratch(L, status_words);
+  if (tile_gemm_launch(L, st)) { err = "self-test launch failed"; return DNNF_ERR_CUDA; }
+  return DNNF_OK;
 }
 
 }  // namespace dnnf

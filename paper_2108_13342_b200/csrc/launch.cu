@@ -14,6 +14,7 @@ int launch_ew(const Launch& L, cudaStream_t st);
 int launch_row(const Launch& L, cudaStream_t st);
 void set_ordered(Launch& L, bool on);
 int launch_contraction(const Launch& L, void* status_words, int block_index, cudaStream_t st, std::string& err);
+int tile_gemm_lose_a_row(Launch L, void* status_words, int block_index, cudaStream_t st, std::string& err);
 void patch_contraction(Launch& L, const std::vector<void*>& in_ptrs, const std::vector<void*>& out_ptrs, std::string& err);
 
 static void* resolve(Graph& g, int t) {
@@ -175,6 +176,13 @@ int selftest_wait_expiry(Graph& g, unsigned long long limit_ns, void* stream) {
   wait_expiry_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(reinterpret_cast<int32_t*>(g.ws_ptr), (int)std::max(1ull, limit_ns / 4000));     // (a poll takes 4 us)
   if (cudaGetLastError() != cudaSuccess) { g.err = "self-test launch failed"; return DNNF_ERR_CUDA; }
   return DNNF_OK;
+}
+
+int selftest_lost_copy(Graph& g, int block, void* stream) {
+  if (!g.planned || !g.ws_ptr) { g.err = "plan the graph and bind a workspace first: the status words live in it"; return DNNF_ERR_WORKSPACE; }
+  if (block < 0 || block >= (int)g.blocks.size()) { g.err = "no such block"; return DNNF_ERR_INVALID_ARG; }
+  g.last_status_base = g.ws_ptr;
+  return tile_gemm_lose_a_row(g.blocks[block].launch, g.ws_ptr, block, (cudaStream_t)stream, g.err);
 }
 
 int read_status(Graph& g, int* status, int* block) {

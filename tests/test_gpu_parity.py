@@ -269,3 +269,27 @@ def test_bounded_wait_expires_and_the_graph_runs_on():
     assert s.g.status() == (0, -1)
     with pytest.raises(B.DnnfError):
         s.g.selftest_wait_expiry(10**12, stream)               # limits beyond 100 ms are refused
+
+
+@pytest.mark.parametrize("mnk,slices", [((300, 128, 256), 1), ((248, 768, 3072), 4)])
+def test_a_gemm_whose_copy_is_lost_stores_nothing(mnk, slices):
+    """A copy that brings less than the kernel waits for: its waits run out, nothing of the incomplete accumulator is stored or
+    handed to the CTAs that share the tile (their counters stand as before: the next run is right without clearing them)."""
+    import torch
+    m, n, k = mnk
+    g = graph()
+    g.ext("A", (m, k), "bf16"); g.ext("Bm", (k, n), "bf16", "weight")
+    g.mark_output(g.add("MatMul", ["A", "Bm"], out="Y"))
+    wl = W.Workload(g, {"A": W.round_to_bf16(rnd((m, k), 990, -1, 1)), "Bm": W.round_to_bf16(rnd((k, n), 991, -0.1, 0.1))})
+    s, got, ref = run_both(wl)
+    close(got["Y"], ref["Y"], RTOL_BF16)
+    b = s.g.blocks()[0]
+    assert b["variant"] == 5 and b["grid"] % slices == 0 and (slices > 1) == (s.g.workspace_zero_bytes() > 256), b
+    s.buffers["Y"].fill_(float("nan"))
+    s.g.selftest_lost_copy(0, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert s.g.status() == (B.ERR_TIMEOUT, 0)
+    assert torch.isnan(s.buffers["Y"]).all()
+    s.workspace[:8].zero_()                                    # the status words alone
+    s.run()
+    assert np.array_equal(s.output("Y"), got["Y"]) and s.g.status() == (0, -1)
