@@ -22,6 +22,7 @@
 #include <mutex>
 #include <string>
 
+#include "bounded_wait.cuh"
 #include "conv_params.h"
 #include "launch_util.h"
 #include "tma_host.h"
@@ -31,7 +32,6 @@ namespace dnnf {
 namespace dwt {
 
 constexpr int THREADS = 256;
-constexpr int kWaitPolls = 1 << 18;
 
 struct Params {
   CUtensorMap tmX;           // dims (C, W, H, N), box (cb, wt + 2, ht + 2, 1), no swizzle
@@ -55,11 +55,9 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded wait: false when the polls ran out, a second at 4 us each (the caller records the failure and leaves).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-#pragma unroll 1
-  for (int i = 0; i < kWaitPolls; ++i) if (mbar_try(bar, parity)) return true;
-  return false;
+// Bounded wait: sets *failed when it ran out (the CTA then records the failure and leaves).
+__device__ __forceinline__ void mbar_wait(uint64_t* bar, uint32_t parity, volatile int* failed) {
+  bounded_wait([=] { return mbar_try(bar, parity); }, failed);
 }
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, uint64_t* bar, int c0, int c1, int c2, int c3) {
   asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
@@ -158,7 +156,7 @@ __global__ void __launch_bounds__(THREADS, 2) dwconv_tma_kernel(const __grid_con
     const int next = tile + gridDim.x;
     // buffer buf^1 was read during iteration k-1, which ended with a barrier
     if (threadIdx.x == 0 && next < q.total_tiles) issue(next, buf ^ 1);
-    if (!mbar_wait(&full_bar[buf], (k >> 1) & 1)) failed = 1;
+    mbar_wait(&full_bar[buf], (k >> 1) & 1, &failed);
     __syncthreads();
     if (failed) break;
     uint32_t t = (uint32_t)tile, u;

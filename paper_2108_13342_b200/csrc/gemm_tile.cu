@@ -88,10 +88,7 @@ __device__ __forceinline__ bool mbar_try_cta(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 __device__ __forceinline__ bool mbar_wait_cta(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-#pragma unroll 1
-  for (int i = 0; i < kWaitPolls; ++i) if (mbar_try_cta(bar, parity)) return true;
-  *abort_flag = 1;
-  return false;
+  return bounded_wait([=] { return mbar_try_cta(bar, parity); }, abort_flag);
 }
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* tm, uint64_t* bar, int c0, int c1, int c2) {
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"

@@ -150,21 +150,30 @@ int profile_measure(Graph& g, void* scratch, size_t scratch_bytes, void* stream,
   return rc_all;
 }
 
-// Self-test of the bounded waits: one CTA waits, with the kernels' own wait routine, on a barrier that nothing will
-// ever signal.  The wait has to give up after `limit_ns`, raise the CTA's abort flag and come back; the kernel then
+// Self-test of the bounded waits: one CTA waits, with the kernels' own wait routine, on a barrier whose phase nothing
+// completes, while a second warp keeps arriving on it (as the other roles of a kernel do: a failed poll then comes back at once).
+// The wait has to give up after its limit, raise the CTA's abort flag and come back; the kernel then
 // records DNNF_ERR_TIMEOUT in the status words the way every tensor-core kernel's tear-down does.  Nothing faults and
 // nothing hangs: this is the path a lost TMA completion or a missing commit would take.
-__global__ void wait_expiry_kernel(int32_t* status, int polls) {
+__global__ void wait_expiry_kernel(int32_t* status, uint32_t limit_cycles) {
+  constexpr uint32_t kArrivals = 1u << 20;         // (a barrier counts up to 2^20 - 1)
   __shared__ uint64_t bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
-    mbar_init(&bar, 1);
+    mbar_init(&bar, kArrivals - 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   bool ok = true;
-  if (threadIdx.x == 0) ok = mbar_wait(&bar, 0, &abort_flag, polls);
+  if (threadIdx.x == 0) ok = mbar_wait(&bar, 0, &abort_flag, limit_cycles);
+  // (100 ms of arrivals at least 400 cycles apart are fewer than the barrier waits for; past half of them it is left alone)
+  if (threadIdx.x == 32)
+    for (uint32_t i = 0; i < kArrivals / 2 && !*(volatile int*)&abort_flag; ++i) {
+      const uint32_t t0 = sm_cycles();
+      mbar_arrive(&bar);
+      for (int spin = 0; spin < 400 && sm_cycles() - t0 < 400u; ++spin) {}
+    }
   __syncthreads();
   if (threadIdx.x == 0 && abort_flag && !ok && status) { atomicExch(&status[0], DNNF_ERR_TIMEOUT); atomicExch(&status[1], -2); }
 }
@@ -173,7 +182,10 @@ int selftest_wait_expiry(Graph& g, unsigned long long limit_ns, void* stream) {
   if (!g.ws_ptr) { g.err = "bind a workspace first: the status words live in it"; return DNNF_ERR_WORKSPACE; }
   if (limit_ns == 0 || limit_ns > 100000000ull) { g.err = "limit must be between 1 ns and 100 ms"; return DNNF_ERR_INVALID_ARG; }
   g.last_status_base = g.ws_ptr;
-  wait_expiry_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(reinterpret_cast<int32_t*>(g.ws_ptr), (int)std::max(1ull, limit_ns / 4000));     // (a poll takes 4 us)
+  int dev = 0, khz = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess || khz <= 0) { g.err = "cannot ask for the clock rate"; return DNNF_ERR_CUDA; }
+  const unsigned long long cycles = limit_ns * (unsigned long long)khz / 1000000ull;     // (at most 2e8)
+  wait_expiry_kernel<<<1, 64, 0, (cudaStream_t)stream>>>(reinterpret_cast<int32_t*>(g.ws_ptr), (uint32_t)cycles);
   if (cudaGetLastError() != cudaSuccess) { g.err = "self-test launch failed"; return DNNF_ERR_CUDA; }
   return DNNF_OK;
 }

@@ -7,6 +7,7 @@
 
 #include <cstdlib>
 
+#include "bounded_wait.cuh"
 #include "chain.cuh"
 #include "gemm_params.h"
 #include "ir.h"
@@ -28,7 +29,6 @@ namespace tc2 {
 #endif
 
 constexpr int BM = 128, BK = 64, EPI_WARPS = 8, THREADS = 64 + 32 * EPI_WARPS;
-constexpr int kWaitPolls = 1 << 18;
 constexpr int kSmemMax = 227 * 1024;
 constexpr int kBiasFloats = 128;                             // per warp, per row-invariant operand
 constexpr int kMaxVec = 2;                                   // row-invariant operands staged in shared memory
@@ -64,13 +64,9 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 __device__ __forceinline__ unsigned long long wall_ns() { unsigned long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
-// Bounded wait: false, with the CTA's abort flag set, once the polls ran out.  A poll that fails has been suspended for 4 us by
-// the hardware, so kWaitPolls of them are a second; nothing else stands in the loop (tc_common.cuh says what it would cost).
+// Bounded wait: false, with the CTA's abort flag set, when it ran out.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-#pragma unroll 1
-  for (int i = 0; i < kWaitPolls; ++i) if (mbar_try(bar, parity)) return true;
-  *abort_flag = 1;
-  return false;
+  return bounded_wait([=] { return mbar_try(bar, parity); }, abort_flag);
 }
 // Operand load of a CTA pair: the bytes land in THIS CTA's shared memory, the completion is
 // counted on the LEADER's barrier (cluster address), so the MMA thread waits on one barrier only.

@@ -7,6 +7,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include "bounded_wait.cuh"
 #include "chain.cuh"
 #include "gemm_params.h"
 
@@ -32,16 +33,9 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
                : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
   return ok != 0;
 }
-// Bounded wait: false, with the CTA's abort flag set, once the polls ran out.  A poll that fails has been suspended for 4 us by
-// the hardware (measured on a barrier nobody signals, with any hint), so kWaitPolls of them are a second.  Nothing else stands in
-// the loop: with a look at the timer and at the abort flag inlined into every wait (or a call to such code), the warp that issues
-// the MMAs of a 128 x 64 tile took 390 instead of 280 cycles per k-tile.
-constexpr int kWaitPolls = 1 << 18;
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int polls = kWaitPolls) {
-#pragma unroll 1
-  for (int i = 0; i < polls; ++i) if (mbar_try(bar, parity)) return true;
-  *abort_flag = 1;
-  return false;
+// Bounded wait: false, with the CTA's abort flag set, when it ran out.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t limit_cycles = kWaitLimitCycles) {
+  return bounded_wait([=] { return mbar_try(bar, parity); }, abort_flag, limit_cycles);
 }
 __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, uint64_t* bar, int c0, int c1, int c2, int c3) {
   asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"

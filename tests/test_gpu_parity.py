@@ -247,20 +247,26 @@ def test_profiling_database_measured_on_the_device_drives_the_plan():
         B.profile_db_clear()
 
 
-def test_bounded_wait_expires_and_the_graph_runs_on():
-    """The failure path of the tensor-core kernels without a failure: a wait on a barrier that nothing signals gives up
-    after its limit (1 ms here), the status words report DNNF_ERR_TIMEOUT, nothing hangs or faults, and after the
-    caller has cleared the status words the graph runs and is correct again."""
+@pytest.mark.parametrize("limit_ms", [1, 50])
+def test_bounded_wait_expires_and_the_graph_runs_on(limit_ms):
+    """The failure path of the tensor-core kernels without a failure: a wait on a barrier whose phase nothing completes (but which
+    others arrive at: polls then come back at once) gives up after its limit and not before, the status words report
+    DNNF_ERR_TIMEOUT, nothing hangs or faults, and after the caller has cleared the status words the graph runs and is correct again."""
     import time
     import torch
     wl = W.ffn_block(m=256, hidden=128, ffn=256)
     s, got, ref = run_both(wl)
     close(got["Y"], ref["Y"], RTOL_BF16)
     stream = torch.cuda.current_stream().cuda_stream
+    begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     t0 = time.perf_counter()
-    s.g.selftest_wait_expiry(1_000_000, stream)
+    begin.record()
+    s.g.selftest_wait_expiry(limit_ms * 1_000_000, stream)
+    end.record()
     torch.cuda.synchronize()
-    assert time.perf_counter() - t0 < 0.5                      # it gave up after about a millisecond, not a second
+    assert time.perf_counter() - t0 < 0.5                      # it gave up after milliseconds, not a second
+    # cycles at the maximum rate: never less, up to four times as long where the SM runs at a quarter of it
+    assert 0.9 * limit_ms < begin.elapsed_time(end) < 4 * limit_ms + 1
     assert s.g.status() == (B.ERR_TIMEOUT, -2)
     s.workspace[: s.g.workspace_zero_bytes()].zero_()
     s.buffers["Y"].fill_(float("nan"))
