@@ -56,6 +56,13 @@ struct Params {
 };
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// Barrier of the 256 softmax threads that also tells whether all of them are `ok`: a warp whose wait ran out must not leave the others
+// at a barrier that it never comes to.
+__device__ __forceinline__ bool softmax_sync_and(bool ok) {
+  uint32_t all;
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.and.pred q, 1, 256, p;\nselp.u32 %0, 1, 0, q;\n}" : "=r"(all) : "r"((uint32_t)ok) : "memory");
+  return all != 0;
+}
 __device__ __forceinline__ float fast_exp2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 
 template <int NC>
@@ -211,10 +218,9 @@ attention_kernel(const __grid_constant__ GemmParams pA, const __grid_constant__ 
       for (int j = 0; j < NC * 32; ++j) x[j] = (col0 + j < Sk) ? load_scalar<false>(ma, moff + (uint32_t)(col0 + j) * (uint32_t)ma.stride[0]) : 0.0f;
     }
     bool ok = __all_sync(0xffffffffu, mbar_wait(bar_s, 0, abort_flag));
-    float inv_sum = 0.0f;
+    float inv_sum = 0.0f, mx = -3.0e38f;
     if (ok) {
       tc_fence_after();
-      float mx = -3.0e38f;
 #pragma unroll
       for (int ch = 0; ch < NC; ++ch) {
         uint32_t raw[32];
@@ -230,7 +236,9 @@ attention_kernel(const __grid_constant__ GemmParams pA, const __grid_constant__ 
         }
       }
       xch[half * BM + row] = mx;
-      asm volatile("bar.sync 1, 256;" ::: "memory");
+    }
+    ok = softmax_sync_and(ok);
+    if (ok) {
       mx = fmaxf(mx, xch[(half ^ 1) * BM + row]);
       // exponentials, their sum, the bf16 P tile (K-major, 128-byte swizzle; columns past Sk are zero)
       float sum = 0.0f;

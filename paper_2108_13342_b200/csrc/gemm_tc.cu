@@ -159,7 +159,7 @@ gemm_tc_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ Gem
       const int tm = (int)fd_div((uint32_t)r, q.fd_tiles_n), tn = r - tm * p.tiles_n;
       const int acc = tcount & 1;
       const uint32_t aph = (tcount >> 1) & 1;
-      if (!mbar_wait(&tfull_bar[acc], aph, abort_flag)) { ok = false; break; }
+      if (!__all_sync(0xffffffffu, mbar_wait(&tfull_bar[acc], aph, abort_flag))) { ok = false; break; }
       if (tcount == 0 && warp == 2 && lane == 0) TRACE(5);
       tc_fence_after();
       TcEpiIO io{p};

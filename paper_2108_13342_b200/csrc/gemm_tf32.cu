@@ -403,7 +403,7 @@ gemm_tf32_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     for (int tile = first_tile; tile < total_tiles && ok; tile += tile_step, ++tcount) {
       const int acc = tcount & 1;
       const uint32_t aph = (tcount >> 1) & 1;
-      { long long t0 = CLK(); if (!mbar_wait(&tfull_bar[acc], aph, abort_flag)) { ok = false; break; } if (warp == 2 && lane == 0) FACC(5, CLK() - t0); }
+      { long long t0 = CLK(); if (!__all_sync(0xffffffffu, mbar_wait(&tfull_bar[acc], aph, abort_flag))) { ok = false; break; } if (warp == 2 && lane == 0) FACC(5, CLK() - t0); }
       const long long t_epi = CLK();
       tc_fence_after();
       const uint32_t t_row = tmem_base + ((uint32_t)(sub * 32) << 16) + (uint32_t)(acc * acc_cols);
