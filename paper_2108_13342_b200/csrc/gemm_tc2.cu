@@ -447,28 +447,41 @@ bool tc2_gemm_eligible(const GemmParams& gp) {
   return true;
 }
 
-void tc2_gemm_plan(Launch& L) {
-  GemmParams& gp = gp_of(L);
-  tc2::Params& q = t2_of(L);
-  q.b_kmajor = (gp.B.stride_col != 1) ? 1 : 0;
-  q.k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
-  const int tiles_m = (gp.M + 255) / 256;
-  // Tile width: the one whose waves of tiles take the fewest cycles.  A k-tile costs a pair about 530 (BN = 256: the tensor
-  // pipe), 450 (192: the operand feed) or 350 cycles (128: the issuer), a tile's epilogue about 1100 cycles per 32 columns of
-  // a warp; main loop and epilogue overlap, the last epilogue does not.  The count ranks the widths; its times come out too
-  // low (4096 x 768 x 3072, 48 tiles of 256 or 64 of 192 columns on 74 pairs: 24.7 us with 256, 22.3 us with 192 columns, 12.7 counted).
-  const int pairs = sm_count() / 2;
+// Tile width: the one whose waves of tiles take the fewest cycles.  A k-tile costs a pair about 530 (BN = 256: the tensor
+// pipe), 450 (192: the operand feed) or 350 cycles (128: the issuer), a tile's epilogue about 1100 cycles per 32 columns of
+// a warp; main loop and epilogue overlap, the last epilogue does not.  The count ranks the widths; its times come out too
+// low (4096 x 768 x 3072, 48 tiles of 256 or 64 of 192 columns on 74 pairs: 24.7 us with 256, 22.3 us with 192 columns, 12.7 counted).
+int tc2_columns(const GemmParams& gp) {
+  const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK, tiles_m = (gp.M + 255) / 256, pairs = sm_count() / 2;
   int best_bn = 128; double best = 0;
   for (int bn : {256, 192, 128}) {
     if (bn / 2 >= gp.N && bn > 128) continue;
     const int tiles = tiles_m * ((gp.N + bn - 1) / bn);
     const int waves = (tiles + pairs - 1) / pairs;
-    const double main_loop = q.k_tiles * (bn == 256 ? 530.0 : bn == 192 ? 450.0 : 350.0), epi = 1100.0 * (bn / 64);
+    const double main_loop = k_tiles * (bn == 256 ? 530.0 : bn == 192 ? 450.0 : 350.0), epi = 1100.0 * (bn / 64);
     const double cost = waves * std::max(main_loop, epi) + epi;
     if (best == 0 || cost < best) { best = cost; best_bn = bn; }
   }
-  if (dev_env("DNNF_PAIR_BN")) best_bn = atoi(dev_env("DNNF_PAIR_BN"));      // development switch
-  q.bn = best_bn;
+  return best_bn;
+}
+
+// split-K when fewer than half of the 74 CTA pairs would have a tile and the k loop is long.  Handing partial
+// tiles over through L2 costs about 3 us (measured), a k-tile about 0.22 us: it pays from 32 k-tiles up, with
+// two or three slices (1024 x 768 x 3072: 15.7 -> 13.2 us; 1024 x 768 x 768: 7.2 -> 9.2 us, so not there).
+int tc2_slices(int k_tiles, int64_t tiles) {
+  const int pairs = sm_count() / 2;
+  if (tiles * 2 > pairs || k_tiles < 32 || plan_flag(DNNF_PLAN_NO_SPLIT_K)) return 1;
+  return (int)std::min<int64_t>(3, pairs / tiles);
+}
+
+void tc2_gemm_plan(Launch& L) {
+  GemmParams& gp = gp_of(L);
+  tc2::Params& q = t2_of(L);
+  q.b_kmajor = (gp.B.stride_col != 1) ? 1 : 0;
+  q.k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
+  const int tiles_m = (gp.M + 255) / 256, pairs = sm_count() / 2;
+  q.bn = tc2_columns(gp);
+  if (dev_env("DNNF_PAIR_BN")) q.bn = atoi(dev_env("DNNF_PAIR_BN"));      // development switch
   q.tiles_n = (gp.N + q.bn - 1) / q.bn;
   q.total_tiles = tiles_m * q.tiles_n;
   q.fd_tiles = make_fastdiv((uint32_t)q.total_tiles);
@@ -485,13 +498,9 @@ void tc2_gemm_plan(Launch& L) {
   if (dev_env("DNNF_PAIR_KPACK")) q.kpack = atoi(dev_env("DNNF_PAIR_KPACK")) == 2 ? 2 : 1;
   const int stage_bytes = sub_bytes * q.kpack;
   q.stages = std::min(8, tc2::kRingBudget2 / stage_bytes);
-  // split-K when fewer than half of the 74 CTA pairs would have a tile and the k loop is long.  Handing partial
-  // tiles over through L2 costs about 3 us (measured), a k-tile about 0.22 us: it pays from 32 k-tiles up, with
-  // two or three slices (1024 x 768 x 3072: 15.7 -> 13.2 us; 1024 x 768 x 768: 7.2 -> 9.2 us, so not there).
   q.ksplit = 1; q.kt_per = q.k_tiles;
   {
-    int want = 1;
-    if (q.total_tiles * 2 <= pairs && q.k_tiles >= 32 && !plan_flag(DNNF_PLAN_NO_SPLIT_K)) want = std::min(3, pairs / q.total_tiles);
+    int want = tc2_slices(q.k_tiles, q.total_tiles);
     if (dev_env("DNNF_SPLIT_K")) want = std::max(1, std::min(8, atoi(dev_env("DNNF_SPLIT_K"))));
     if (want > 1) {
       int per = (q.k_tiles + want - 1) / want;

@@ -35,6 +35,7 @@
 
 #include <algorithm>
 #include <cstdlib>
+#include <numeric>
 
 #include "ir.h"
 #include "tc2_common.cuh"
@@ -518,6 +519,8 @@ static const tile::Params& tl_of(const Launch& L) { return *reinterpret_cast<con
 size_t tile_blob_bytes() { return sizeof(tile::Params); }
 
 bool tc_gemm_eligible(const GemmParams& gp);
+int tc2_columns(const GemmParams& gp);
+int tc2_slices(int k_tiles, int64_t tiles);
 
 // Same operand and epilogue forms as the CTA-pair kernel (plain 2-D problem, one bf16 row-major output, at most one
 // bf16 full-tile input, row-invariant others), without its lower bounds on M and N.
@@ -548,16 +551,30 @@ static int ws_slices(const GemmParams& gp) {
   return s >= 3 ? (int)s : 1;
 }
 
-// Microseconds of an unsplit problem with tiles of 128 x bn: set-up, and the k-tiles and epilogues of the CTAs that share an SM one
-// after the other (rows x N x K, measured / counted: 1024 x 768 x 768 in 64 columns 4.8 / 4.8, 128 6.0 / 6.0, 192 7.3 / 7.2;
-// 1024 x 768 x 3072 in 64 columns 10.0 / 10.0; 4096 x 768 x 768 in 128 columns, two CTAs per SM, 8.8 / 9.3).  A third CTA of an SM
-// starts when another has left.
+// Share of an operand's rows that do not begin on a 128-byte line: such a row of a tile comes out of two lines.
+static double off_lines(int64_t pitch, int64_t base) {
+  const int64_t g = std::gcd(2 * pitch, (int64_t)128);
+  return g == 128 ? (base % 64 ? 1.0 : 0.0) : 1.0 - (double)g / 128.0;
+}
+static int64_t pitch_b(const GemmParams& gp) { return gp.B.stride_col == 1 ? gp.B.stride_row : gp.B.stride_col; }
+static int full_operands(const GemmParams& gp) { int n = 0; for (int i = 0; i < gp.n_in; ++i) n += gp.in[i].mode != 1; return n; }
+// How much longer a k-tile of rows_a x rows_b takes for the lines; only the rows of A that exist count.
+static double line_factor(const GemmParams& gp, double rows_b, double weight_a, double weight_b) {
+  const double tiles_m = (gp.M + tc2::BM - 1) / tc2::BM, a = off_lines(gp.A.stride_row, gp.A.base) * gp.M / tiles_m, b = off_lines(pitch_b(gp), gp.B.base) * rows_b;
+  return 1.0 + (weight_a * a + weight_b * b) / (tc2::BM + rows_b);
+}
+
+// Microseconds of an unsplit problem with tiles of 128 x bn: set-up, the k-tiles and epilogues of the CTAs that share an SM one after the
+// other; a third starts when another has left, and the last of an odd number has the SM to itself.  Constants fitted to 1430 timings
+// of 700 shapes (M 33 .. 16384, N 32 .. 5120, K 64 .. 5120, operands in L2; error 10 % rms).  Rows x N x K, measured / counted: 1024 x 768 x 768
+// in 64 columns 4.6 / 4.4, 1024 x 3072 x 768 in 192 8.1 / 6.6; off the lines 173 x 2152 x 1096 in 64 columns 8.8 / 7.0, 1682 x 1144 x 2792 in 128 23.4 / 19.1.
 static double tile_us(const GemmParams& gp, int bn) {
   const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
-  const int64_t tiles = (int64_t)((gp.M + tc2::BM - 1) / tc2::BM) * ((gp.N + bn - 1) / bn);
-  const double c = (double)((tiles + sm_count() - 1) / sm_count());
-  const double k_us = bn == 64 ? 0.145 : bn == 128 ? 0.2 : 0.235, epi_us = bn == 64 ? 0.3 : bn == 128 ? 0.85 : 1.6;
-  return 2.75 + c * (k_tiles * k_us + epi_us) + (c > 2 ? 1.5 * (c - 2) : 0.0);
+  const int64_t tiles = (int64_t)((gp.M + tc2::BM - 1) / tc2::BM) * ((gp.N + bn - 1) / bn), c = (tiles + sm_count() - 1) / sm_count();
+  const double k_us = (bn == 64 ? 0.129 : bn == 128 ? 0.182 : 0.226) * line_factor(gp, bn, 1.0, 1.3);
+  const double epi_us = (bn == 64 ? 0.59 : bn == 128 ? 0.97 : 1.55) + full_operands(gp) * (bn == 64 ? 0.27 : bn == 128 ? 0.77 : 1.13);
+  const double one = k_tiles * k_us + epi_us;
+  return 2.3 + c * one + 0.9 * ((c - 1) / 2) + (c > 1 && c % 2 ? 0.4 * one : 0.0);
 }
 // 192 columns only while every tile has an SM to itself (its ring leaves no room for a second CTA) and 64 divides N (one request for B).
 static int tile_columns(const GemmParams& gp) {
@@ -567,29 +584,30 @@ static int tile_columns(const GemmParams& gp) {
   if (gp.N > 128 && gp.N % 64 == 0 && tiles_m * ((gp.N + 191) / 192) <= sm_count() && tile_us(gp, 192) < tile_us(gp, best)) best = 192;
   return best;
 }
-// The same for the CTA-pair kernel: one wave of 256-row tiles after the other, the last epilogue on its own (512 x 768 x 768 7.2 / 7.2,
-// 2048 x 384 x 1536 9.6 / 9.6, 4096 x 2304 x 768 14.9 / 15.8).
+// The same for the CTA-pair kernel with the width and the K slices that its plan takes: one wave of 256-row tiles after the other, the last
+// epilogue on its own, a hand-over where K is sliced.  A CTA of a pair reads half of B, so that rows off the lines cost it less.
 static double pair_us(const GemmParams& gp) {
-  const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
-  double best = 0.0;
-  for (int bn : {256, 192, 128}) {
-    const int64_t tiles = (int64_t)((gp.M + 255) / 256) * ((gp.N + bn - 1) / bn);
-    const double waves = (double)((tiles + sm_count() / 2 - 1) / (sm_count() / 2));
-    const double main_us = k_tiles * (bn == 256 ? 0.28 : bn == 192 ? 0.24 : 0.2), epi_us = bn == 256 ? 2.3 : bn == 192 ? 1.7 : 1.15;
-    const double us = 3.6 + waves * std::max(main_us, epi_us) + epi_us + 0.9 * (waves - 1);
-    if (best == 0.0 || us < best) best = us;
-  }
-  return best;
+  const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK, bn = tc2_columns(gp), pairs = sm_count() / 2;
+  const int64_t tiles = (int64_t)((gp.M + 255) / 256) * ((gp.N + bn - 1) / bn), waves = (tiles + pairs - 1) / pairs;
+  const double k_us = (bn == 256 ? 0.273 : bn == 192 ? 0.238 : 0.201) * line_factor(gp, bn / 2, 0.58, 0.53);
+  const double epi_us = (bn == 256 ? 2.3 : bn == 192 ? 1.3 : 0.2) + full_operands(gp) * 0.74 * bn / 128;
+  const int slices = tc2_slices(k_tiles, tiles);
+  if (slices > 1) return 4.4 + (k_tiles + slices - 1) / slices * k_us + epi_us + 4.7;
+  return 4.4 + waves * std::max(k_tiles * k_us, epi_us) + epi_us + 1.8 * (waves - 1);
 }
 
-// Against the CTA-pair kernel: whichever the counts say is the faster (1024 x 768 x 768 4.8 against 7.2 us, 2048 x 2304 x 768 8.9 / 11.3,
-// 2048 x 768 x 3072 13.4 / 15.2, 4096 x 768 x 3072 16.8 / 17.8; 4096 x 2304 x 768 16.9 / 14.9).
+// Against the CTA-pair kernel: whichever the counts say is the faster (1024 x 768 x 768 4.6 us against 6.9, 4096 x 768 x 3072 + residual
+// 17.8 / 19.2; 9710 x 2816 x 128 with B transposed 16.7 / 22.6; 3219 x 1920 x 576 12.1 / 10.5, 1682 x 1144 x 2792 23.4 / 19.7, 4145 x 496 x 4056
+// 26.5 / 23.3).  They were fitted to at most six tiles per SM; more go to the pair kernel (6996 x 1328 x 80 + residual 16.3 / 14.1).  Over 611
+// shapes the kernel taken is 0.9 % slower than the best one; by the number of 256 x 256 tiles and K <= 1024 it was 4 %.
 bool tile_gemm_preferred(const GemmParams& gp) {
   if (plan_flag(DNNF_PLAN_NO_TILE_GEMM)) return false;
   if (dev_env("DNNF_GEMM_TILE")) return atoi(dev_env("DNNF_GEMM_TILE")) != 0;
   if (ws_slices(gp) > 1) return true;
   if (plan_flag(DNNF_PLAN_CLUSTER_SPLIT_K)) return (int64_t)((gp.M + 255) / 256) * ((gp.N + 255) / 256) < sm_count() / 2;
-  return tile_us(gp, tile_columns(gp)) < pair_us(gp);
+  const int bn = tile_columns(gp);
+  if ((int64_t)((gp.M + tc2::BM - 1) / tc2::BM) * ((gp.N + bn - 1) / bn) > 6 * sm_count()) return false;
+  return tile_us(gp, bn) < pair_us(gp);
 }
 
 void tile_gemm_plan(Launch& L) {

@@ -818,3 +818,28 @@ def test_deep_fp32_contraction_of_few_rows_takes_the_faster_kernel(m, k, n, vari
     g.mark_output(g.add("MatMul", ["X", "Wt"]))
     G, ids, st = _plan_desc(g)
     assert [b["variant"] for b in G.blocks()] == [variant], G.blocks()
+
+
+@pytest.mark.parametrize("mnk,epi,kmajor_b,variant,grid", [
+    # rows that begin off the 128-byte lines: a long K goes to CTA pairs (with K slices where few tiles leave pairs idle) ...
+    ((1682, 1144, 2792), "bias", False, 3, 2 * 7 * 9), ((440, 2280, 5096), "bias", False, 3, 2 * 2 * 18 * 2), ((4219, 448, 4792), "residual", True, 3, 2 * 17 * 4),
+    # ... and few k-tiles to 128 columns, one tile to an SM
+    ((2897, 568, 80), "bias", False, 5, 23 * 5), ((13491, 112, 88), "none", False, 5, 106), ((673, 3072, 104), "none", False, 5, 6 * 24),
+    # rows on the lines: one narrow tile per SM, 192 columns where that makes it one
+    ((1024, 768, 768), "bias", False, 5, 8 * 12), ((1024, 3072, 768), "bias", False, 5, 8 * 16), ((4096, 768, 3072), "residual", False, 5, 32 * 4),
+    # more tiles to an SM than the counted times were fitted to
+    ((6996, 1328, 80), "residual", False, 3, 148)])
+def test_bf16_product_goes_to_the_kernel_that_was_measured_faster(mnk, epi, kmajor_b, variant, grid):
+    m, n, k = mnk
+    g = W.GraphDesc("t")
+    g.ext("A", (m, k), "bf16")
+    b = g.add("Transpose", [g.ext("Bt", (n, k), "bf16", "weight")], perm=(1, 0)) if kmajor_b else g.ext("Bm", (k, n), "bf16", "weight")
+    y = g.add("MatMul", ["A", b])
+    if epi != "none":
+        y = g.add("Add", [y, g.ext("bias", (n,))])
+    if epi == "residual":
+        y = g.add("Add", [y, g.ext("R", (m, n), "bf16")])
+    g.mark_output(y)
+    gr = build_graph(g)[0]
+    gr.plan(B.PLAN_FUSED)
+    assert [(x["variant"], x["grid"]) for x in gr.blocks()] == [(variant, grid)]
