@@ -339,7 +339,9 @@ gemm_tile_kernel(const __grid_constant__ GemmParams p, const __grid_constant__ P
     stage_vectors(true);
     // The k-tiles of a weight beyond the ring's first ones go into L2 while the previous kernel runs: from DRAM, a ring of four
     // stages is a microsecond's latency every four k-tiles.  The CTAs of a column of tiles and their epilogue warps take turns.
-    if (q.b_static)
+    // Not in a run's first kernel: it has waited already, and requests beside those of the ring only hold them up (operands in L2,
+    // 123 x 2456 x 816 6.4 us with them, 5.7 without; 45 x 1360 x 1464 8.2 / 7.1; 1024 x 3072 x 768 8.8 / 8.1).
+    if (q.b_static && !p.ordered)
       for (int kt = stages + tm * kEpiWarps + ew; kt < k_tiles; kt += p.tiles_m * kEpiWarps)
         if (elect_one()) {
           if (kBK) {
