@@ -182,19 +182,29 @@ int launch_row_shift(const Launch& L, cudaStream_t st) {
   }
 }
 
-// Rows of up to 122 elements, four to a warp: 64 x 12 x 61 x 61 masked softmax 13.5 -> 6.5 us, 131072 x 93 LayerNorm + GELU 38.6.  Longer
+// Rows of up to 125 elements, four to a warp: 64 x 12 x 61 x 61 masked softmax 13.5 -> 6.5 us.  Longer
 // ones stay with one element per lane and load: with a warp or a CTA to a row the branches between the loads serialise them
-// (8000 x 4095 91 -> 150 us, 32 x 12 x 317 x 317 80.8 -> 84.6).
+// (8000 x 4095 91 -> 150 us, 32 x 12 x 317 x 317 80.8 -> 84.6).  So do launches of few rows, where a lane's longer chain is the time and not
+// the bytes in flight: the fewest rows per SM that win, by operands (softmax; with a mask; LayerNorm) and vectors a lane.  Rows x length,
+// us element by element / here:
+//   softmax             2000 x 21 1.4 / 1.4, 3000 1.6 / 1.4; 5000 x 58 2.1 / 2.1; 3500 x 91 1.7 / 2.0, 5000 2.1 / 2.1; 4500 x 122 1.9 / 2.1, 6000 2.3 / 2.3
+//   masked softmax      2000 x 21 1.5 / 1.7, 3000 1.7 / 1.7; 5000 x 58 2.4 / 2.4; 5000 x 91 2.4 / 2.9, 8500 3.4 / 3.3; 6000 x 122 2.7 / 3.1, 10500 3.9 / 3.9
+//   LayerNorm           2000 x 21 2.0 / 2.1, 4300 2.2 / 2.2; 5000 x 58 2.8 / 2.9, 7200 3.0 / 3.0; 5000 x 91 2.9 / 3.1, 8500 3.4 / 3.4;
+//                       13000 x 122 5.0 / 5.7, 20000 6.9 / 6.1
+// A row that a warp holds in one element per lane but eight lanes only in two vectors each (30 and 31 elements): where the element-wise form
+// takes four rows to a warp, only softmax alone wins (50000 x 31 5.3 / 4.8 us; with a mask 6.5 / 7.0, LayerNorm 8.6 / 10.4), LayerNorm never does.
 bool finalize_row_shift(Launch& L) {
   RowParams& p = L.row;
   const int vectors = (p.L + 6) / 4;                             // up to three elements in front of the row
-  if (vectors > 32) return false;
+  const int lpr = 8, nv = (vectors + lpr - 1) / lpr;
+  static constexpr int kRowsPerSm[3][4] = {{16, 35, 34, 38}, {20, 36, 57, 70}, {29, 48, 57, 122}};
+  if (nv > 4 || p.rows < (int64_t)sm_count() * kRowsPerSm[p.n_in == 1 ? 0 : p.n_in == 2 ? 1 : 2][nv - 1]) return false;
+  if (nv == 2 && p.L <= 32 && p.n_in > 1 && (p.n_in > 2 || p.rows >= 16000)) return false;
   for (int i = 0; i < p.n_in; ++i) if (p.in[i].dtype != 0) return false;
   for (int i = 0; i < p.n_out; ++i) if (p.out[i].dtype != 0 || p.out[i].stride[0] != 1) return false;
   if (p.in[0].stride[0] != 1) return false;
   L.static_id = StaticSet<RowStatic>::find(p.prog);
   if (!L.static_id) return false;
-  const int lpr = 8, nv = (vectors + lpr - 1) / lpr;
   L.variant = 900000 + nv * 1000 + lpr;
   const int64_t rows_per_cta = lpr > 32 ? 1 : 32 * kRowWarpsPerCta / lpr;
   L.grid = (int)((p.rows + rows_per_cta - 1) / rows_per_cta);
