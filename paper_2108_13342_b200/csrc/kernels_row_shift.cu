@@ -1,4 +1,4 @@
-// Row blocks of fp32 tensors whose rows fit no 16-byte vector (a length of 197, an odd slice), with 16-byte accesses all the same.
+// Short row blocks of fp32 tensors whose rows fit no 16-byte vector (61 elements, an odd slice), with 16-byte accesses all the same.
 //
 // A row that starts m elements behind a 16-byte boundary is seen through aligned vectors: vector g covers the elements
 // 4 g - m .. 4 g - m + 3, the ones in front of the row and behind its end are masked.  Which element a lane holds is of no concern to
@@ -11,20 +11,19 @@ namespace dnnf {
 
 namespace {
 
-// LPR lanes share a row, each with NV vectors of four.
-template <int NV, int LPR>
+constexpr int kLanesPerRow = 8, kRowsPerCta = 32 * kRowWarpsPerCta / kLanesPerRow;
+
+// A lane holds NV vectors of four of its row.
+template <int NV>
 struct ShiftIO {
   static constexpr int VV = 4 * NV;
   const RowParams& p;
   uint32_t outer[kMaxDims];
   bool row_ok;
   int lane_in_row, m;
-  float* xchg;                     // shared memory, 2 x 8 floats (LPR == 256)
-  mutable int xslot = 0;
-  // Vectors that can reach past an end of the row: the first, and the last two (with no form for seven vectors, three of eight).
-  // The ones between lie in the row whole, and so does the window of eight that an operand of another alignment is read through.
-  static constexpr bool edge(int j) { return j == 0 || j >= NV - (NV == 8 ? 3 : 2); }
-  __device__ __forceinline__ int col(int j) const { return 4 * (j * LPR + lane_in_row) - m; }
+  // Vectors that can reach past an end of the row: the first, and the last two.  The ones between lie in the row whole.
+  static constexpr bool edge(int j) { return j == 0 || j >= NV - 2; }
+  __device__ __forceinline__ int col(int j) const { return 4 * (j * kLanesPerRow + lane_in_row) - m; }
   __device__ __forceinline__ bool valid(int c) const { return (unsigned)c < (unsigned)p.L; }
   __device__ __forceinline__ const float* row_ptr(const TensorArg& a) const {
     uint32_t off = (uint32_t)a.base;
@@ -46,36 +45,14 @@ struct ShiftIO {
       for (int e = 0; e < VV; ++e) dst[e] = x;
       return;
     }
-    const int by = (misalignment(q) - m) & 3;      // this operand's vectors lie `by` elements earlier (the same for a warp but where rows share one)
-    if (by == 0) {
-#pragma unroll
-      for (int j = 0; j < NV; ++j) {
-        const int c = col(j);
-        float* d = &dst[4 * j];
-        if (row_ok && (!edge(j) || (c >= 0 && c + 4 <= p.L))) {
-          const float4 w = __ldg(reinterpret_cast<const float4*>(q + c));
-          d[0] = w.x; d[1] = w.y; d[2] = w.z; d[3] = w.w;
-        } else {
-          masked(q, c, d);
-        }
-      }
-      return;
-    }
-    if (LPR < 32) {
-#pragma unroll
-      for (int j = 0; j < NV; ++j) masked(q, col(j), &dst[4 * j]);
-      return;
-    }
+    const bool same = misalignment(q) == m;
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       const int c = col(j);
       float* d = &dst[4 * j];
-      if (row_ok && (!edge(j) || (c >= by && c + 8 <= p.L))) {
-        const float4 u = __ldg(reinterpret_cast<const float4*>(q + c - by)), w = __ldg(reinterpret_cast<const float4*>(q + c - by) + 1);
-        d[0] = by == 1 ? u.y : by == 2 ? u.z : u.w;
-        d[1] = by == 1 ? u.z : by == 2 ? u.w : w.x;
-        d[2] = by == 1 ? u.w : by == 2 ? w.x : w.y;
-        d[3] = by == 1 ? w.x : by == 2 ? w.y : w.z;
+      if (same && row_ok && (!edge(j) || (c >= 0 && c + 4 <= p.L))) {
+        const float4 w = __ldg(reinterpret_cast<const float4*>(q + c));
+        d[0] = w.x; d[1] = w.y; d[2] = w.z; d[3] = w.w;
       } else {
         masked(q, c, d);
       }
@@ -114,31 +91,26 @@ struct ShiftIO {
     join(part[0], part[1]); join(part[2], part[3]); join(part[0], part[2]);
     float red = part[0];
 #pragma unroll
-    for (int o = (LPR < 32 ? LPR : 32) / 2; o > 0; o >>= 1) join(red, __shfl_xor_sync(0xffffffffu, red, o));
-    if (LPR > 32) {
-      // two exchange areas used in turn: the barrier of this exchange also tells that everybody has read the one before
-      float* x = xchg + xslot * (LPR / 32);
-      xslot ^= 1;
-      if ((threadIdx.x & 31) == 0) x[threadIdx.x >> 5] = red;
-      __syncthreads();
-      red = x[0];
-#pragma unroll
-      for (int w = 1; w < LPR / 32; ++w) join(red, x[w]);
-    }
+    for (int o = kLanesPerRow / 2; o > 0; o >>= 1) join(red, __shfl_xor_sync(0xffffffffu, red, o));
     const float x = op == M_ROWMEAN ? red * p.inv_L : red;
 #pragma unroll
     for (int e = 0; e < VV; ++e) acc[e] = x;
   }
 };
 
-template <int NV, int LPR, class SP>
-__global__ void __launch_bounds__(LPR > 32 ? LPR : 32 * kRowWarpsPerCta) row_shift_kernel(const __grid_constant__ RowParams p) {
-  __shared__ float xchg[LPR > 32 ? 2 * LPR / 32 : 1];
-  constexpr int kRows = LPR > 32 ? 1 : 32 * kRowWarpsPerCta / LPR;      // rows of a CTA
-  ShiftIO<NV, LPR> io{p};
-  io.xchg = xchg;
-  io.lane_in_row = (int)(threadIdx.x % LPR);
-  uint32_t row = blockIdx.x * kRows + threadIdx.x / LPR;
+// (row_reduce knows no running sum along the row)
+template <class SP>
+constexpr bool scans_a_row() {
+  for (int i = 0; i < SP::n; ++i) if (SP::op(i).op >= M_ROWSCAN) return true;
+  return false;
+}
+
+template <int NV, class SP>
+__global__ void __launch_bounds__(32 * kRowWarpsPerCta) row_shift_kernel(const __grid_constant__ RowParams p) {
+  static_assert(!scans_a_row<SP>(), "a running sum needs the element-wise form");
+  ShiftIO<NV> io{p};
+  io.lane_in_row = (int)(threadIdx.x % kLanesPerRow);
+  uint32_t row = blockIdx.x * kRowsPerCta + threadIdx.x / kLanesPerRow;
   io.row_ok = row < (uint32_t)p.rows;
   if (!io.row_ok) row = 0;                                              // (its lanes still take part in the shuffles)
   uint32_t lin = row;
@@ -156,28 +128,28 @@ __global__ void __launch_bounds__(LPR > 32 ? LPR : 32 * kRowWarpsPerCta) row_shi
   run_program<4 * NV, SP>(p.prog, io);
 }
 
-template <int NV, int LPR>
+template <int NV>
 struct ShiftLauncher {
   const Launch& L; cudaStream_t st; cudaError_t rc = cudaSuccess;
-  template <class SP> void run() { rc = launch_pdl(row_shift_kernel<NV, LPR, SP>, L.grid, L.threads, 0, st, L.row); }
+  template <class SP> void run() { rc = launch_pdl(row_shift_kernel<NV, SP>, L.grid, L.threads, 0, st, L.row); }
 };
 
-template <int NV, int LPR>
+template <int NV>
 int launch_shift(const Launch& L, cudaStream_t st) {
-  ShiftLauncher<NV, LPR> F{L, st};
+  ShiftLauncher<NV> F{L, st};
   if (!StaticSet<RowStatic>::dispatch(L.static_id, F)) return 1;
   return F.rc == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : 1;
 }
 
 }  // namespace
 
-// variant encoding: 900000 + NV * 1000 + LPR
+// variant encoding: 900000 + vectors a lane * 1000 + lanes per row
 int launch_row_shift(const Launch& L, cudaStream_t st) {
   switch (L.variant) {
-    case 901008: return launch_shift<1, 8>(L, st);
-    case 902008: return launch_shift<2, 8>(L, st);
-    case 903008: return launch_shift<3, 8>(L, st);
-    case 904008: return launch_shift<4, 8>(L, st);
+    case 901008: return launch_shift<1>(L, st);
+    case 902008: return launch_shift<2>(L, st);
+    case 903008: return launch_shift<3>(L, st);
+    case 904008: return launch_shift<4>(L, st);
     default: return 2;
   }
 }
@@ -196,7 +168,7 @@ int launch_row_shift(const Launch& L, cudaStream_t st) {
 bool finalize_row_shift(Launch& L) {
   RowParams& p = L.row;
   const int vectors = (p.L + 6) / 4;                             // up to three elements in front of the row
-  const int lpr = 8, nv = (vectors + lpr - 1) / lpr;
+  const int nv = (vectors + kLanesPerRow - 1) / kLanesPerRow;
   static constexpr int kRowsPerSm[3][4] = {{16, 35, 34, 38}, {20, 36, 57, 70}, {29, 48, 57, 122}};
   if (nv > 4 || p.rows < (int64_t)sm_count() * kRowsPerSm[p.n_in == 1 ? 0 : p.n_in == 2 ? 1 : 2][nv - 1]) return false;
   if (nv == 2 && p.L <= 32 && p.n_in > 1 && (p.n_in > 2 || p.rows >= 16000)) return false;
@@ -205,10 +177,9 @@ bool finalize_row_shift(Launch& L) {
   if (p.in[0].stride[0] != 1) return false;
   L.static_id = StaticSet<RowStatic>::find(p.prog);
   if (!L.static_id) return false;
-  L.variant = 900000 + nv * 1000 + lpr;
-  const int64_t rows_per_cta = lpr > 32 ? 1 : 32 * kRowWarpsPerCta / lpr;
-  L.grid = (int)((p.rows + rows_per_cta - 1) / rows_per_cta);
-  L.threads = lpr > 32 ? lpr : 32 * kRowWarpsPerCta;
+  L.variant = 900000 + nv * 1000 + kLanesPerRow;
+  L.grid = (int)((p.rows + kRowsPerCta - 1) / kRowsPerCta);
+  L.threads = 32 * kRowWarpsPerCta;
   set_fastdiv(p.it);
   return true;
 }
