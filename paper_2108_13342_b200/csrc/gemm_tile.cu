@@ -2,12 +2,12 @@
 //
 // For problems with too few 256-row tiles to fill the machine with the persistent CTA-pair kernel
 // (the projection and feed-forward GEMMs of a 1024-token encoder layer): every CTA computes ONE
-// 128 x BN tile (BN = 64 or 128) and leaves.  The kernel is built for latency and for overlap
+// 128 x BN tile (BN = 64, 128 or 192) and leaves.  The kernel is built for latency and for overlap
 // between CTAs instead of a long steady state:
-//   * at most ~106 KB of shared memory and BN tensor-memory columns per CTA, so two CTAs share an
+//   * with 64 or 128 columns at most ~110 KB of shared memory and BN tensor-memory columns per CTA, so two CTAs share an
 //     SM: while one runs its epilogue the other's MMAs use the tensor cores, and the CTAs of the
 //     NEXT kernel on the stream (programmatic dependent launch) become resident, set up and fetch
-//     their weights while this kernel drains;
+//     their weights while this kernel drains (192 columns take ~130 KB and 256 tensor-memory columns: one CTA per SM);
 //   * the B operand of a block is normally a weight, which no kernel of the graph writes: its
 //     first ring stages are requested BEFORE the wait on the previous kernel, as are the bias
 //     vectors; only the loads of A (and of a residual tile) wait;
@@ -18,10 +18,10 @@
 // columns at a time -> bf16 -> swizzled 32 x 32 chunk -> TMA store.  With four warps and 32 columns at a time the epilogue
 // was the longer half of these kernels: 248 x 2304 x 768 + bias 6.1 -> 5.4 us, 248 x 768 x 768 5.5 -> 4.8, 248 x 3072 x 768 +
 // GELU 6.8 -> 6.0, 1024 x 768 x 768 6.0 -> 5.4.
-// Tile widths: 64, 128 or 192 columns, by counted time (tile_us): a k-tile costs a CTA 0.145, 0.2 or 0.235 us, so wide tiles are for
-// the problems whose narrow ones would share SMs (1024 x 3072 x 768 + GELU: 192 tiles of 128 columns 10.8 us, 128 of 192 8.9).
+// Tile widths: 64, 128 or 192 columns, by counted time (tile_us): a k-tile costs a CTA 0.13, 0.18 or 0.23 us, so wide tiles are for
+// the problems whose narrow ones would share SMs (1024 x 3072 x 768 + GELU: 192 tiles of 128 columns 10.8 us, 128 of 192 8.1).
 // The issuer's and the producers' loops hold nothing but their wait, their requests and their commit: conditional commits, a branch
-// on B's order, and the timer and abort flag inside the wait made a k-tile of 64 columns cost 500 cycles instead of 280
+// on B's order, and the global timer and abort flag inside the wait made a k-tile of 64 columns cost 500 cycles instead of 280
 // (1024 x 768 x 3072 unsplit 12.4 -> 10.0 us, 248 x 768 x 768 5.2 -> 4.6).  The k-tiles of a weight beyond the ring go into L2 before
 // the wait on the previous kernel: in a chain of layers the weights come from DRAM (twelve decoder layers 600 -> 568 us).
 // Long K, few tiles: the k-tiles of a tile are shared by three or four CTAs that meet in the workspace (kMode 2): every epilogue
@@ -29,7 +29,7 @@
 // and adds all in slice order.  248 x 768 x 3072: 14.0 us as one CTA per tile, 10.5 with plain loads of all slices, 8.5 now.
 // Every wait is bounded; on expiry the CTA records DNNF_ERR_TIMEOUT and releases tensor memory.
 //
-// Every TMA load in this file is a plain per-CTA load; no clusters are used.
+// Every TMA load in this file is a plain per-CTA load; clusters are used by kMode 1 only (DNNF_PLAN_CLUSTER_SPLIT_K).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -542,9 +542,9 @@ bool tile_gemm_eligible(const GemmParams& gp) {
   return full <= 1 && vec <= tc2::kMaxVec;
 }
 
-// Slices of K that meet in the workspace: with long K (the hand-over costs about 5 us, a k-tile 0.22) and few enough 128 x 64
-// tiles for three or four CTAs each, two per SM, and at least eight k-tiles per CTA.  Two slices are no gain over CTA pairs
-// (1024 x 768 x 3072: 13.9 against 13.7 us; with three 12.9).
+// Slices of K that meet in the workspace: with long K and few enough 128 x 64 tiles for three or four CTAs each, two per SM, and at
+// least eight k-tiles per CTA.  Not by counted time: 248 x 768 x 3072 takes 8.6 us in four slices and 10.1 unsplit, and
+// 1024 x 768 x 3072 in three 12.7 against 9.9 with the operands in L2, but 19.5 against 22.5 with the operands in DRAM.
 static int ws_slices(const GemmParams& gp) {
   const int k_tiles = (gp.K + tc2::BK - 1) / tc2::BK;
   const int64_t tiles = (int64_t)((gp.M + tc2::BM - 1) / tc2::BM) * ((gp.N + 63) / 64);
@@ -626,12 +626,10 @@ void tile_gemm_plan(Launch& L) {
   q.tiles_n = (gp.N + q.bn - 1) / q.bn;
   q.fd_tiles_n = make_fastdiv((uint32_t)q.tiles_n);
   gp.tiles_m = tiles_m; gp.tiles_n = q.tiles_n;
-  // Split over K through a cluster (DNNF_PLAN_CLUSTER_SPLIT_K only): a k-tile costs a CTA about 0.35 us whatever the
-  // tile's size, so the k-tiles of a tile are shared by a cluster of 4 or 2 CTAs as long as two CTAs per SM hold the
-  // whole grid and every CTA keeps at least three k-tiles.  Measured, it does not pay at these sizes: the main loop of
-  // 1024 x 768 x 768 ends after 2.6 instead of 5.9 us, but the hand-over (0.6 us barrier, 1.2 us of remote stores, 2 us
-  // until every CTA's stores have arrived) and 2.5 us more per launch of a cluster in a chain of dependent kernels eat
-  // all of it (11.5 against 8.5 us per launch), hence off by default.
+  // Split over K through a cluster (DNNF_PLAN_CLUSTER_SPLIT_K only): the k-tiles of a tile are shared by a cluster of 4 or 2 CTAs as
+  // long as two CTAs per SM hold the whole grid and every CTA keeps at least three k-tiles.  When it was measured, with k-tiles of
+  // 0.35 us, the hand-over (0.6 us barrier, 1.2 us of remote stores, 2 us until every CTA's stores have arrived) ate what the shorter
+  // main loop gave (1024 x 768 x 768 11.5 against 8.5 us per launch in a chain); unsplit that product takes 4.6 us now.  Off by default.
   int S = 1;
   q.ws_split = ws_slices(gp) > 1;
   if (q.ws_split) {
