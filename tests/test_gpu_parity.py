@@ -258,6 +258,8 @@ def test_bounded_wait_expires_and_the_graph_runs_on(limit_ms):
     s, got, ref = run_both(wl)
     close(got["Y"], ref["Y"], RTOL_BF16)
     stream = torch.cuda.current_stream().cuda_stream
+    s.g.selftest_wait_expiry(1000, stream)                     # (the kernel's code is loaded by its first launch, while the events' time runs)
+    torch.cuda.synchronize()
     begin, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     t0 = time.perf_counter()
     begin.record()
